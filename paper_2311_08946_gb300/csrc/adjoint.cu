@@ -34,18 +34,24 @@ __global__ void __launch_bounds__(256) k_grad_dirichlet(Problem P, int N, const 
 }
 
 // grad[q] = sum_d partial_disk[d][q] (q < nw + nf) + sum_s partial_mc[s][q] + dirichlet[q - nw - nf]
-// (q >= nw + nf), in the layout [c weights][f weights][g coefficients], each sum in a fixed order
-__global__ void k_sum_partials(int nw, int nf, int ng, const double *pd, int nd, const double *pm, int nm,
-                               const double *pg, double *grad) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    const int np = nw + nf + ng;
-    if (q >= np) return;
+// (q >= nw + nf), in the layout [c weights][f weights][g coefficients]: one CTA per parameter, each
+// thread every 128th partial, the threads' sums added in a fixed order
+__global__ void __launch_bounds__(128) k_sum_partials(int nw, int nf, int ng, const double *pd, int nd,
+                                                      const double *pm, int nm, const double *pg, double *grad) {
+    __shared__ double red[4];
+    const int q = blockIdx.x, np = nw + nf + ng;
     double s = 0.0;
     if (q < nw + nf)
-        for (int d = 0; d < nd; ++d) s += pd[(long)d * (nw + nf) + q];
-    for (int r = 0; r < nm; ++r) s += pm[(long)r * np + q];
-    if (q >= nw + nf && pg) s += pg[q - nw - nf];
-    grad[q] = s;
+        for (int d = threadIdx.x; d < nd; d += 128) s += pd[(long)d * (nw + nf) + q];
+    for (int r = threadIdx.x; r < nm; r += 128) s += pm[(long)r * np + q];
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s = ((red[0] + red[1]) + red[2]) + red[3];
+        if (q >= nw + nf && pg) s += pg[q - nw - nf];
+        grad[q] = s;
+    }
 }
 
 void grad_impl(const pdd_cover &cov, const Problem &P, const pdd_assembly_opts &o, const pdd_system &sys,
@@ -83,7 +89,7 @@ void grad_impl(const pdd_cover &cov, const Problem &P, const pdd_assembly_opts &
     grad_mc(cov, P, o, sys, u, lambda, pm, nm, st);
     // layout of grad: [c weights][f weights][g coefficients] (families the operator does not use
     // have no entries)
-    PDD_LAUNCH(k_sum_partials, cdiv(n_all, 128), 128, 0, st, nw, nf, ng, pd.p, nd, pm.p, nm, ng ? pg.p : nullptr,
+    PDD_LAUNCH(k_sum_partials, n_all, 128, 0, st, nw, nf, ng, pd.p, nd, pm.p, nm, ng ? pg.p : nullptr,
                grad);
     PDD_CUDA(cudaStreamSynchronize(st));
 }

@@ -23,6 +23,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "exp64.cuh"
 #include "handles.cuh"
 
 namespace pdd {
@@ -1360,23 +1361,48 @@ struct GradArgs {
     const long *kinv_off;
     const double *kinv;
     double c2;
-    int n_par;
-    double *partial;          // [slot][n_rbf + n_gcoef]
+    int n_par, splits;        // a row's paths are cut into `splits` parts, one CTA each
+    double *partial;          // [slot][part][n_rbf + n_frbf + n_gcoef]
 };
 
+// Four lanes carry one path: they hold its state in common and each owns every fourth basis
+// function (of c, f and g) and its running sums in shared memory, [index / 4][thread].  The cost is
+// the FP64 pipe (one Gaussian per basis function and step, exp_neg, evaluated once: psi is kept in
+// shared memory for the update that needs c first), so nothing else is repeated by the four lanes:
+// lane s of a path draws the normals of step k + s for all four, the payoff's basis sum and the
+// boundary series are split over them.  A warp owns a fixed range of path ids and its eight
+// paths take the next id of that range in lane order (deterministic); a path that ends waits for
+// the next group of four steps, so the normals of all eight are drawn together.
+// 116 rows x 1,000 paths, 64 + 16 + 32 parameters: 1240 -> 86 ms.
+static constexpr int kGradThreads = 128, kGradLanes = 4;
+static constexpr int kGradMaxParams = 438;       // 3 nw + nf + ng: at most 164 KB of shared memory
+
+__host__ __device__ constexpr size_t grad_smem_doubles(int nw, int nf, int ng) {
+    return kMaxStencil + 2 * kExpTab + 3 * (size_t)(nw + nf) +
+           (size_t)kGradThreads * (4 * ((nw + 3) / 4) + (nf + 3) / 4 + (ng + 3) / 4);
+}
+
 template <typename R, bool SRC>
-__global__ void __launch_bounds__(64) k_paths_grad(Problem P, PathArgs A, GradArgs G) {
-    extern __shared__ double gsm[];
-    const int T = blockDim.x, tid = threadIdx.x;
+__global__ void __launch_bounds__(kGradThreads) k_paths_grad(Problem P, PathArgs A, GradArgs G) {
+    extern __shared__ __align__(16) double gsm[];
+    constexpr int T = kGradThreads;
+    constexpr unsigned kAll = 0xffffffffu;
+    const int tid = threadIdx.x, lane = tid & 31, sub = lane & 3, lead = lane & 28;
+    const unsigned gmask = 0xfu << lead;
     const int nw = P.n_rbf, ng = (P.g_kind == PDD_G_BOUNDARY_FOURIER) ? P.n_gcoef : 0;
     const int nf = (P.f_kind == PDD_F_RBF) ? P.n_frbf : 0;
-    double *alpha = gsm;                         // kMaxStencil
-    double *S = alpha + kMaxStencil;             // [nw][T]
-    double *dZ = S + (size_t)nw * T;             // [nw][T]
-    double *Gw = dZ + (size_t)nw * T;            // [nw][T]
-    double *Gg = Gw + (size_t)nw * T;            // [ng][T]
-    double *Gf = Gg + (size_t)ng * T;            // [nf][T]: sum over paths of dZ_tau / dv_q
-    const int slot = blockIdx.x;
+    const int nw4 = (nw + 3) / 4, nf4 = (nf + 3) / 4, ng4 = (ng + 3) / 4;
+    double2 *etab = reinterpret_cast<double2 *>(gsm);     // exp_neg's table
+    double *rx = gsm + 2 * kExpTab, *ry = rx + nw, *rw = ry + nw;
+    double *fx = rw + nw, *fy = fx + nf, *fw = fy + nf;
+    double *alpha = fw + nf;                              // kMaxStencil
+    double *S = alpha + kMaxStencil + tid;                // [nw4][T] each: S_q, dZ_q, psi_q, the sums over paths
+    double *dZ = S + (size_t)nw4 * T;
+    double *psi = dZ + (size_t)nw4 * T;
+    double *Gw = psi + (size_t)nw4 * T;
+    double *Gf = Gw + (size_t)nw4 * T;                    // [nf4][T]: sum over paths of dZ_tau / dv_q
+    double *Gg = Gf + (size_t)nf4 * T;                    // [ng4][T]
+    const int slot = blockIdx.x / G.splits, part = blockIdx.x - slot * G.splits;
     const int gsl = A.gslot ? A.gslot[slot] : slot;
     const int i = A.rows[slot], m = A.subs[gsl];
     const uint32_t kw = A.kword ? (uint32_t)A.kword[gsl] : 0u;
@@ -1393,9 +1419,20 @@ __global__ void __launch_bounds__(64) k_paths_grad(Problem P, PathArgs A, GradAr
         }
         alpha[l] = v;
     }
-    for (int q = 0; q < nw; ++q) Gw[q * T + tid] = 0.0;
-    for (int k = 0; k < ng; ++k) Gg[k * T + tid] = 0.0;
-    for (int q = 0; q < nf; ++q) Gf[q * T + tid] = 0.0;
+    for (int q = tid; q < kExpTab; q += T) etab[q] = kExp2Tab[q];
+    for (int q = tid; q < nw; q += T) {
+        rx[q] = P.rbf_x[q];
+        ry[q] = P.rbf_y[q];
+        rw[q] = P.rbf_w[q];
+    }
+    for (int q = tid; q < nf; q += T) {
+        fx[q] = P.frbf_x[q];
+        fy[q] = P.frbf_y[q];
+        fw[q] = P.frbf_w[q];
+    }
+    for (int q = 0; q < nw4; ++q) Gw[q * T] = 0.0;
+    for (int q = 0; q < nf4; ++q) Gf[q * T] = 0.0;
+    for (int q = 0; q < ng4; ++q) Gg[q * T] = 0.0;
     __syncthreads();
     const double inv2f = nf ? 1.0 / (2.0 * P.frbf_sigma * P.frbf_sigma) : 0.0;
     const double cx = A.ccx[m], cy = A.ccy[m], rad = A.cr[m];
@@ -1415,130 +1452,153 @@ __global__ void __launch_bounds__(64) k_paths_grad(Problem P, PathArgs A, GradAr
     const R h = (R)A.h, sh = Num<R>::sq((R)A.h);
     const double inv2s = nw ? 1.0 / (2.0 * P.rbf_sigma * P.rbf_sigma) : 0.0;
     const int npath = A.npaths ? A.npaths[slot] : A.paths;
-    for (int p = tid; p < npath; p += T) {
-        R x = (R)A.kx[i], y = (R)A.ky[i];
-        double Yv = 1.0, Zv = 0.0;
-        for (int q = 0; q < nw; ++q) {
-            S[q * T + tid] = 0.0;
-            dZ[q * T + tid] = 0.0;
-        }
-        int k = 0;
-        int side = 2;
-        double su = 0.0;
-        for (;;) {
-            if (k >= max_steps) break;
-            R xi0, xi1;
-            Num<R>::normals(A.seed, (uint32_t)i, kw, (uint32_t)k, (uint32_t)p, xi0, xi1);
-            R bx, by;
-            Num<R>::drift(P, x, y, bx, by);
-            const double xd = (double)x, yd = (double)y;
-            double cv = 0.0;
-            if (P.c_kind == PDD_C_RBF) {
-                double s = 0.0;
-                for (int q = 0; q < nw; ++q) {
-                    const double ddx = xd - P.rbf_x[q], ddy = yd - P.rbf_y[q];
-                    s += P.rbf_w[q] * exp(-(ddx * ddx + ddy * ddy) * inv2s);
-                }
-                cv = s < 0.0 ? s : 0.0;
-            } else {
-                cv = (sizeof(R) == 8) ? killing(P, xd, yd) : (double)killing32(P, (float)x, (float)y);
-            }
-            const double fv = SRC ? ((sizeof(R) == 8) ? source(P, xd, yd) : (double)source32(P, (float)x, (float)y)) : 0.0;
-            if (nw && cv < 0.0) {
-                const double fac = A.h / (1.0 + cv * A.h);
-                for (int q = 0; q < nw; ++q) {
-                    const double ddx = xd - P.rbf_x[q], ddy = yd - P.rbf_y[q];
-                    const double psi = exp(-(ddx * ddx + ddy * ddy) * inv2s);
-                    if (SRC) dZ[q * T + tid] += fv * A.h * Yv * S[q * T + tid];
-                    S[q * T + tid] += psi * fac;
-                }
-            } else if (SRC && nw) {
-                for (int q = 0; q < nw; ++q) dZ[q * T + tid] += fv * A.h * Yv * S[q * T + tid];
-            }
-            const double Yn = Yv * (1.0 + cv * A.h);
-            const double Zn = Zv + fv * Yv * A.h;
-            // f's weights: dZ_{k+1} / dv_q = dZ_k / dv_q + psi^f_q(X_k) Y_k h (kept for the paths that exit)
-            for (int q = 0; q < nf; ++q) {
-                const double ddx = xd - P.frbf_x[q], ddy = yd - P.frbf_y[q];
-                Gf[q * T + tid] += exp(-(ddx * ddx + ddy * ddy) * inv2f) * Yv * A.h;
-            }
-            const R nx = x + bx * h + sh * xi0;
-            const R ny = y + by * h + sh * xi1;
-            ++k;
-            const R ddx = nx - rcx, ddy = ny - rcy;
-            const bool out_c = !(ddx * ddx + ddy * ddy < r2);
-            const bool out_d = !inside_domain(Ps, (double)nx, (double)ny);
-            if (!out_c && !out_d) {
-                x = nx;
-                y = ny;
-                Yv = Yn;
-                Zv = Zn;
-                continue;
-            }
-            const double dx = (double)nx - xd, dy = (double)ny - yd;
-            double tc = 2.0, td = 2.0;
-            int ed = -1;
-            if (out_c) tc = circle_exit_t(xd, yd, dx, dy, cx, cy, rs);
-            if (out_d) {
-                if (Ps.dom_kind == 0) {
-                    double t;
-                    if ((double)nx <= Ps.dom[0]) { t = (Ps.dom[0] - xd) / dx; if (t < td) { td = t; ed = 3; } }
-                    if ((double)nx >= Ps.dom[2]) { t = (Ps.dom[2] - xd) / dx; if (t < td) { td = t; ed = 1; } }
-                    if ((double)ny <= Ps.dom[1]) { t = (Ps.dom[1] - yd) / dy; if (t < td) { td = t; ed = 0; } }
-                    if ((double)ny >= Ps.dom[3]) { t = (Ps.dom[3] - yd) / dy; if (t < td) { td = t; ed = 2; } }
-                } else {
-                    td = circle_exit_t(xd, yd, dx, dy, Ps.dom[0], Ps.dom[1], Ps.dom[2]);
-                    ed = 0;
-                }
-            }
-            const bool proj = A.shift > 0.0;
-            if (td <= tc) {
-                side = 1;
-                double ex = xd + td * dx, ey = yd + td * dy;
-                if (proj) {                          // projection onto the true boundary
-                    ex = (double)nx;
-                    ey = (double)ny;
-                    if (P.dom_kind == 0) {
-                        ex = ex < P.dom[0] ? P.dom[0] : (ex > P.dom[2] ? P.dom[2] : ex);
-                        ey = ey < P.dom[1] ? P.dom[1] : (ey > P.dom[3] ? P.dom[3] : ey);
-                        if (ed == 0) ey = P.dom[1];
-                        else if (ed == 1) ex = P.dom[2];
-                        else if (ed == 2) ey = P.dom[3];
-                        else ex = P.dom[0];
+    // this warp's path ids [next, last)
+    const int per_w = (npath + G.splits * (T / 32) - 1) / (G.splits * (T / 32));
+    int next = min(npath, (part * (T / 32) + (tid >> 5)) * per_w);
+    const int last = min(npath, next + per_w);
+    const R x_start = (R)A.kx[i], y_start = (R)A.ky[i];
+    R x = x_start, y = y_start, n0 = (R)0, n1 = (R)0;
+    double Yv = 1.0;
+    int p = 0, k = 0;
+    bool active = false;
+    for (unsigned it = 0;; ++it) {
+        if ((it & 3) == 0) {
+            const unsigned want = __ballot_sync(kAll, !active && sub == 0);
+            if (!active) {
+                p = next + __popc(want & ((1u << lead) - 1u));
+                if (p < last) {
+                    active = true;
+                    x = x_start;
+                    y = y_start;
+                    Yv = 1.0;
+                    k = 0;
+                    for (int q = 0; q < nw4; ++q) {
+                        S[q * T] = 0.0;
+                        dZ[q * T] = 0.0;
                     }
                 }
-                su = boundary_s(P, ex, ey, ed);
-            } else {
-                const double ex = proj ? (double)nx : xd + tc * dx, ey = proj ? (double)ny : yd + tc * dy;
-                double th = atan2(ey - cy, ex - cx);
-                if (th < 0.0) th += PDD_TWO_PI;
-                double uu = th - A.theta_s[m];
-                if (uu < 0.0) uu += PDD_TWO_PI;
-                if (uu >= PDD_TWO_PI) uu -= PDD_TWO_PI;
-                side = 0;
-                su = uu;
             }
-            Yv = Yn;
-            Zv = Zn;
-            break;
+            next = min(last, next + __popc(want));
+            if (!__any_sync(kAll, active)) break;
+            if (active) Num<R>::normals(A.seed, (uint32_t)i, kw, (uint32_t)(k + sub), (uint32_t)p, n0, n1);
         }
-        if (side == 2) continue;
-        double payoff;
-        if (side == 1) {
-            double ex, ey;
-            boundary_point(P, su, ex, ey);
-            payoff = gdata(P, ex, ey, su);
-            if (ng) {
-                const int kc = (P.n_gcoef + 1) / 2;
-                const double wv = PDD_TWO_PI * su / P.perimeter;
-                for (int kk = 0; kk < ng; ++kk) {
-                    const double basis = (kk < kc) ? cos(kk * wv) : sin((kk - kc + 1) * wv);
-                    Gg[kk * T + tid] += Yv * basis;
+        const int src = lead + (int)(it & 3);
+        const R xi0 = __shfl_sync(kAll, n0, src), xi1 = __shfl_sync(kAll, n1, src);
+        if (active && k >= max_steps) active = false;     // a capped path adds nothing to the c and g sums
+        const double xd = (double)x, yd = (double)y;
+        // c and f at X_k: each lane its own basis functions, the two sums over the four lanes
+        double cv = 0.0, fv = 0.0;
+        if (P.c_kind == PDD_C_RBF) {
+            double s = 0.0;
+#pragma unroll 2
+            for (int q = sub, j = 0; q < nw; q += kGradLanes, ++j) {
+                const double ddx = xd - rx[q], ddy = yd - ry[q];
+                const double e = exp_neg(-(ddx * ddx + ddy * ddy) * inv2s, etab);
+                psi[j * T] = e;
+                s += rw[q] * e;
+            }
+            s += __shfl_xor_sync(kAll, s, 1);
+            s += __shfl_xor_sync(kAll, s, 2);
+            cv = s < 0.0 ? s : 0.0;
+        } else {
+            cv = (sizeof(R) == 8) ? killing(P, xd, yd) : (double)killing32(P, (float)x, (float)y);
+        }
+        const double yh = active ? Yv * A.h : 0.0;
+        if (nf) {
+            // f's weights: dZ_{k+1} / dv_q = dZ_k / dv_q + psi^f_q(X_k) Y_k h
+            double s = 0.0;
+            for (int q = sub, j = 0; q < nf; q += kGradLanes, ++j) {
+                const double ddx = xd - fx[q], ddy = yd - fy[q];
+                const double e = exp_neg(-(ddx * ddx + ddy * ddy) * inv2f, etab);
+                Gf[j * T] += e * yh;
+                s += fw[q] * e;
+            }
+            s += __shfl_xor_sync(kAll, s, 1);
+            s += __shfl_xor_sync(kAll, s, 2);
+            fv = s;
+        }
+        if (SRC && sizeof(R) == 4) fv = (double)source32(P, (float)x, (float)y);
+        else if (SRC && !nf) fv = source(P, xd, yd);
+        if (!active) continue;
+        const double fac = cv < 0.0 ? A.h / (1.0 + cv * A.h) : 0.0;
+        const double fhy = fv * yh;
+#pragma unroll 4
+        for (int j = 0; j < nw4; ++j) {
+            const double s = S[j * T];
+            if (SRC) dZ[j * T] += fhy * s;
+            S[j * T] = s + psi[j * T] * fac;
+        }
+        Yv = Yv * (1.0 + cv * A.h);
+        R bx, by;
+        Num<R>::drift(P, x, y, bx, by);
+        const R nx = x + bx * h + sh * xi0;
+        const R ny = y + by * h + sh * xi1;
+        ++k;
+        const R ex0 = nx - rcx, ey0 = ny - rcy;
+        const bool out_c = !(ex0 * ex0 + ey0 * ey0 < r2);
+        const bool out_d = !inside_domain(Ps, (double)nx, (double)ny);
+        if (!out_c && !out_d) {
+            x = nx;
+            y = ny;
+            continue;
+        }
+        active = false;
+        const double dx = (double)nx - xd, dy = (double)ny - yd;
+        double tc = 2.0, td = 2.0;
+        int ed = -1;
+        if (out_c) tc = circle_exit_t(xd, yd, dx, dy, cx, cy, rs);
+        if (out_d) {
+            if (Ps.dom_kind == 0) {
+                double t;
+                if ((double)nx <= Ps.dom[0]) { t = (Ps.dom[0] - xd) / dx; if (t < td) { td = t; ed = 3; } }
+                if ((double)nx >= Ps.dom[2]) { t = (Ps.dom[2] - xd) / dx; if (t < td) { td = t; ed = 1; } }
+                if ((double)ny <= Ps.dom[1]) { t = (Ps.dom[1] - yd) / dy; if (t < td) { td = t; ed = 0; } }
+                if ((double)ny >= Ps.dom[3]) { t = (Ps.dom[3] - yd) / dy; if (t < td) { td = t; ed = 2; } }
+            } else {
+                td = circle_exit_t(xd, yd, dx, dy, Ps.dom[0], Ps.dom[1], Ps.dom[2]);
+                ed = 0;
+            }
+        }
+        const bool proj = A.shift > 0.0;
+        double payoff = 0.0;
+        if (td <= tc) {
+            double ex = xd + td * dx, ey = yd + td * dy;
+            if (proj) {                          // projection onto the true boundary
+                ex = (double)nx;
+                ey = (double)ny;
+                if (P.dom_kind == 0) {
+                    ex = ex < P.dom[0] ? P.dom[0] : (ex > P.dom[2] ? P.dom[2] : ex);
+                    ey = ey < P.dom[1] ? P.dom[1] : (ey > P.dom[3] ? P.dom[3] : ey);
+                    if (ed == 0) ey = P.dom[1];
+                    else if (ed == 1) ex = P.dom[2];
+                    else if (ed == 2) ey = P.dom[3];
+                    else ex = P.dom[0];
                 }
             }
+            const double su = boundary_s(P, ex, ey, ed);
+            if (ng) {
+                // the boundary series and its coefficients' derivatives share their basis values
+                const int kc = (P.n_gcoef + 1) / 2;
+                const double wv = PDD_TWO_PI * su / P.perimeter;
+                for (int kk = sub, j = 0; kk < ng; kk += kGradLanes, ++j) {
+                    const double basis = (kk < kc) ? cos(kk * wv) : sin((kk - kc + 1) * wv);
+                    Gg[j * T] += Yv * basis;
+                    payoff += P.g_coef[kk] * basis;
+                }
+                payoff += __shfl_xor_sync(gmask, payoff, 1);
+                payoff += __shfl_xor_sync(gmask, payoff, 2);
+            } else {
+                boundary_point(P, su, ex, ey);
+                payoff = gdata(P, ex, ey, su);
+            }
         } else {
-            payoff = 0.0;
-            for (int l = 0; l < ns; ++l) {
+            const double ex = proj ? (double)nx : xd + tc * dx, ey = proj ? (double)ny : yd + tc * dy;
+            double th = atan2(ey - cy, ex - cx);
+            if (th < 0.0) th += PDD_TWO_PI;
+            double su = th - A.theta_s[m];
+            if (su < 0.0) su += PDD_TWO_PI;
+            if (su >= PDD_TWO_PI) su -= PDD_TWO_PI;
+            for (int l = sub; l < ns; l += kGradLanes) {
                 double ph;
                 if (imq) {
                     const double d = su - G.ku[a + l];
@@ -1549,18 +1609,21 @@ __global__ void __launch_bounds__(64) k_paths_grad(Problem P, PathArgs A, GradAr
                 }
                 payoff += alpha[l] * ph;
             }
+            payoff += __shfl_xor_sync(gmask, payoff, 1);
+            payoff += __shfl_xor_sync(gmask, payoff, 2);
         }
-        for (int q = 0; q < nw; ++q) Gw[q * T + tid] += payoff * Yv * S[q * T + tid] + dZ[q * T + tid];
+        for (int j = 0; j < nw4; ++j) Gw[j * T] += payoff * Yv * S[j * T] + dZ[j * T];
     }
     __syncthreads();
-    // partial layout [c weights][f weights][g coefficients]
+    // partial layout [c weights][f weights][g coefficients]; index q sits with the lanes of sub q mod 4
     const double scale = G.lambda[i] / npath;
     for (int q = tid; q < nw + nf + ng; q += T) {
-        const double *src = (q < nw) ? Gw + (size_t)q * T
-                                     : (q < nw + nf ? Gf + (size_t)(q - nw) * T : Gg + (size_t)(q - nw - nf) * T);
+        const double *src = (q < nw) ? Gw - tid : (q < nw + nf ? Gf - tid : Gg - tid);
+        const int l = q < nw ? q : (q < nw + nf ? q - nw : q - nw - nf);
+        src += (size_t)(l >> 2) * T + (l & 3);
         double s = 0.0;
-        for (int t = 0; t < T; ++t) s += src[t];
-        G.partial[(long)slot * G.n_par + q] = scale * s;
+        for (int t = 0; t < T; t += kGradLanes) s += src[t];
+        G.partial[(long)blockIdx.x * G.n_par + q] = scale * s;
     }
 }
 
@@ -1576,8 +1639,14 @@ void grad_mc(const pdd_cover &cov, const Problem &P, const pdd_assembly_opts &o,
     DevBuf<long> koff_m;
     build_imq_inverses(cov, o.imq_c2, kinv, koff_m, kcond, st);
     const int n_par = nw + nf + ng;
-    partial.alloc((size_t)nmc * n_par);
-    PDD_CUDA(cudaMemsetAsync(partial.p, 0, sizeof(double) * nmc * n_par, st));
+    // parts of a row: enough CTAs to even out rows of unequal path lengths over the SMs, each warp
+    // keeping at least 64 paths of a full row (eight per group of four lanes) so that the lanes idle
+    // while a warp's last paths finish stay few
+    int dev = 0, sms = 0;
+    PDD_CUDA(cudaGetDevice(&dev));
+    PDD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int splits = std::max(1, std::min({cdiv(8L * sms, nmc), cdiv(o.paths, 64 * (kGradThreads / 32)), 64}));
+    partial.alloc((size_t)nmc * splits * n_par);
     DevBuf<unsigned long long> steps;
     DevBuf<int> capped;
     steps.alloc(1);
@@ -1586,16 +1655,15 @@ void grad_mc(const pdd_cover &cov, const Problem &P, const pdd_assembly_opts &o,
                cov.theta_s.p, o.paths, o.h, o.seed, nullptr, nullptr, nullptr, nullptr, steps.p, capped.p,
                sys.mc_np.p, nullptr, nullptr, o.boundary_shift ? kGmC0 * sqrt(o.h) : 0.0, nullptr, o.max_steps, 0, 0,
                nullptr};
-    GradArgs G{u, lambda, cov.knot_ptr.p, cov.floating.p, cov.ku.p, koff_m.p, kinv.p, o.imq_c2, n_par, partial.p};
-    const int T = 64;
-    const size_t smem = (size_t)(kMaxStencil + (3 * nw + ng + nf) * T) * sizeof(double);
-    if (smem > 220 * 1024) fail(PDD_EINVAL, "too many gradient parameters for the replay kernel");
+    GradArgs G{u, lambda, cov.knot_ptr.p, cov.floating.p, cov.ku.p, koff_m.p, kinv.p, o.imq_c2, n_par, splits, partial.p};
+    const size_t smem = grad_smem_doubles(nw, nf, ng) * sizeof(double);
+    if (3 * nw + ng + nf > kGradMaxParams) fail(PDD_EINVAL, "too many gradient parameters for the replay kernel");
     const bool src = P.f_kind != PDD_F_ZERO;
 #define PDD_GRAD_LAUNCH(R, SRCV)                                                                          \
     do {                                                                                                  \
         PDD_CUDA(cudaFuncSetAttribute(k_paths_grad<R, SRCV>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                       (int)smem));                                                       \
-        PDD_LAUNCH((k_paths_grad<R, SRCV>), nmc, T, smem, st, P, A, G);                                   \
+        PDD_LAUNCH((k_paths_grad<R, SRCV>), nmc * splits, kGradThreads, smem, st, P, A, G);                                   \
     } while (0)
     if (path_mixed(o)) {
         if (src) PDD_GRAD_LAUNCH(float, true); else PDD_GRAD_LAUNCH(float, false);
@@ -1603,7 +1671,7 @@ void grad_mc(const pdd_cover &cov, const Problem &P, const pdd_assembly_opts &o,
         if (src) PDD_GRAD_LAUNCH(double, true); else PDD_GRAD_LAUNCH(double, false);
     }
 #undef PDD_GRAD_LAUNCH
-    n_part = nmc;
+    n_part = nmc * splits;
 }
 
 }  // namespace pdd
