@@ -165,7 +165,8 @@ __device__ __forceinline__ void u46_derivs(T x, T y, T &u, T &ux, T &uy, T &lap)
     lap = (cs * lap_s - ss * g2s + sech2 * (lap_w - T(2) * t * (wx * wx + wy * wy))) * third;
 }
 
-__device__ __forceinline__ double source(const Problem &P, double x, double y) {
+// f from already evaluated b and c
+__device__ __forceinline__ double source_given(const Problem &P, double x, double y, double bx, double by, double cv) {
     if (P.f_kind == PDD_F_RBF) {
         const double inv = 1.0 / (2.0 * P.frbf_sigma * P.frbf_sigma);
         double s = 0.0;
@@ -183,17 +184,23 @@ __device__ __forceinline__ double source(const Problem &P, double x, double y) {
         double u = spx * cpy;
         double ux = PDD_PI * cpx * cpy;
         double uy = -PDD_PI * spx * spy;
-        double bx, by;
-        drift(P, x, y, bx, by);
-        return -(-PDD_PI * PDD_PI * u + bx * ux + by * uy + killing(P, x, y) * u);
+        return -(-PDD_PI * PDD_PI * u + bx * ux + by * uy + cv * u);
     }
     if (P.f_kind == PDD_F_EQ46) {
-        double u, ux, uy, lap, bx, by;
+        double u, ux, uy, lap;
         u46_derivs(x, y, u, ux, uy, lap);
-        drift(P, x, y, bx, by);
-        return -(0.5 * lap + bx * ux + by * uy + killing(P, x, y) * u);
+        return -(0.5 * lap + bx * ux + by * uy + cv * u);
     }
     return 0.0;
+}
+
+__device__ __forceinline__ double source(const Problem &P, double x, double y) {
+    if (P.f_kind == PDD_F_MANUFACTURED || P.f_kind == PDD_F_EQ46) {
+        double bx, by;
+        drift(P, x, y, bx, by);
+        return source_given(P, x, y, bx, by, killing(P, x, y));
+    }
+    return source_given(P, x, y, 0.0, 0.0, 0.0);
 }
 
 // boundary Fourier series at arclength s (a_0..a_{Kc-1} cos, b_1..b_Ks sin)
@@ -339,10 +346,16 @@ __device__ __forceinline__ U4 philox10(uint32_t c0, uint32_t c1, uint32_t c2, ui
     return U4{c0, c1, c2, c3};
 }
 
-// two 53-bit uniforms in (0, 1] from the four words
+// (m + 1/2) 2^-53 rounded to FP64, m the 53 bits of two words: in (0, 1].  Put together from the bit
+// fields: below 2^52 m + 1/2 is exact (one subtraction from 2^52 + m); above, the half is a tie,
+// rounded to the even neighbour by an integer addition.
 __device__ __forceinline__ double uniform53(uint32_t a, uint32_t b) {
-    uint64_t m = ((uint64_t)a << 21) ^ (uint64_t)(b >> 11);
-    return ((double)m + 0.5) * 1.1102230246251565e-16;
+    const uint64_t m = ((uint64_t)a << 21) ^ (uint64_t)(b >> 11);
+    const uint64_t ml = m & 0xfffffffffffffULL;
+    const uint64_t bits = 0x4330000000000000ULL | ml;
+    const double v = (a >> 31) ? __longlong_as_double((long long)(bits + (ml & 1)))
+                               : __longlong_as_double((long long)bits) - 4503599627370495.5;
+    return __hiloint2double(__double2hiint(v) - (53 << 20), __double2loint(v));
 }
 
 // key (seed_lo32, knot), counter (step, path, 0, sub): sub is the position of the subdomain in the

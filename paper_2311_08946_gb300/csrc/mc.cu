@@ -275,8 +275,10 @@ __device__ __forceinline__ void cv_accumulate(R (&cq)[kMaxCv], int D, R xr, R yr
     }
 }
 
-template <typename R, bool KILL, bool SRC, bool CV>
+// mixed form: positions, drift and normals in FP32, weights in FP64
+template <bool KILL, bool SRC, bool CV>
 __global__ void __launch_bounds__(256) k_paths(Problem P, PathArgs A) {
+    using R = float;
     __shared__ int next_path;
     const int slot = blockIdx.x;
     const int gsl = A.gslot ? A.gslot[slot] : slot;
@@ -342,7 +344,7 @@ __global__ void __launch_bounds__(256) k_paths(Problem P, PathArgs A) {
             A.su[rec] = 0.0;
             A.Y[rec] = 0.0;
             A.Z[rec] = 0.0;
-            if constexpr (sizeof(R) == 4) A.ez[rec] = make_float2(0.f, 0.f);
+            A.ez[rec] = make_float2(0.f, 0.f);
             if constexpr (CV)
                 for (int q = 0; q < A.ncv; ++q) A.cvq[rec * A.ncv + q] = 0.0;
             ++my_capped;
@@ -352,23 +354,17 @@ __global__ void __launch_bounds__(256) k_paths(Problem P, PathArgs A) {
             Num<R>::normals(A.seed, (uint32_t)i, kw, (uint32_t)k, (uint32_t)p, xi0, xi1);
             if constexpr (CV) {
                 // Y_k sqrt(h) grad psi(X_k) . xi_k / r, with Y_k the weight before this step
-                const R yk = sizeof(R) == 8 ? (R)Yv : (R)((float)Yv * (1.0f + e));
+                const R yk = (float)Yv * (1.0f + e);
                 cv_accumulate<R>(cq, A.cvd, (x - rcx) / crad, (y - rcy) / crad, yk * sh / crad, xi0, xi1);
             }
             R bx, by;
             Num<R>::drift(P, x, y, bx, by);
             double Yn = Yv, Zn = Zv;
             float en = e, zn = z;
-            if constexpr (sizeof(R) == 8) {
-                // FP64 form: the same expressions as the definition (identical streams)
-                if (KILL) Yn = Yv * (1.0 + killing(P, (double)x, (double)y) * A.h);
-                if (SRC) Zn = Zv + source(P, (double)x, (double)y) * Yv * A.h;
-            } else {
-                const float cv = KILL ? killing32(P, (float)x, (float)y) : 0.f;
-                // Z_{k+1} = Z_k + f_k h Y_k and Y_{k+1} = Y_k (1 + c_k h), with Y_k = Yv (1 + e)
-                if (SRC) zn = fmaf(source32_given(P, (float)x, (float)y, (float)bx, (float)by, cv) * hf, 1.0f + e, z);
-                if (KILL) en = fmaf(cv * hf, 1.0f + e, e);
-            }
+            const float cv = KILL ? killing32(P, x, y) : 0.f;
+            // Z_{k+1} = Z_k + f_k h Y_k and Y_{k+1} = Y_k (1 + c_k h), with Y_k = Yv (1 + e)
+            if (SRC) zn = fmaf(source32_given(P, x, y, bx, by, cv) * hf, 1.0f + e, z);
+            if (KILL) en = fmaf(cv * hf, 1.0f + e, e);
             const R nx = x + bx * h + sh * xi0;
             const R ny = y + by * h + sh * xi1;
             ++k;
@@ -382,16 +378,14 @@ __global__ void __launch_bounds__(256) k_paths(Problem P, PathArgs A) {
                 in_d = ex0 * ex0 + ey0 * ey0 < dr2;
             }
             const bool out_d = !in_d;
-            if constexpr (sizeof(R) == 4) {
-                // fold the FP32 increments into the FP64 weights every 8 iterations of the loop (the
-                // same iterations in every lane of the warp, so the FP64 work is not divergent); the
-                // increments left at the exit go to the record and the finalize folds them
-                if ((++it & 7) == 0) {
-                    Zn = fma(Yv, (double)zn, Zv);
-                    Yn = fma(Yv, (double)en, Yv);
-                    en = 0.f;
-                    zn = 0.f;
-                }
+            // fold the FP32 increments into the FP64 weights every 8 iterations of the loop (the
+            // same iterations in every lane of the warp, so the FP64 work is not divergent); the
+            // increments left at the exit go to the record and the finalize folds them
+            if ((++it & 7) == 0) {
+                Zn = fma(Yv, (double)zn, Zv);
+                Yn = fma(Yv, (double)en, Yv);
+                en = 0.f;
+                zn = 0.f;
             }
             if (!out_c && !out_d) {
                 x = nx;
@@ -401,7 +395,7 @@ __global__ void __launch_bounds__(256) k_paths(Problem P, PathArgs A) {
                 e = en;
                 z = zn;
             } else {
-                // exit point on the segment, in the position type (FP64 form: FP64; mixed: FP32); with
+                // exit point on the segment, in FP32; with
                 // the boundary shift the piece crossed first (on the shrunk boundaries) is scored at the
                 // projection of the first point outside onto the true boundary
                 const R dx = nx - x, dy = ny - y;
@@ -451,7 +445,7 @@ __global__ void __launch_bounds__(256) k_paths(Problem P, PathArgs A) {
                 }
                 A.Y[rec] = Yn;
                 A.Z[rec] = Zn;
-                if constexpr (sizeof(R) == 4) A.ez[rec] = make_float2(en, zn);
+                A.ez[rec] = make_float2(en, zn);
                 if constexpr (CV) {
 #pragma unroll
                     for (int q = 0; q < kMaxCv; ++q)
@@ -497,6 +491,340 @@ __global__ void __launch_bounds__(256) k_paths(Problem P, PathArgs A) {
         }
         atomicAdd(A.steps, t);
         if (c) atomicAdd(A.capped, c);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// FP64 form.  The FP64 pipe bounds it (1/64 of the FP32 rate: a warp instruction occupies an SM's
+// unit for 16 cycles whatever the number of its lanes in use), so the design keeps the lanes full
+// and takes FP64 instructions out of the step, with every value rounded as the plain expressions are:
+//   * persistent warps; a lane whose path exits takes the launch's next path, of whatever row (rows
+//     of unequal path lengths or fewer rows than SMs leave nothing idle);
+//   * when the queue is empty, a warp with few paths left hands their states over and ends; the next
+//     launch packs them into full warps (four launches, the last runs to completion);
+//   * the exit point of a path (roots, divisions, an arctangent) is left to k_exit64, one thread per
+//     record, instead of being computed by one lane while 31 wait;
+//   * the uniforms are put together from their bits, the comparisons with the domain's box are integer
+//     comparisons, the circle is tested in FP32 first.
+// 4 x 4 lattice (116 rows x 1,000 paths): 9.4 -> 6.1 ms; 140 circles with variable coefficients, 10^4
+// paths a row: 325 -> 189 ms.
+// ---------------------------------------------------------------------------
+struct alignas(16) Slot64 {          // what a path reads when it starts
+    double cx, cy, r, r2, x0, y0;    // r2: of the disk shrunk by the boundary shift
+    long rbase;
+    int i, max_steps;
+    uint32_t kw;
+};
+struct alignas(16) PathState {
+    double x, y, Y, Z;
+    int slot, p, k, pad;
+};
+struct alignas(16) Seg64 {
+    double x, y, nx, ny;
+};
+struct PathPool {
+    const Slot64 *slots;
+    int nslots;
+    unsigned long long total;        // paths of the launch (first pass)
+    unsigned long long *next;        // queue position
+    const PathState *in;             // states handed over by the previous pass (null: first pass)
+    const unsigned *n_in;
+    PathState *out;                  // and by this one
+    unsigned *n_out;
+    int keep;                        // fewer live paths than this in a warp are handed over (0: none are)
+    const double *cq_in;             // control-variate features of the states, [state][ncv]
+    double *cq_out;
+    Seg64 *seg;                      // per record: the last step's segment
+};
+
+static constexpr int kP64Threads = 64;
+static constexpr int kP64WarpsPerSm = 8;
+static constexpr int kP64Staged = 1024;        // most Gaussians kept in shared memory (24 KB)
+
+__global__ void k_slots64(int n, PathArgs A, Slot64 *out) {
+    const int slot = blockIdx.x * blockDim.x + threadIdx.x;
+    if (slot >= n) return;
+    const int gsl = A.gslot ? A.gslot[slot] : slot;
+    const int i = A.rows[slot], m = A.subs[gsl];
+    const double rad = A.cr[m], rs = rad - A.shift;
+    Slot64 s;
+    s.cx = A.ccx[m];
+    s.cy = A.ccy[m];
+    s.r = rad;
+    s.r2 = rs * rs;
+    s.x0 = A.kx[i];
+    s.y0 = A.ky[i];
+    s.rbase = A.rec_off ? A.rec_off[slot] : (long)slot * A.paths;
+    s.i = i;
+    s.max_steps = A.max_steps > 0 ? A.max_steps : (int)fmin(2147483647.0, ceil(50.0 * rad * rad / A.h));
+    s.kw = A.kword ? (uint32_t)A.kword[gsl] : 0u;
+    out[slot] = s;
+}
+
+// the slot of record g (the records of the slots are contiguous and in slot order)
+__device__ __forceinline__ int slot_of(const PathArgs &A, const Slot64 *slots, int nslots, unsigned long long g) {
+    if (!A.rec_off) return (int)((unsigned)g / (unsigned)A.paths);      // at most 2^31 records per launch
+    int lo = 0, hi = nslots - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if ((unsigned long long)slots[mid].rbase <= g) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
+// an order-preserving integer of a double (-0 below +0; no NaN)
+__device__ __forceinline__ long long order_key(double v) {
+    const long long b = __double_as_longlong(v);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+
+// the leading 24 bits of a double as FP32 (values below 2^-126 give an arbitrary value at most 4)
+__device__ __forceinline__ float trunc32(double v) {
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    return __uint_as_float(((__funnelshift_l(lo, hi, 3) ^ 0x40000000u) & 0x7fffffffu) | (hi & 0x80000000u));
+}
+
+template <bool KILL, bool SRC, bool CV>
+__global__ void __launch_bounds__(kP64Threads) k_paths64(Problem P, PathArgs A, PathPool Q) {
+    constexpr unsigned kAll = 0xffffffffu;
+    // killing by Gaussians: exp_neg's table, then x, y, w (in global memory when they are many)
+    extern __shared__ __align__(16) double psm64[];
+    const double2 *etab = reinterpret_cast<const double2 *>(psm64);
+    const int nr = KILL && P.c_kind == PDD_C_RBF ? P.n_rbf : 0;
+    const bool staged = nr <= kP64Staged;
+    const double *rx = staged ? psm64 + 2 * kExpTab : P.rbf_x, *ry = staged ? rx + nr : P.rbf_y;
+    const double *rw = staged ? ry + nr : P.rbf_w;
+    const double inv2s = nr ? 1.0 / (2.0 * P.rbf_sigma * P.rbf_sigma) : 0.0;
+    if (nr) {
+        double2 *et = reinterpret_cast<double2 *>(psm64);
+        double *rt = psm64 + 2 * kExpTab;
+        for (int q = threadIdx.x; q < kExpTab; q += kP64Threads) et[q] = kExp2Tab[q];
+        for (int q = threadIdx.x; staged && q < nr; q += kP64Threads) {
+            rt[q] = P.rbf_x[q];
+            rt[nr + q] = P.rbf_y[q];
+            rt[2 * nr + q] = P.rbf_w[q];
+        }
+        __syncthreads();
+    }
+    const bool sq_dom = P.dom_kind == 0, has_b = P.b_kind != PDD_B_ZERO;
+    const double sft = A.shift;
+    const double d0 = sq_dom ? P.dom[0] + sft : P.dom[0], d1 = sq_dom ? P.dom[1] + sft : P.dom[1];
+    const double d2 = P.dom[2] - sft, d3 = P.dom[3] - sft;
+    const double dr2 = (P.dom[2] - sft) * (P.dom[2] - sft);
+    const long long q0 = order_key(d0 + 0.0), q1 = order_key(d1 + 0.0), q2 = order_key(d2), q3 = order_key(d3);
+    const double h = A.h, sh = sqrt(A.h);
+    const unsigned long long total = Q.in ? (unsigned long long)*Q.n_in : Q.total;
+    unsigned long long my_steps = 0;
+    int my_capped = 0;
+    bool have = false, drained = false;
+    double x = 0.0, y = 0.0, Yv = 1.0, Zv = 0.0, cx = 0.0, cy = 0.0, r2 = 0.0, crad = 1.0;
+    float r2f = 0.f;
+    long rec = 0;
+    int slot = 0, p = 0, k = 0, knot = 0, max_steps = 0;
+    uint32_t kw = 0;
+    double cq[CV ? kMaxCv : 1];
+    for (;;) {
+        if (!have && !drained) {
+            const unsigned long long g = atomicAdd(Q.next, 1ULL);
+            drained = g >= total;
+            if (!drained) {
+                have = true;
+                if (Q.in) {
+                    const PathState s = Q.in[g];
+                    slot = s.slot;
+                    p = s.p;
+                    k = s.k;
+                    x = s.x;
+                    y = s.y;
+                    Yv = s.Y;
+                    Zv = s.Z;
+                } else {
+                    slot = slot_of(A, Q.slots, Q.nslots, g);
+                    p = (int)(g - (unsigned long long)Q.slots[slot].rbase);
+                    k = 0;
+                    x = Q.slots[slot].x0;
+                    y = Q.slots[slot].y0;
+                    Yv = 1.0;
+                    Zv = 0.0;
+                }
+                const Slot64 *S = Q.slots + slot;
+                cx = S->cx;
+                cy = S->cy;
+                if (CV) crad = S->r;
+                r2 = S->r2;
+                r2f = trunc32(r2) * 0.9999f;
+                rec = S->rbase + p;
+                knot = S->i;
+                max_steps = S->max_steps;
+                kw = S->kw;
+                if constexpr (CV) {
+#pragma unroll
+                    for (int q = 0; q < kMaxCv; ++q) cq[q] = (Q.in && q < A.ncv) ? Q.cq_in[g * A.ncv + q] : 0.0;
+                }
+            }
+        }
+        const unsigned live = __ballot_sync(kAll, have);
+        if (__popc(live) < Q.keep || !live) {             // (below `keep` only once the queue is empty)
+            if (have) {
+                const unsigned o = atomicAdd(Q.n_out, 1u);
+                Q.out[o] = PathState{x, y, Yv, Zv, slot, p, k, 0};
+                if constexpr (CV) {
+#pragma unroll
+                    for (int q = 0; q < kMaxCv; ++q)
+                        if (q < A.ncv) Q.cq_out[(size_t)o * A.ncv + q] = cq[q];
+                }
+            }
+            break;
+        }
+        if (!have) continue;
+        if (k >= max_steps) {
+            A.side[rec] = 2;
+            A.su[rec] = 0.0;
+            A.Y[rec] = 0.0;
+            A.Z[rec] = 0.0;
+            if constexpr (CV)
+                for (int q = 0; q < A.ncv; ++q) A.cvq[rec * A.ncv + q] = 0.0;
+            ++my_capped;
+            my_steps += (unsigned long long)k;
+            have = false;
+            continue;
+        }
+        double xi0, xi1;
+        normals64(A.seed, (uint32_t)knot, kw, (uint32_t)k, (uint32_t)p, xi0, xi1);
+        if constexpr (CV) {
+            // Y_k sqrt(h) grad psi(X_k) . xi_k / r, with Y_k the weight before this step
+            cv_accumulate<double>(cq, A.cvd, (x - cx) / crad, (y - cy) / crad, Yv * sh / crad, xi0, xi1);
+        }
+        double bx = 0.0, by = 0.0;
+        if (has_b) drift(P, x, y, bx, by);
+        double Yn = Yv, Zn = Zv, cv = 0.0;
+        if (KILL) {
+            if (nr) {
+                double s = 0.0;
+#pragma unroll 4
+                for (int q = 0; q < nr; ++q) {
+                    const double dx = x - rx[q], dy = y - ry[q];
+                    s += rw[q] * exp_neg(-(dx * dx + dy * dy) * inv2s, etab);
+                }
+                cv = s < 0.0 ? s : 0.0;
+            } else {
+                cv = killing(P, x, y);
+            }
+            Yn = Yv * (1.0 + cv * A.h);
+        }
+        if (SRC) Zn = Zv + source_given(P, x, y, bx, by, cv) * Yv * A.h;
+        const double nx = has_b ? x + bx * h + sh * xi0 : x + sh * xi0;
+        const double ny = has_b ? y + by * h + sh * xi1 : y + sh * xi1;
+        ++k;
+        const double ddx = nx - cx, ddy = ny - cy;
+        const float fx = trunc32(ddx), fy = trunc32(ddy);
+        // surely inside below 0.9999 r^2 (the FP32 sum is off by 2^-21), for |ddx| and |ddy| below 2^49
+        const unsigned top = max((unsigned)__double2hiint(ddx) & 0x7fffffffu, (unsigned)__double2hiint(ddy) & 0x7fffffffu);
+        bool out = !(fx * fx + fy * fy < r2f && top < 0x43000000u);
+        if (out) out = !(ddx * ddx + ddy * ddy < r2);
+        if (sq_dom) {
+            const long long kx = order_key(nx), ky = order_key(ny);
+            out = out || !(kx > q0 && kx < q2 && ky > q1 && ky < q3);
+        } else {
+            const double ex0 = nx - d0, ey0 = ny - d1;
+            out = out || !(ex0 * ex0 + ey0 * ey0 < dr2);
+        }
+        if (!out) {
+            x = nx;
+            y = ny;
+            Yv = Yn;
+            Zv = Zn;
+            continue;
+        }
+        A.side[rec] = 3;                                  // k_exit64 finds the side and the exit point
+        Q.seg[rec] = Seg64{x, y, nx, ny};
+        A.Y[rec] = Yn;
+        A.Z[rec] = Zn;
+        if constexpr (CV) {
+#pragma unroll
+            for (int q = 0; q < kMaxCv; ++q)
+                if (q < A.ncv) A.cvq[rec * A.ncv + q] = cq[q];
+        }
+        my_steps += (unsigned long long)k;
+        have = false;
+    }
+    for (int o = 16; o; o >>= 1) {
+        my_steps += __shfl_xor_sync(kAll, my_steps, o);
+        my_capped += __shfl_xor_sync(kAll, my_capped, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        if (my_steps) atomicAdd(A.steps, my_steps);
+        if (my_capped) atomicAdd(A.capped, my_capped);
+    }
+}
+
+// the exit point of every record's last segment, as in k_paths (in FP64)
+__global__ void __launch_bounds__(256) k_exit64(Problem P, PathArgs A, PathPool Q) {
+    const unsigned long long rec = blockIdx.x * 256ULL + threadIdx.x;
+    if (rec >= Q.total || A.side[rec] != 3) return;
+    const int slot = slot_of(A, Q.slots, Q.nslots, rec);
+    const int m = A.subs[A.gslot ? A.gslot[slot] : slot];
+    const bool sq_dom = P.dom_kind == 0;
+    const double sft = A.shift;
+    const double d0 = sq_dom ? P.dom[0] + sft : P.dom[0], d1 = sq_dom ? P.dom[1] + sft : P.dom[1];
+    const double d2 = P.dom[2] - sft, d3 = P.dom[3] - sft;
+    const double dr2 = (P.dom[2] - sft) * (P.dom[2] - sft);
+    const double rcx = Q.slots[slot].cx, rcy = Q.slots[slot].cy, r2 = Q.slots[slot].r2, rs = A.cr[m] - sft;
+    const Seg64 s = Q.seg[rec];
+    const double x = s.x, y = s.y, nx = s.nx, ny = s.ny;
+    const double ddx = nx - rcx, ddy = ny - rcy;
+    const bool out_c = !(ddx * ddx + ddy * ddy < r2);
+    bool out_d;
+    if (sq_dom) {
+        out_d = !(nx > d0 && nx < d2 && ny > d1 && ny < d3);
+    } else {
+        const double ex0 = nx - d0, ey0 = ny - d1;
+        out_d = !(ex0 * ex0 + ey0 * ey0 < dr2);
+    }
+    const double dx = nx - x, dy = ny - y;
+    double tc = 2.0, td = 2.0;
+    int ed = -1;
+    if (out_c) tc = circle_exit_t(x, y, dx, dy, rcx, rcy, rs);
+    if (out_d) {
+        if (sq_dom) {
+            double t;
+            if (nx <= d0) { t = (d0 - x) / dx; if (t < td) { td = t; ed = 3; } }
+            if (nx >= d2) { t = (d2 - x) / dx; if (t < td) { td = t; ed = 1; } }
+            if (ny <= d1) { t = (d1 - y) / dy; if (t < td) { td = t; ed = 0; } }
+            if (ny >= d3) { t = (d3 - y) / dy; if (t < td) { td = t; ed = 2; } }
+        } else {
+            td = circle_exit_t(x, y, dx, dy, d0, d1, d2);
+            ed = 0;
+        }
+    }
+    const bool proj = A.shift > 0.0;
+    if (td <= tc) {
+        double ex = x + td * dx, ey = y + td * dy;
+        if (proj) {
+            ex = nx;
+            ey = ny;
+            if (sq_dom) {
+                const double x0 = P.dom[0], y0 = P.dom[1], x1 = P.dom[2], y1 = P.dom[3];
+                ex = ex < x0 ? x0 : (ex > x1 ? x1 : ex);
+                ey = ey < y0 ? y0 : (ey > y1 ? y1 : ey);
+                if (ed == 0) ey = y0;
+                else if (ed == 1) ex = x1;
+                else if (ed == 2) ey = y1;
+                else ex = x0;
+            }                                             // disk domain: the arclength is the angle's
+        }
+        A.side[rec] = 1;
+        A.su[rec] = boundary_s(P, ex, ey, ed);
+    } else {
+        const double ex = proj ? nx : x + tc * dx, ey = proj ? ny : y + tc * dy;
+        double th = atan2(ey - rcy, ex - rcx);
+        if (th < 0.0) th += PDD_TWO_PI;
+        double u = th - A.theta_s[m];
+        if (u < 0.0) u += PDD_TWO_PI;
+        if (u >= PDD_TWO_PI) u -= PDD_TWO_PI;
+        A.side[rec] = 0;
+        A.su[rec] = u;
     }
 }
 
@@ -1145,19 +1473,81 @@ __global__ void k_need(int nmc, const int *rows, const int *subs, const int *spo
     need[slot] = w > Pmax ? Pmax : w;
 }
 
-template <typename R, bool CV>
+template <bool CV>
 static void launch_paths_cv(const Problem &P, const PathArgs &A, int nrows, cudaStream_t st) {
     const bool kill = P.c_kind != PDD_C_ZERO, src = P.f_kind != PDD_F_ZERO;
-    if (kill && src) PDD_LAUNCH((k_paths<R, true, true, CV>), nrows, 256, 0, st, P, A);
-    else if (kill) PDD_LAUNCH((k_paths<R, true, false, CV>), nrows, 256, 0, st, P, A);
-    else if (src) PDD_LAUNCH((k_paths<R, false, true, CV>), nrows, 256, 0, st, P, A);
-    else PDD_LAUNCH((k_paths<R, false, false, CV>), nrows, 256, 0, st, P, A);
+    if (kill && src) PDD_LAUNCH((k_paths<true, true, CV>), nrows, 256, 0, st, P, A);
+    else if (kill) PDD_LAUNCH((k_paths<true, false, CV>), nrows, 256, 0, st, P, A);
+    else if (src) PDD_LAUNCH((k_paths<false, true, CV>), nrows, 256, 0, st, P, A);
+    else PDD_LAUNCH((k_paths<false, false, CV>), nrows, 256, 0, st, P, A);
 }
 
-template <typename R>
 static void launch_paths(const Problem &P, const PathArgs &A, int nrows, cudaStream_t st) {
-    if (A.cvd > 0) launch_paths_cv<R, true>(P, A, nrows, st);
-    else launch_paths_cv<R, false>(P, A, nrows, st);
+    if (A.cvd > 0) launch_paths_cv<true>(P, A, nrows, st);
+    else launch_paths_cv<false>(P, A, nrows, st);
+}
+
+// buffers of the FP64 form's passes, kept over the waves of one assembly
+struct Paths64Bufs {
+    DevBuf<Slot64> slots;
+    DevBuf<PathState> state[2];
+    DevBuf<double> cq[2];
+    DevBuf<Seg64> seg;
+    DevBuf<unsigned long long> next;     // one queue per pass
+    DevBuf<unsigned> count;
+};
+static constexpr int kP64Passes = 4;
+
+template <bool CV>
+static void launch_pass64(const Problem &P, const PathArgs &A, const PathPool &Q, int grid, size_t sm,
+                          cudaStream_t st) {
+    const bool kill = P.c_kind != PDD_C_ZERO, src = P.f_kind != PDD_F_ZERO;
+    auto kern = kill ? (src ? k_paths64<true, true, CV> : k_paths64<true, false, CV>)
+                     : (src ? k_paths64<false, true, CV> : k_paths64<false, false, CV>);
+    PDD_LAUNCH(kern, grid, kP64Threads, sm, st, P, A, Q);
+}
+
+// nrows slots with `total` paths in all, their records contiguous in slot order
+static void run_paths64(const Problem &P, const PathArgs &A, int nrows, long total, Paths64Bufs &B, cudaStream_t st) {
+    int dev = 0, sms = 0;
+    PDD_CUDA(cudaGetDevice(&dev));
+    PDD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int ctas = std::max(1, std::min(cdiv(total, kP64Threads), sms * kP64WarpsPerSm * 32 / kP64Threads));
+    const size_t lanes = (size_t)ctas * kP64Threads;
+    if (B.slots.n < (size_t)nrows) B.slots.alloc(nrows);
+    if (B.seg.n < (size_t)total) B.seg.alloc(total);
+    if (B.state[0].n < lanes)
+        for (auto &s : B.state) s.alloc(lanes);
+    if (A.ncv && B.cq[0].n < lanes * A.ncv)
+        for (auto &c : B.cq) c.alloc(lanes * A.ncv);
+    if (!B.next.n) {
+        B.next.alloc(kP64Passes);
+        B.count.alloc(kP64Passes);
+    }
+    PDD_CUDA(cudaMemsetAsync(B.next.p, 0, kP64Passes * sizeof(unsigned long long), st));
+    PDD_CUDA(cudaMemsetAsync(B.count.p, 0, kP64Passes * sizeof(unsigned), st));
+    PDD_LAUNCH(k_slots64, cdiv(nrows, 128), 128, 0, st, nrows, A, B.slots.p);
+    size_t sm = 0;
+    if (P.c_kind == PDD_C_RBF)
+        sm = (2 * (size_t)kExpTab + (P.n_rbf <= kP64Staged ? 3 * (size_t)P.n_rbf : 0)) * sizeof(double);
+    PathPool Q{B.slots.p, nrows, (unsigned long long)total, nullptr, nullptr, nullptr, nullptr, nullptr, 0, nullptr,
+               nullptr, B.seg.p};
+    int grid = ctas;
+    for (int pass = 0; pass < kP64Passes; ++pass) {
+        const bool last = pass == kP64Passes - 1;
+        Q.next = B.next.p + pass;
+        Q.in = pass ? B.state[(pass - 1) & 1].p : nullptr;
+        Q.n_in = pass ? B.count.p + pass - 1 : nullptr;
+        Q.cq_in = B.cq[(pass + 1) & 1].p;
+        Q.out = B.state[pass & 1].p;
+        Q.cq_out = B.cq[pass & 1].p;
+        Q.n_out = B.count.p + pass;
+        Q.keep = last ? 0 : 16;
+        if (A.cvd > 0) launch_pass64<true>(P, A, Q, grid, sm, st);
+        else launch_pass64<false>(P, A, Q, grid, sm, st);
+        grid = std::max(1, (grid + 1) / 2);               // every warp hands over at most half its lanes
+    }
+    PDD_LAUNCH(k_exit64, cdiv(total, 256), 256, 0, st, P, A, Q);
 }
 
 McStats assemble_mc(const pdd_cover &cov, const Problem &P, const pdd_assembly_opts &o, pdd_system &sys,
@@ -1196,7 +1586,8 @@ McStats assemble_mc(const pdd_cover &cov, const Problem &P, const pdd_assembly_o
     const int mixed = path_mixed(o) ? 1 : 0;
     const int cvd = o.cv_degree, ncv = cvd * (cvd + 3) / 2;          // control-variate features per path
     const int cv_stride = cov.max_stencil + 1;
-    const size_t rec_bytes = 1 + 3 * sizeof(double) + (mixed ? sizeof(float2) : 0) + (size_t)ncv * sizeof(double);
+    const size_t rec_bytes =
+        1 + 3 * sizeof(double) + (mixed ? sizeof(float2) : sizeof(Seg64)) + (size_t)ncv * sizeof(double);
     const size_t per_row = (size_t)P_ * rec_bytes;
     const int wave = (int)std::max<size_t>(1, std::min<size_t>(nmc, ((size_t)8 << 30) / per_row));
     DevBuf<int8_t> side;
@@ -1230,15 +1621,16 @@ McStats assemble_mc(const pdd_cover &cov, const Problem &P, const pdd_assembly_o
     PDD_CUDA(cudaFuncSetAttribute(k_mc_finalize<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm));
     // per-slot arrays (subs, spos, kword, momp, bmean) are indexed like the global slot gs: offset to
     // the wave's first slot when gsl is null, or the whole arrays with gsl
-    auto run_wave = [&](const int *rows, int nr, const int *np, const long *roff, const int *gsl, const int *momp,
-                        double *bmean, size_t w0) {
+    Paths64Bufs p64;
+    auto run_wave = [&](const int *rows, int nr, long nrec, const int *np, const long *roff, const int *gsl,
+                        const int *momp, double *bmean, size_t w0) {
         const int *subs = sys.mc_subs.p + w0, *spos = sys.mc_spos.p + w0, *kword = sys.mc_kword.p + w0;
         PathArgs A{rows, subs, kword, cov.kx.p, cov.ky.p, cov.cx.p, cov.cy.p, cov.r.p,
                    cov.theta_s.p, o.paths, o.h, o.seed, side.p, su.p, Y.p, Z.p, steps.p, capped.p, np, roff, ez.p,
                    o.boundary_shift ? kGmC0 * sqrt(o.h) : 0.0, gsl, o.max_steps, cvd, ncv, cvq.p};
         PDD_CUDA(cudaEventRecord(e0, st));
-        if (mixed) launch_paths<float>(P, A, nr, st);
-        else launch_paths<double>(P, A, nr, st);
+        if (mixed) launch_paths(P, A, nr, st);
+        else run_paths64(P, A, nr, nrec, p64, st);
         PDD_CUDA(cudaEventRecord(e1, st));
         FinalArgs F{rows, subs, spos, cov.sub_off.p, cov.knot_ptr.p, cov.rowptr.p, cov.floating.p,
                     cov.ku.p, koff_m.p, kinv.p, kcond.p, o.imq_c2, o.paths, mcf, mixed, np, roff, gsl, side.p, su.p,
@@ -1265,7 +1657,7 @@ McStats assemble_mc(const pdd_cover &cov, const Problem &P, const pdd_assembly_o
     };
     for (int w0 = 0; w0 < nmc; w0 += wave) {
         const int nr = std::min(wave, nmc - w0);
-        run_wave(sys.mc_rows.p + w0, nr, nullptr, nullptr, nullptr, sys.mom_ptr.p + w0, sys.bmean.p + w0, w0);
+        run_wave(sys.mc_rows.p + w0, nr, (long)nr * P_, nullptr, nullptr, nullptr, sys.mom_ptr.p + w0, sys.bmean.p + w0, w0);
     }
     ms.paths_total = (int64_t)nmc * P_;
     sys.mc_np.alloc(nmc);
@@ -1322,7 +1714,7 @@ McStats assemble_mc(const pdd_cover &cov, const Problem &P, const pdd_assembly_o
                 if (mixed) ez.alloc(off);
                 if (ncv) cvq.alloc((size_t)off * ncv);
             }
-            run_wave(drows.p, (int)rows.size(), dnp.p, droff.p, dgsl.p, sys.mom_ptr.p, sys.bmean.p, 0);
+            run_wave(drows.p, (int)rows.size(), off, dnp.p, droff.p, dgsl.p, sys.mom_ptr.p, sys.bmean.p, 0);
         }
     }
     PDD_CUDA(cudaMemcpyAsync(sys.mc_np.p, need.data(), nmc * sizeof(int), cudaMemcpyHostToDevice, st));
