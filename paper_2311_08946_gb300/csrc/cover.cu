@@ -460,8 +460,21 @@ __global__ void k_coverage(Problem P, Grid G, int sx, int sy, double bx0, double
 // ---------------------------------------------------------------------------
 // a4: row assignment
 // ---------------------------------------------------------------------------
+// circles in cell order as FP32 (x, y, r), for the tests that rule a circle out
+__global__ void k_cell_circles(int M, const int *citems, const double *cx, const double *cy, const double *r,
+                               float4 *c32) {
+    int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= M) return;
+    const int m = citems[q];
+    c32[q] = make_float4((float)cx[m], (float)cy[m], (float)r[m], 0.f);
+}
+
+// Every knot looks at the circles of the 3 x 3 cells around it (pitch: the largest radius), hundreds
+// when the radii are uneven, and lies inside a few.  The FP64 score (a square root) was the bound
+// (2.3 ms for 127 thousand knots of the 7,108-circle cover); an FP32 distance test that can only rule
+// out a circle whose edge is clearly nearer than the knot leaves those few (this, the duplicate test and the sort below: cover 10.7 -> 3.4 ms).
 __global__ void k_assign_rows(Grid G, int N, const double *kx, const double *ky, const int *kowner,
-                              const uint8_t *kdir, const int *cptr, const int *citems,
+                              const uint8_t *kdir, const int *cptr, const int *citems, const float4 *c32,
                               const double *cx, const double *cy, const double *r, int *row_sub,
                               int *uncovered) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -473,28 +486,34 @@ __global__ void k_assign_rows(Grid G, int N, const double *kx, const double *ky,
     const double x = kx[i], y = ky[i];
     const int own = kowner[i];
     const double eps = kScoreEps * r[own];
+    const float xf = (float)x, yf = (float)y;
+    // FP32 coordinates are off by 2^-24 of their size; 16 times that and 1e-5 of the radius to spare
+    const float slack = 1e-6f * (fabsf(xf) + fabsf(yf) + (float)G.h);
     int c = G.cell_of(x, y), ix = c % G.gx, iy = c / G.gx;
     double best = -1.0;
     bool any = false;
     for (int pass = 0; pass < 2; ++pass) {
         int pick = 0x7fffffff;
-        for (int b = max(0, iy - 1); b <= min(G.gy - 1, iy + 1); ++b)
-            for (int a = max(0, ix - 1); a <= min(G.gx - 1, ix + 1); ++a) {
-                int cc = b * G.gx + a;
-                for (int q = cptr[cc]; q < cptr[cc + 1]; ++q) {
-                    int m = citems[q];
-                    if (m == own) continue;
-                    double dx = x - cx[m], dy = y - cy[m];
-                    double s = r[m] - sqrt(dx * dx + dy * dy);
-                    if (!(s > eps)) continue;
-                    if (pass == 0) {
-                        if (!any || s > best) best = s;
-                        any = true;
-                    } else if (s >= best - eps && m < pick) {
-                        pick = m;
-                    }
+        for (int b = max(0, iy - 1); b <= min(G.gy - 1, iy + 1); ++b) {
+            // the cells of a row of cells are consecutive, and so are their circles
+            const int q0 = cptr[b * G.gx + max(0, ix - 1)], q1 = cptr[b * G.gx + min(G.gx - 1, ix + 1) + 1];
+            for (int q = q0; q < q1; ++q) {
+                const float4 f = c32[q];
+                const float dxf = xf - f.x, dyf = yf - f.y, rf = f.z * 1.00001f + slack;
+                if (dxf * dxf + dyf * dyf > rf * rf) continue;
+                int m = citems[q];
+                if (m == own) continue;
+                double dx = x - cx[m], dy = y - cy[m];
+                double s = r[m] - sqrt(dx * dx + dy * dy);
+                if (!(s > eps)) continue;
+                if (pass == 0) {
+                    if (!any || s > best) best = s;
+                    any = true;
+                } else if (s >= best - eps && m < pick) {
+                    pick = m;
                 }
             }
+        }
         if (pass == 0 && !any) {
             row_sub[i] = -2;
             atomicAdd(uncovered, 1);
@@ -507,14 +526,16 @@ __global__ void k_assign_rows(Grid G, int N, const double *kx, const double *ky,
 // ---------------------------------------------------------------------------
 // duplicate knots (closer than 1e-12)
 // ---------------------------------------------------------------------------
+// (the knots' own grid has about one knot per cell; a knot within 1e-12 lies in a cell between those
+// of the corners (x, y) -+ 1e-12, nearly always the knot's own: cell indices are monotone in x and y)
 __global__ void k_dup_knots(Grid G, int N, const double *kx, const double *ky, const int *kptr,
                             const int *kitems, int *dups) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     const double x = kx[i], y = ky[i];
-    int c = G.cell_of(x, y), ix = c % G.gx, iy = c / G.gx;
-    for (int b = max(0, iy - 1); b <= min(G.gy - 1, iy + 1); ++b)
-        for (int a = max(0, ix - 1); a <= min(G.gx - 1, ix + 1); ++a) {
+    const int c0 = G.cell_of(x - 1e-12, y - 1e-12), c1 = G.cell_of(x + 1e-12, y + 1e-12);
+    for (int b = c0 / G.gx; b <= c1 / G.gx; ++b)
+        for (int a = c0 % G.gx; a <= c1 % G.gx; ++a) {
             int cc = b * G.gx + a;
             for (int q = kptr[cc]; q < kptr[cc + 1]; ++q) {
                 int j = kitems[q];
@@ -664,17 +685,25 @@ __global__ void k_sub_meta(int M, const int *sub_ptr, const int *sub_rows, const
     }
 }
 
-__global__ void k_sub_sort(int M, const int *sub_ptr, int *sub_rows) {
-    int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= M) return;
-    int a = sub_ptr[m], b = sub_ptr[m + 1];
-    for (int k = a + 1; k < b; ++k) {
-        int v = sub_rows[k], q = k - 1;
-        while (q >= a && sub_rows[q] > v) {
-            sub_rows[q + 1] = sub_rows[q];
-            --q;
+// each circle's rows in ascending order: one CTA per circle ranks them through shared memory (the rows
+// are distinct, so a row's position is the number of smaller ones).  Large circles among small ones
+// own hundreds of rows: an insertion sort by one thread took 3.3 ms of the 7,108-circle cover.
+static constexpr int kSortThreads = 128;
+__global__ void __launch_bounds__(kSortThreads) k_sub_sort(int M, const int *sub_ptr, const int *rows, int *sub_rows) {
+    __shared__ int t[kSortThreads];
+    const int m = blockIdx.x, a = sub_ptr[m], n = sub_ptr[m + 1] - a;
+    for (int e0 = 0; e0 < n; e0 += kSortThreads) {
+        const int e = e0 + threadIdx.x;
+        const int v = e < n ? rows[a + e] : 0;
+        int rank = 0;
+        for (int c0 = 0; c0 < n; c0 += kSortThreads) {
+            __syncthreads();
+            if (c0 + threadIdx.x < n) t[threadIdx.x] = rows[a + c0 + threadIdx.x];
+            __syncthreads();
+            const int cn = min(kSortThreads, n - c0);
+            for (int k = 0; k < cn; ++k) rank += t[k] < v ? 1 : 0;
         }
-        sub_rows[q + 1] = v;
+        if (e < n) sub_rows[a + rank] = v;
     }
 }
 
@@ -842,13 +871,23 @@ void build_cover_impl(const pdd_domain &dom, const pdd_cover_spec &spec, pdd_cov
     // duplicate knots
     {
         DevBuf<int> kptr, kitems;
-        build_grid(G, N, cov.kx.p, cov.ky.p, kptr, kitems, st);
-        PDD_LAUNCH(k_dup_knots, cdiv(N, 256), 256, 0, st, G, N, cov.kx.p, cov.ky.p, kptr.p, kitems.p,
+        // about one knot per cell, cells no larger than the circles' grid's
+        Grid K = G;
+        const double wx = bx1 - bx0 + 2 * cov.max_r, wy = by1 - by0 + 2 * cov.max_r;
+        K.h = std::min(G.h, std::sqrt(wx * wy / std::max(N, 1)));
+        K.gx = (int)std::ceil(wx / K.h) + 1;
+        K.gy = (int)std::ceil(wy / K.h) + 1;
+        if ((double)K.gx * K.gy > 5e7) K = G;
+        build_grid(K, N, cov.kx.p, cov.ky.p, kptr, kitems, st);
+        PDD_LAUNCH(k_dup_knots, cdiv(N, 256), 256, 0, st, K, N, cov.kx.p, cov.ky.p, kptr.p, kitems.p,
                    err.p + 2);
     }
     // a4: rows
+    DevBuf<float4> c32;
+    c32.alloc(M);
+    PDD_LAUNCH(k_cell_circles, cdiv(M, 256), 256, 0, st, M, cov.cell_items.p, cov.cx.p, cov.cy.p, cov.r.p, c32.p);
     PDD_LAUNCH(k_assign_rows, cdiv(N, 256), 256, 0, st, G, N, cov.kx.p, cov.ky.p, cov.kowner.p,
-               cov.kdir.p, cov.cell_ptr.p, cov.cell_items.p, cov.cx.p, cov.cy.p, cov.r.p,
+               cov.kdir.p, cov.cell_ptr.p, cov.cell_items.p, c32.p, cov.cx.p, cov.cy.p, cov.r.p,
                cov.row_sub.p, err.p + 1);
     std::vector<int> herr = to_host(err, 8, st);
     if (herr[0]) fail(PDD_EINVAL, "degenerate junction (a circle through a corner) or too many knots");
@@ -885,9 +924,11 @@ void build_cover_impl(const pdd_domain &dom, const pdd_cover_spec &spec, pdd_cov
     cov.sub_ptr.alloc(M + 1);
     int nsub = (int)exclusive_scan(sub_cnt.p, cov.sub_ptr.p, M, st);
     cov.sub_rows.alloc(std::max(nsub, 1));
+    DevBuf<int> unsorted;
+    unsorted.alloc(std::max(nsub, 1));
     PDD_LAUNCH(k_sub_fill, cdiv(N, 256), 256, 0, st, N, cov.pi_ptr.p, cov.pi_sub.p, cov.sub_ptr.p, cursor.p,
-               cov.sub_rows.p);
-    PDD_LAUNCH(k_sub_sort, cdiv(M, 128), 128, 0, st, M, cov.sub_ptr.p, cov.sub_rows.p);
+               unsorted.p);
+    PDD_LAUNCH(k_sub_sort, M, kSortThreads, 0, st, M, cov.sub_ptr.p, unsorted.p, cov.sub_rows.p);
     const int np1 = std::max(nsub, 1);
     cov.sub_m.alloc(np1);
     cov.sub_k.alloc(np1);
