@@ -4,6 +4,7 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <string>
 
 #include <vector>
@@ -22,6 +23,104 @@ std::string cuda_msg(cudaError_t e, const char *what) {
 }
 
 void count_launch(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
+
+// ---------------------------------------------------------------------------
+// the device memory pools
+// ---------------------------------------------------------------------------
+// What a pool keeps of the memory that is not in use: the working set of a repeated assembly while the
+// device has covers or systems (the 864 disks of the variable-coefficient workload take 9 GB), little when it has none.
+static constexpr unsigned long long kPoolKeep = 16ULL << 30, kPoolKeepIdle = 1ULL << 30;
+// Buffers that the pool could not keep anyway come from cudaMalloc: mapping and unmapping them in the
+// pool added 47 ms a call on the scaled workload (two buffers of 23 GB)
+static constexpr size_t kDirectBytes = (size_t)(kPoolKeep / 2);
+static constexpr int kPoolDevices = 64;
+static std::mutex g_pool_mu;
+static cudaMemPool_t g_pool[kPoolDevices] = {nullptr};
+static int g_live[kPoolDevices] = {0};
+static thread_local cudaStream_t g_call_stream = nullptr;
+
+CallStream::CallStream(cudaStream_t st) : prev(g_call_stream) { g_call_stream = st; }
+CallStream::~CallStream() { g_call_stream = prev; }
+
+static int current_device() {
+    int dev = 0;
+    PDD_CUDA(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= kPoolDevices) fail(PDD_EINVAL, "device ordinal out of range");
+    return dev;
+}
+
+static cudaMemPool_t pool_of(int dev) {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (!g_pool[dev]) {
+        cudaMemPoolProps pr{};
+        pr.allocType = cudaMemAllocationTypePinned;
+        pr.handleTypes = cudaMemHandleTypeNone;
+        pr.location.type = cudaMemLocationTypeDevice;
+        pr.location.id = dev;
+        PDD_CUDA(cudaMemPoolCreate(&g_pool[dev], &pr));
+        unsigned long long keep = g_live[dev] > 0 ? kPoolKeep : kPoolKeepIdle;
+        PDD_CUDA(cudaMemPoolSetAttribute(g_pool[dev], cudaMemPoolAttrReleaseThreshold, &keep));
+    }
+    return g_pool[dev];
+}
+
+void *pool_alloc(size_t bytes) {
+    void *p = nullptr;
+    if (bytes > kDirectBytes) {
+        PDD_CUDA(cudaMalloc(&p, bytes));
+        return p;
+    }
+    PDD_CUDA(cudaMallocFromPoolAsync(&p, bytes, pool_of(current_device()), g_call_stream));
+    return p;
+}
+
+void pool_free(void *p, size_t bytes) {
+    if (bytes > kDirectBytes) cudaFree(p);               // waits for the device
+    else cudaFreeAsync(p, g_call_stream);
+}
+
+size_t free_device_bytes() {
+    size_t freeb = 0, totb = 0;
+    PDD_CUDA(cudaMemGetInfo(&freeb, &totb));
+    cudaMemPool_t pool = pool_of(current_device());
+    unsigned long long held = 0, used = 0;
+    PDD_CUDA(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held));
+    PDD_CUDA(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used));
+    return freeb + (size_t)(held > used ? held - used : 0);
+}
+
+// the first handle of a device raises its pool's bound, the last one lowers it and gives the rest back
+static void count_handle(int dev, int d) {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    g_live[dev] += d;
+    if (!g_pool[dev] || !(d > 0 ? g_live[dev] == 1 : g_live[dev] == 0)) return;
+    unsigned long long keep = d > 0 ? kPoolKeep : kPoolKeepIdle;
+    cudaMemPoolSetAttribute(g_pool[dev], cudaMemPoolAttrReleaseThreshold, &keep);
+    if (d < 0) cudaMemPoolTrimTo(g_pool[dev], (size_t)keep);
+}
+
+// a handle's buffers may still be read on any stream (its accessors lend them): like cudaFree, wait for
+// the device, then return them in the order of the default stream
+template <typename H>
+static void destroy_handle(H *h) {
+    if (!h) return;
+    int prev = 0;
+    const bool moved = cudaGetDevice(&prev) == cudaSuccess && prev != h->live.dev;
+    if (moved) cudaSetDevice(h->live.dev);
+    cudaDeviceSynchronize();
+    {
+        CallStream scope(nullptr);
+        delete h;
+    }
+    if (moved) cudaSetDevice(prev);
+}
+
+}  // namespace pdd
+
+pdd_handle_count::pdd_handle_count() : dev(pdd::current_device()) { pdd::count_handle(dev, 1); }
+pdd_handle_count::~pdd_handle_count() { pdd::count_handle(dev, -1); }
+
+namespace pdd {
 
 void ProblemHolder::set(const pdd_domain &dom, const pdd_operator &op, cudaStream_t st) {
     P = Problem{};
@@ -205,7 +304,10 @@ static void check_opts(const pdd_assembly_opts *o) {
 
 using namespace pdd;
 
-#define API_BEGIN try {
+// entry points: allocations of the call belong to its stream; failures become statuses
+#define API_BEGIN(stream)                 \
+    try {                                 \
+        CallStream call_scope((cudaStream_t)(stream));
 #define API_END                                                        \
     }                                                                  \
     catch (const Fail &f) {                                            \
@@ -226,7 +328,7 @@ int64_t pdd_launch_count(void) { return (int64_t)g_launches.load(); }
 const char *pdd_version(void) { return "pdd-gb300 1.0 (sm_103a)"; }
 
 pdd_status pdd_build_cover(const pdd_domain *domain, const pdd_cover_spec *spec, pdd_cover **out, void *stream) {
-    API_BEGIN
+    API_BEGIN(stream)
     if (!out) fail(PDD_EINVAL, "null output handle");
     *out = nullptr;
     check_domain(domain);
@@ -244,7 +346,7 @@ pdd_status pdd_build_cover(const pdd_domain *domain, const pdd_cover_spec *spec,
 }
 
 pdd_status pdd_cover_info(const pdd_cover *cov, int *M, int *M_floating, int *N, int64_t *nnz) {
-    API_BEGIN
+    API_BEGIN(nullptr)
     if (!cov) fail(PDD_EINVAL, "null cover");
     if (M) *M = cov->M;
     if (M_floating) *M_floating = cov->M_floating;
@@ -257,7 +359,7 @@ pdd_status pdd_cover_arrays(const pdd_cover *cov, const double **cx, const doubl
                             const uint8_t **floating, const int **knot_ptr, const double **kx, const double **ky,
                             const double **ku, const int **kowner, const uint8_t **kdir, const int **row_sub,
                             const int **rowptr, const int **col) {
-    API_BEGIN
+    API_BEGIN(nullptr)
     if (!cov) fail(PDD_EINVAL, "null cover");
     if (cx) *cx = cov->cx.p;
     if (cy) *cy = cov->cy.p;
@@ -275,11 +377,11 @@ pdd_status pdd_cover_arrays(const pdd_cover *cov, const double **cx, const doubl
     API_END
 }
 
-void pdd_destroy_cover(pdd_cover *cov) { delete cov; }
+void pdd_destroy_cover(pdd_cover *cov) { destroy_handle(cov); }
 
 pdd_status pdd_assemble_G(const pdd_cover *cov, const pdd_operator *op, const pdd_assembly_opts *opts,
                           pdd_system **out, void *stream) {
-    API_BEGIN
+    API_BEGIN(stream)
     if (!out) fail(PDD_EINVAL, "null output handle");
     *out = nullptr;
     if (!cov) fail(PDD_EINVAL, "null cover");
@@ -371,7 +473,7 @@ pdd_status pdd_assemble_G(const pdd_cover *cov, const pdd_operator *op, const pd
 
 pdd_status pdd_system_csr(const pdd_system *sys, const double **val, const double **b, const double **se,
                           const double **se_b) {
-    API_BEGIN
+    API_BEGIN(nullptr)
     if (!sys) fail(PDD_EINVAL, "null system");
     if (val) *val = sys->val.p;
     if (b) *b = sys->b.p;
@@ -382,7 +484,7 @@ pdd_status pdd_system_csr(const pdd_system *sys, const double **val, const doubl
 
 pdd_status pdd_system_mc(const pdd_system *sys, int *n_rows, const int **rows, const int **mom_ptr,
                          const double **moments, const double **bmean) {
-    API_BEGIN
+    API_BEGIN(nullptr)
     if (!sys) fail(PDD_EINVAL, "null system");
     if (n_rows) *n_rows = sys->n_mc;
     if (rows) *rows = sys->mc_rows.p;
@@ -393,7 +495,7 @@ pdd_status pdd_system_mc(const pdd_system *sys, int *n_rows, const int **rows, c
 }
 
 pdd_status pdd_cover_rows(const pdd_cover *cov, int *n_pairs, const int **pi_ptr, const int **pi_sub) {
-    API_BEGIN
+    API_BEGIN(nullptr)
     if (!cov) fail(PDD_EINVAL, "null cover");
     if (n_pairs) *n_pairs = cov->npairs;
     if (pi_ptr) *pi_ptr = cov->pi_ptr.p;
@@ -402,20 +504,20 @@ pdd_status pdd_cover_rows(const pdd_cover *cov, int *n_pairs, const int **pi_ptr
 }
 
 pdd_status pdd_system_mc_subs(const pdd_system *sys, const int **subs) {
-    API_BEGIN
+    API_BEGIN(nullptr)
     if (!sys) fail(PDD_EINVAL, "null system");
     if (subs) *subs = sys->mc_subs.p;
     API_END
 }
 
 pdd_status pdd_system_stats(const pdd_system *sys, pdd_assembly_stats *stats) {
-    API_BEGIN
+    API_BEGIN(nullptr)
     if (!sys || !stats) fail(PDD_EINVAL, "null argument");
     *stats = sys->stats;
     API_END
 }
 
-void pdd_destroy_system(pdd_system *sys) { delete sys; }
+void pdd_destroy_system(pdd_system *sys) { destroy_handle(sys); }
 
 static void check_solve_opts(const pdd_solve_opts *o) {
     if (!o) fail(PDD_EINVAL, "null solve options");
@@ -426,7 +528,7 @@ static void check_solve_opts(const pdd_solve_opts *o) {
 
 pdd_status pdd_solve_csr(int n, const int *rowptr, const int *col, const double *val, const double *b, double *u,
                          const pdd_solve_opts *opts, pdd_solve_info *info, void *stream) {
-    API_BEGIN
+    API_BEGIN(stream)
     check_solve_opts(opts);
     if (opts->precond != PDD_PRECOND_NONE) fail(PDD_EINVAL, "the RAS preconditioner needs the cover: use pdd_solve");
     if (n <= 0 || !rowptr || !col || !val || !b || !u) fail(PDD_EINVAL, "null array or n <= 0");
@@ -462,7 +564,7 @@ pdd_status pdd_solve(const pdd_system *sys, const pdd_solve_opts *opts, double *
     }
     if (!opts || opts->precond == PDD_PRECOND_NONE)
         return pdd_solve_csr(sys->N, sys->cov->rowptr.p, sys->cov->col.p, sys->val.p, sys->b.p, u, opts, info, stream);
-    API_BEGIN
+    API_BEGIN(stream)
     check_solve_opts(opts);
     if (opts->transpose) fail(PDD_EINVAL, "the preconditioned solve takes C itself (transpose = 0)");
     if (!u) fail(PDD_EINVAL, "null u");
@@ -481,7 +583,7 @@ pdd_status pdd_solve(const pdd_system *sys, const pdd_solve_opts *opts, double *
 }
 
 pdd_status pdd_ras_apply(const pdd_system *sys, const double *v, double *y, void *stream) {
-    API_BEGIN
+    API_BEGIN(stream)
     if (!sys || !v || !y) fail(PDD_EINVAL, "null argument");
     if (sys->cov->averaged) fail(PDD_EINVAL, "the RAS subsets need one subdomain per row (a farthest-interface cover)");
     cudaStream_t st = (cudaStream_t)stream;
@@ -494,7 +596,7 @@ pdd_status pdd_ras_apply(const pdd_system *sys, const double *v, double *y, void
 
 pdd_status pdd_spmv_csr(int n, const int *rowptr, const int *col, const double *val, const double *x, double *y,
                         int transpose, void *stream) {
-    API_BEGIN
+    API_BEGIN(stream)
     if (n <= 0 || !rowptr || !col || !val || !x || !y) fail(PDD_EINVAL, "null array or n <= 0");
     cudaStream_t st = (cudaStream_t)stream;
     if (transpose) {
@@ -515,7 +617,7 @@ pdd_status pdd_spmv_csr(int n, const int *rowptr, const int *col, const double *
 pdd_status pdd_grad(const pdd_cover *cov, const pdd_operator *op, const pdd_assembly_opts *opts,
                     const pdd_system *sys, const double *u, const double *dJdu, double *grad, double *lambda,
                     void *stream) {
-    API_BEGIN
+    API_BEGIN(stream)
     if (!cov || !sys || !u || !dJdu || !grad) fail(PDD_EINVAL, "null argument");
     if (sys->cov != cov) fail(PDD_EINVAL, "system was not assembled on this cover");
     if (cov->averaged) fail(PDD_EINVAL, "the adjoint gradient needs one subdomain per row (a farthest-interface cover)");

@@ -47,7 +47,25 @@ inline void fail(pdd_status st, const std::string &msg) {
     throw Fail{st};
 }
 
-// device buffer owned by a handle
+// Device memory of the library: one stream-ordered pool per device (api.cu).  cudaMalloc and cudaFree
+// cost 10-40 us each (a free also waits for the device) and a call makes 15 to 190 of them, more than
+// the kernels of a small call; from the pool an allocation takes about 1 us.  A buffer belongs to the
+// stream of the entry point that allocates it (CallStream) and goes back to the pool in that stream's
+// order, so a later allocation on any stream, of any thread, waits for its last use.
+void *pool_alloc(size_t bytes);
+void pool_free(void *p, size_t bytes);
+size_t free_device_bytes();                 // free memory, what the pool holds unused included
+
+// the calling thread's stream for allocations, for the duration of an entry point
+struct CallStream {
+    cudaStream_t prev;
+    explicit CallStream(cudaStream_t st);
+    ~CallStream();
+    CallStream(const CallStream &) = delete;
+    CallStream &operator=(const CallStream &) = delete;
+};
+
+// device buffer
 template <typename T>
 struct DevBuf {
     T *p = nullptr;
@@ -55,11 +73,11 @@ struct DevBuf {
     void alloc(size_t count) {
         release();
         if (count == 0) return;
-        PDD_CUDA(cudaMalloc((void **)&p, count * sizeof(T)));
+        p = static_cast<T *>(pool_alloc(count * sizeof(T)));
         n = count;
     }
     void release() {
-        if (p) cudaFree(p);
+        if (p) pool_free(p, n * sizeof(T));
         p = nullptr;
         n = 0;
     }

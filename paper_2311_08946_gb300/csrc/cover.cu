@@ -118,13 +118,12 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(const int *in, int 
 // the total also goes to *total_dev when given
 void exclusive_scan_async(const int *in, int *out, int n, cudaStream_t st, long long *total_dev) {
     const int ntiles = std::max(1, cdiv(n, kScanTile));
-    long long *ts = nullptr;                     // stream-ordered: freed after the launches that read it
-    PDD_CUDA(cudaMallocAsync((void **)&ts, sizeof(long long) * ntiles, st));
-    if (n > 0) PDD_LAUNCH(k_scan_reduce, ntiles, kScanThreads, 0, st, in, n, ts);
-    else PDD_CUDA(cudaMemsetAsync(ts, 0, sizeof(long long), st));
-    PDD_LAUNCH(k_scan_tiles, 1, kScanThreads, 0, st, ts, ntiles, out + n, total_dev);
-    if (n > 0) PDD_LAUNCH(k_scan_apply, ntiles, kScanThreads, 0, st, in, out, n, ts);
-    PDD_CUDA(cudaFreeAsync(ts, st));
+    DevBuf<long long> ts;                        // freed in stream order, after the launches that read it
+    ts.alloc(ntiles);
+    if (n > 0) PDD_LAUNCH(k_scan_reduce, ntiles, kScanThreads, 0, st, in, n, ts.p);
+    else PDD_CUDA(cudaMemsetAsync(ts.p, 0, sizeof(long long), st));
+    PDD_LAUNCH(k_scan_tiles, 1, kScanThreads, 0, st, ts.p, ntiles, out + n, total_dev);
+    if (n > 0) PDD_LAUNCH(k_scan_apply, ntiles, kScanThreads, 0, st, in, out, n, ts.p);
 }
 
 int64_t exclusive_scan(const int *in, int *out, int n, cudaStream_t st) {

@@ -1521,8 +1521,7 @@ static DiskStats run_group(const pdd_cover &cov, const Problem &P, const pdd_ass
     const size_t perNp = use_np ? (size_t)lu_np_inv_floats(S.n) * sizeof(float) : 0;
     const size_t perDisk = perA + perR * (mixed ? 3 : 1) + (size_t)S.n * S.nrhs * sizeof(T) +
                            (size_t)S.n * sizeof(NodeCoef) + (size_t)S.n * sizeof(int) + perDinv + perNp + 64;
-    size_t freeb = 0, totb = 0;
-    PDD_CUDA(cudaMemGetInfo(&freeb, &totb));
+    const size_t freeb = free_device_bytes();
     size_t budget = std::min<size_t>((size_t)(0.6 * freeb), (size_t)64 << 30);
     if (use_np) {           // the GEMM tile scratch comes out of the same budget
         const size_t scr = lu_np_scratch_floats_per_disk(S.n) * sizeof(float) *
@@ -1649,7 +1648,7 @@ static DiskStats run_group(const pdd_cover &cov, const Problem &P, const pdd_ass
             const long items = (long)nd * nblk * 2;
             PDD_LAUNCH(k_diag_inv, (int)((items + 3) / 4), 128, 0, st, reinterpret_cast<const float *>(A.p), S.n, sA,
                        nd, dinv.p);
-            if ((S.n & 3) == 0)       // rows and disks start on 16-byte boundaries (cudaMalloc'd buffers)
+            if ((S.n & 3) == 0)       // rows and disks start on 16-byte boundaries (pool buffers)
                 PDD_LAUNCH(k_transpose_f32_v4, dim3(cdiv(S.n, 64), cdiv(S.n, 64), nd), 256, 0, st,
                            reinterpret_cast<const float *>(A.p), AT.p, S.n, sA);
             else
@@ -2011,8 +2010,7 @@ void grad_disks(const pdd_cover &cov, const Problem &P, const double *u, const d
         const auto &disks = kv.second;
         const size_t perDisk = (size_t)S.n * S.n * 8 + (size_t)S.n * S.nrhs * 8 * 3 + (size_t)S.n * 8 * 4 +
                                (size_t)S.n * sizeof(NodeCoef) + (size_t)S.n * 4 + 64;
-        size_t freeb = 0, totb = 0;
-        PDD_CUDA(cudaMemGetInfo(&freeb, &totb));
+        const size_t freeb = free_device_bytes();
         int wave = (int)std::max<size_t>(1, std::min<size_t>((size_t)(0.5 * freeb), (size_t)32 << 30) / perDisk);
         wave = std::min<int>(wave, (int)disks.size());
         DevBuf<double> A, W, RHS, X, Vb, Eb, Zb, Wt;

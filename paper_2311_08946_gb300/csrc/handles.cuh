@@ -6,7 +6,15 @@
 
 #include "common.cuh"
 
+// counts the live handles of a device, for the pool's bound (api.cu)
+struct pdd_handle_count {
+    int dev;
+    pdd_handle_count();
+    ~pdd_handle_count();
+};
+
 struct pdd_cover {
+    pdd_handle_count live;                 // first member: destroyed after the buffers
     pdd_domain domain;
     int M = 0, M_floating = 0, N = 0;
     int64_t nnz = 0;
@@ -41,6 +49,7 @@ struct pdd_cover {
 };
 
 struct pdd_system {
+    pdd_handle_count live;
     int N = 0;
     int64_t nnz = 0;
     const pdd_cover *cov = nullptr;

@@ -1314,6 +1314,7 @@ extern "C" pdd_status pdd_batched_gemm_sub_tf32x3(int batch, int M, int N, int K
             fail(PDD_EINVAL, "negative size or null operand");
         if (lda < K || ldb < N || ldc < N) fail(PDD_EINVAL, "leading dimension smaller than the row length");
         cudaStream_t st = (cudaStream_t)stream;
+        CallStream scope(st);
         DevBuf<int> err;
         err.alloc(1);
         PDD_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), st));
@@ -1339,6 +1340,7 @@ extern "C" pdd_status pdd_batched_gemm_tf32x3(int batch, int M, int N, int K, co
         if (lda < K || ldb < N || ldc < N) fail(PDD_EINVAL, "leading dimension smaller than the row length");
         if (batch == 0 || M == 0 || N == 0 || K == 0) return PDD_OK;
         cudaStream_t st = (cudaStream_t)stream;
+        CallStream scope(st);
         DevBuf<int> err;
         err.alloc(1);
         PDD_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), st));
