@@ -6,7 +6,8 @@
 // contiguous); dot products are block partial sums reduced in a fixed order
 // (deterministic).  Orthogonalisation is classical Gram-Schmidt applied
 // twice (CGS2).  The m Arnoldi iterations of a restart cycle run in one
-// cooperative kernel (k_arnoldi_fused); the Hessenberg matrix, Givens
+// cooperative kernel of clusters (k_arnoldi_fused) that keeps each CTA's part
+// of the basis in shared memory; the Hessenberg matrix, Givens
 // rotations and the residual estimate live on the device, and the host
 // synchronises once per restart cycle to read the true residual.
 #include <cstdlib>
@@ -24,14 +25,14 @@ static constexpr int kRowsPerBlock = 32;    // 8 lanes per row, 256 threads
 static constexpr int kDotBlock = 256;
 
 struct GState {
-    int stop, iters, k_used, pad;
+    int stop, iters, k_used, err;
     double bnorm, res;
+    double rr;                  // |b - C u|^2 of the cycle's end
 };
 
-// y = C x, 8 lanes per row
+// y = C x, or y = b - C x with b given; 8 lanes per row
 __global__ void __launch_bounds__(256) k_spmv(int n, const int *rowptr, const int *col, const double *val,
-                                              const double *x, double *y, const GState *gs) {
-    if (gs && gs->stop) return;
+                                              const double *x, double *y, const double *b) {
     const int row = blockIdx.x * kRowsPerBlock + (threadIdx.x >> 3), l = threadIdx.x & 7;
     double s = 0.0;
     if (row < n)
@@ -39,7 +40,7 @@ __global__ void __launch_bounds__(256) k_spmv(int n, const int *rowptr, const in
     s += __shfl_xor_sync(0xffffffffu, s, 4);
     s += __shfl_xor_sync(0xffffffffu, s, 2);
     s += __shfl_xor_sync(0xffffffffu, s, 1);
-    if (row < n && l == 0) y[row] = s;
+    if (row < n && l == 0) y[row] = b ? b[row] - s : s;
 }
 
 // partial[t * G + bx] = sum over the rows of block column bx of V[t] . w.  The grid is
@@ -107,13 +108,42 @@ __global__ void __launch_bounds__(kDotBlock) k_normalize(int n, const double *w,
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) v[r] = w[r] * inv;
 }
 
-// y = H^-1 g (upper triangular k x k), single thread; then stop is cleared for the next cycle
-__global__ void k_upper_solve(const double *H, int ldh, const double *g, double *y, GState *gs) {
-    const int k = gs->k_used;
-    for (int i = k - 1; i >= 0; --i) {
-        double s = g[i];
-        for (int c = i + 1; c < k; ++c) s -= H[(long)c * ldh + i] * y[c];
-        y[i] = s / H[(long)i * ldh + i];
+// y = H^-1 g (upper triangular k x k), column by column: one warp holds the right-hand side, 32 columns
+// of H at a time staged in shared memory.  One thread walking rows of H in global memory took 45-100 us
+// a cycle (13-25 us).
+static constexpr int kUpperThreads = 256, kUpperCols = 32;
+static constexpr int kUpperSlices = (kMaxDots - 1 + 31) / 32;
+__global__ void __launch_bounds__(kUpperThreads) k_upper_solve(const double *H, int ldh, const double *g, double *y,
+                                                               const GState *gs) {
+    extern __shared__ double hs[];                        // [kUpperCols][k]
+    const int k = gs->k_used, lane = threadIdx.x & 31;
+    double s[kUpperSlices];
+#pragma unroll
+    for (int q = 0; q < kUpperSlices; ++q) s[q] = (lane + 32 * q < k) ? g[lane + 32 * q] : 0.0;
+    for (int c0 = ((k - 1) / kUpperCols) * kUpperCols; k > 0 && c0 >= 0; c0 -= kUpperCols) {
+        const int nc = min(kUpperCols, k - c0);
+        __syncthreads();
+        for (int e = threadIdx.x; e < nc * k; e += kUpperThreads) {
+            const int c = e / k, r = e - c * k;
+            if (r <= c0 + c) hs[e] = H[(long)(c0 + c) * ldh + r];
+        }
+        __syncthreads();
+        if (threadIdx.x >= 32) continue;
+        const double inv = lane < nc ? 1.0 / hs[lane * k + c0 + lane] : 0.0;      // of the tile's diagonal
+        const int qc = c0 >> 5;                                                   // c0 is a multiple of 32
+        for (int c = nc - 1; c >= 0; --c) {
+            double sq = 0.0;
+#pragma unroll
+            for (int q = 0; q < kUpperSlices; ++q)
+                if (q == qc) sq = s[q];
+            const double v = __shfl_sync(0xffffffffu, sq * inv, c);
+            if (lane == 0) y[c0 + c] = v;
+#pragma unroll
+            for (int q = 0; q < kUpperSlices; ++q) {
+                const int r = lane + 32 * q;
+                if (r < c0 + c) s[q] -= hs[c * k + r] * v;
+            }
+        }
     }
 }
 
@@ -124,11 +154,6 @@ __global__ void k_xupdate(int n, const double *V, const double *y, const GState 
         for (int t = 0; t < k; ++t) s += V[(long)t * n + r] * y[t];
         x[r] = s;
     }
-}
-
-// r = b - C x (Cx precomputed in r)
-__global__ void k_residual_vec(int n, const double *b, double *r) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) r[i] = b[i] - r[i];
 }
 
 __global__ void k_cycle_start(GState *gs, const double *hsum, double *g, int m, double rtol, int max_iters,
@@ -145,34 +170,42 @@ __global__ void k_cycle_start(GState *gs, const double *hsum, double *g, int m, 
 
 void spmv_csr(int n, const int *rowptr, const int *col, const double *val, const double *x, double *y,
               cudaStream_t st) {
-    PDD_LAUNCH(k_spmv, cdiv(n, kRowsPerBlock), 256, 0, st, n, rowptr, col, val, x, y, (const GState *)nullptr);
+    PDD_LAUNCH(k_spmv, cdiv(n, kRowsPerBlock), 256, 0, st, n, rowptr, col, val, x, y, (const double *)nullptr);
 }
 
 // ---------------------------------------------------------------------------
-// One restart cycle's Arnoldi iterations in a single cooperative launch.
-// Block b owns rows [b per, (b+1) per): it computes w = C v_j on them, their
-// partial dot products with the basis, their part of the CGS2 updates and of
-// |w|; partial sums meet in global memory and are added in block order after
-// a grid barrier (deterministic).  Block 0 keeps the Hessenberg column, the
-// Givens rotations and g in shared memory and writes the stop flag that every
-// block reads after the iteration's last barrier.  Four grid barriers per
-// iteration; each is a bounded spin that records an error and returns.
+// One restart cycle's Arnoldi iterations in a single cooperative launch of clusters of eight CTAs.
+// Each CTA owns `per` rows: it computes w = C v_j on them, keeps w and (as far as shared memory goes:
+// 64 vectors of 400 rows) its part of the basis in shared memory, and takes part in two passes of
+// classical Gram-Schmidt.  Dot products are added over a CTA's warps, then over the cluster through
+// distributed shared memory, then over the clusters through global memory, always in the same order
+// (deterministic).  |w| after the second pass comes from that pass: |w1|^2 - |h2|^2, w1 being almost
+// orthogonal already (else it is summed again).  Every CTA keeps the rotations and decides on stopping
+// by itself from the same sums, so an iteration has three grid-wide barriers.
+// Why: four barriers, basis slices read from L2 by latency-bound loops, 152 partial sums per vector
+// read by every CTA and a serial rotation on the critical path cost 22 us an iteration at n = 204 and
+// 52 us at n = 32,768; what is left is the FP64 pipe (4 n j products an iteration) and the barriers: 13 and 37 us.
+// With RAS (Eq. 44-45) z_j = M^-1 v_j comes first (two more barriers), one warp per subset.
 // ---------------------------------------------------------------------------
-static constexpr int kFusedThreads = 512;
+static constexpr int kFusedThreads = 512, kFusedWarps = kFusedThreads / 32;
+static constexpr int kClusterMax = 8;
+static constexpr int kRowsPerCta = 64;                  // fewer clusters than the device holds below this
+static constexpr size_t kFusedSmem = 222 * 1024;
 static constexpr long long kBarrierLimit = 1LL << 22;   // polls (an L2 read each, ~0.2 us) before giving up
 
 struct FusedArnoldi {
     int n, m;
     const int *rowptr, *col;
     const double *val;
-    double *V, *w, *part;        // part: 3 x kMaxDots x gridDim.x partial sums
-    double *H, *cs, *sn, *g;     // H column-major (ldh = m + 1)
+    double *V, *part;            // part: 3 x kMaxDots x clusters partial sums
+    double *w;                   // w in global memory when a CTA's rows do not fit in shared memory, else null
+    double *H, *g;               // H column-major (ldh = m + 1)
     GState *gs;
     unsigned *bar;               // [0] arrivals, [1] generation
-    int *err;
     double rtol;
     int max_iters;
-    unsigned bar_extra;          // arrivals a barrier waits for beyond the grid (0; 1 = never completes)
+    int per, ld, ks;             // rows of a CTA, their padded count, basis vectors kept in shared memory
+    unsigned bar_extra;          // arrivals a barrier waits for beyond the clusters (0; 1 = never completes)
     long long bar_limit;         // polls before a barrier wait gives up
     // right preconditioner (Eq. 44-45); ras_P = 0: none
     int ras_P, ras_NP;
@@ -182,17 +215,65 @@ struct FusedArnoldi {
     double *ras_Z;               // z_j = M^-1 v_j of the cycle, m x n (flexible GMRES)
 };
 
-// The block's writes are ordered before thread 0's device-scope fence by the block barrier
-// (the same pattern as a cooperative-groups grid sync), so only thread 0 fences; the waiters
-// poll the generation word without sleeping.
-__device__ __forceinline__ bool grid_barrier(const FusedArnoldi &F) {
-    __shared__ int s_bad;
-    __syncthreads();
-    if (threadIdx.x == 0) {
+// doubles of shared memory besides the basis: w, h, column, rotations, g, sums of the warps' row
+// chunks and of the CTA (twice), the update's parts; the RAS right-hand sides share the latter two
+__host__ __device__ constexpr size_t fused_fixed_doubles(int m, int ld) {
+    return (size_t)ld + 5 * (size_t)(m + 2) + (size_t)kFusedWarps * 8 + (size_t)kFusedWarps * 8 + 2 * (size_t)(m + 2) +
+           kFusedThreads + kFusedWarps * 64;
+}
+
+__device__ __forceinline__ unsigned cluster_rank() {
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ unsigned cluster_size() {
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_arrive() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// the double at p of this CTA's shared memory, in CTA `rank` of the cluster
+__device__ __forceinline__ double remote_load(const double *p, unsigned rank) {
+    uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+    double v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(r));
+    return v;
+}
+__device__ __forceinline__ int remote_load(const int *p, unsigned rank) {
+    uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+    int v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(r) : "memory");
+    return v;
+}
+
+// Grid-wide barrier, bounded.  The first cluster barrier orders the cluster's writes before thread 0
+// of its first CTA, which alone arrives and polls (and gives up after bar_limit polls); the second one
+// releases the cluster, all of whose CTAs read the outcome from the first, so they leave together (after
+// one more cluster barrier: the first CTA's shared memory must outlive the others' reads).
+// `meanwhile` runs between the arrival and the wait (one warp's scalar work).
+template <typename Work>
+__device__ __forceinline__ bool grid_barrier(const FusedArnoldi &F, unsigned nclusters, unsigned rank, int *s_bad,
+                                             Work meanwhile) {
+    cluster_arrive();
+    meanwhile();
+    cluster_wait();
+    if (nclusters == 1 && F.bar_extra == 0) return true;
+    if (rank == 0 && threadIdx.x == 0) {
         volatile unsigned *gen = F.bar + 1;
         const unsigned g0 = *gen;
         __threadfence();
-        if (atomicAdd(F.bar, 1u) == gridDim.x - 1 + F.bar_extra) {
+        if (atomicAdd(F.bar, 1u) == nclusters - 1 + F.bar_extra) {
             atomicExch(F.bar, 0u);
             __threadfence();
             atomicAdd(F.bar + 1, 1u);
@@ -200,16 +281,19 @@ __device__ __forceinline__ bool grid_barrier(const FusedArnoldi &F) {
             long long it = 0;
             while (*gen == g0) {
                 if (++it > F.bar_limit) {
-                    atomicExch(F.err, 1);
+                    atomicExch(&F.gs->err, 1);
                     break;
                 }
             }
         }
         __threadfence();
-        s_bad = *(volatile int *)F.err;
+        *s_bad = *(volatile int *)&F.gs->err;
     }
-    __syncthreads();
-    return s_bad == 0;
+    cluster_barrier();
+    return remote_load(s_bad, 0) == 0;
+}
+__device__ __forceinline__ bool grid_barrier(const FusedArnoldi &F, unsigned nclusters, unsigned rank, int *s_bad) {
+    return grid_barrier(F, nclusters, rank, s_bad, [] {});
 }
 
 __device__ __forceinline__ double warp_sum(double s) {
@@ -217,227 +301,473 @@ __device__ __forceinline__ double warp_sum(double s) {
     return s;
 }
 
-__global__ void __launch_bounds__(kFusedThreads) k_arnoldi_fused(FusedArnoldi F) {
-    constexpr int NW = kFusedThreads / 32;
-    __shared__ double h[kMaxDots], hcol[kMaxDots + 1], cs[kMaxDots], sn[kMaxDots], gv[kMaxDots + 1];
-    __shared__ double red[NW];
-    __shared__ float vs[4 * 128];
-    __shared__ int s_stop;
-    const int G = gridDim.x, b = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int n = F.n, m = F.m, ldh = m + 1;
-    const int per = (n + G - 1) / G, r0 = min(n, b * per), r1 = min(n, r0 + per);
-    if (b == 0)
-        for (int i = tid; i <= m; i += kFusedThreads) gv[i] = F.g[i];
-    for (int j = 0; j < m; ++j) {
-        if (tid == 0) s_stop = __ldcg(&F.gs->stop);
+// z_p = C_p^-1 (R_p v) of one subset by one warp: lane owns rows lane + 32 i (i < RR)
+template <int RR>
+__device__ __forceinline__ void ras_subset(const FusedArnoldi &F, int p, const double *vj, float *vs, int lane) {
+    const int NP = F.ras_NP, wb = F.ras_wptr[p], np = F.ras_wptr[p + 1] - wb;
+    for (int q = lane; q < NP; q += 32) vs[q] = q < np ? (float)__ldcg(vj + F.ras_widx[wb + q]) : 0.f;
+    __syncwarp();
+    const float *ci = F.ras_cinvT + (long)p * NP * NP + lane;
+    float s[RR];
+#pragma unroll
+    for (int i = 0; i < RR; ++i) s[i] = 0.f;
+    for (int q0 = 0; q0 < np; q0 += 16) {
+        float c[16][RR];
+#pragma unroll
+        for (int u = 0; u < 16; ++u)
+#pragma unroll
+            for (int i = 0; i < RR; ++i)
+                c[u][i] = (q0 + u < np && lane + 32 * i < NP) ? ci[(long)(q0 + u) * NP + 32 * i] : 0.f;
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+            const float v = vs[q0 + u < 128 ? q0 + u : 0];
+#pragma unroll
+            for (int i = 0; i < RR; ++i) s[i] = fmaf(c[u][i], v, s[i]);
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < RR; ++i)
+        if (lane + 32 * i < NP) F.ras_z[(long)p * NP + lane + 32 * i] = s[i];
+}
+
+extern __shared__ __align__(16) double asm_[];            // the basis [ks][ld], w [ld], the small arrays
+
+// loc[t] = sum over the CTA's rows of V_t . w for t <= j, loc[j + 1] = w . w when `norm` (j = -1 with
+// norm: w . w alone in loc[0]).  Warps take units of eight vectors x a chunk of rows; in a warp, eight
+// lanes name the vector and four row phases (the padded row count keeps them on different banks).
+// SM: every vector is in shared memory (addressed as such; the general form loads through generic
+// pointers).
+template <bool SM>
+__device__ __forceinline__ void local_dots_t(const FusedArnoldi &F, const double *ws, int rows, int r0, int j, bool norm,
+                                             double *chunk, double *loc, int warp, int lane) {
+    const int nv = j + 1 + (norm ? 1 : 0), ng = (nv + 7) >> 3;
+    const int C = max(1, kFusedWarps / ng), rc = (rows + C - 1) / C, wo = F.ks * F.ld;
+    for (int u = warp; u < ng * C; u += kFusedWarps) {
+        const int g = u / C, c = u - g * C, t = 8 * g + (lane & 7);
+        const int ra = c * rc + (lane >> 3), rb = min(rows, (c + 1) * rc);
+        double s0 = 0.0, s1 = 0.0;
+        if (SM) {
+            const int vo = t > j ? wo : t * F.ld;
+            if (t < nv) {
+                int r = ra;
+                for (; r + 4 < rb; r += 8) {
+                    s0 += asm_[vo + r] * asm_[wo + r];
+                    s1 += asm_[vo + r + 4] * asm_[wo + r + 4];
+                }
+                if (r < rb) s0 += asm_[vo + r] * asm_[wo + r];
+            }
+        } else {
+            const double *v = t > j ? ws : (t < F.ks ? asm_ + (size_t)t * F.ld : F.V + (long)t * F.n + r0);
+            if (t < nv) {
+                int r = ra;
+                for (; r + 4 < rb; r += 8) {
+                    s0 += v[r] * ws[r];
+                    s1 += v[r + 4] * ws[r + 4];
+                }
+                if (r < rb) s0 += v[r] * ws[r];
+            }
+        }
+        s0 += s1;
+        s0 += __shfl_xor_sync(0xffffffffu, s0, 8);
+        s0 += __shfl_xor_sync(0xffffffffu, s0, 16);
+        if (lane < 8) {
+            if (C > 1) chunk[u * 8 + lane] = s0;
+            else if (t < nv) loc[t] = s0;
+        }
+    }
+    __syncthreads();
+    if (C > 1) {
+        for (int t = threadIdx.x; t < nv; t += kFusedThreads) {
+            double a = 0.0, b = 0.0;                     // two chains over the chunks
+            for (int c = 0; c < C; c += 2) {
+                a += chunk[((t >> 3) * C + c) * 8 + (t & 7)];
+                if (c + 1 < C) b += chunk[((t >> 3) * C + c + 1) * 8 + (t & 7)];
+            }
+            loc[t] = a + b;
+        }
         __syncthreads();
-        if (s_stop) break;
-        // w = C v_j on this block's rows, 8 lanes per row; v_j was written by every block
+    }
+}
+__device__ __forceinline__ void local_dots(const FusedArnoldi &F, const double *ws, int rows, int r0, int j, bool norm,
+                                           double *chunk, double *loc, int warp, int lane) {
+    if (j < F.ks && F.ks > 0) local_dots_t<true>(F, ws, rows, r0, j, norm, chunk, loc, warp, lane);
+    else local_dots_t<false>(F, ws, rows, r0, j, norm, chunk, loc, warp, lane);
+}
+
+// the sum over the cluster's CTAs of loc[t]
+__device__ __forceinline__ double cluster_sum(const double *loc, int t, unsigned csize) {
+    double v[kClusterMax];
+#pragma unroll
+    for (unsigned q = 0; q < kClusterMax; ++q) v[q] = q < csize ? remote_load(loc + t, q) : 0.0;
+    return ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+}
+
+// out[t] = the sums of every CTA's loc[t], t < nv; `pp` this reduction's partial sums in global memory
+__device__ __forceinline__ bool grid_sum(const FusedArnoldi &F, int nv, const double *loc, double *pp, double *out,
+                                         unsigned ncl, unsigned cid, unsigned rank, unsigned csize, int *s_bad) {
+    const int tid = threadIdx.x;
+    cluster_barrier();                                   // every CTA of the cluster has its loc
+    if (ncl == 1) {
+        for (int t = tid; t < nv; t += kFusedThreads) out[t] = cluster_sum(loc, t, csize);
+        __syncthreads();
+        return F.bar_extra ? grid_barrier(F, ncl, rank, s_bad) : true;
+    }
+    for (int t = rank + tid * csize; t < nv; t += kFusedThreads * csize) pp[(long)t * ncl + cid] = cluster_sum(loc, t, csize);
+    if (!grid_barrier(F, ncl, rank, s_bad)) return false;
+    // eight lanes per sum
+    for (int t0 = 0; t0 < nv; t0 += kFusedThreads / 8) {
+        const int t = t0 + (tid >> 3);
+        if (t0 + ((tid & ~31) >> 3) >= nv) break;        // none of the warp's four sums
+        double s = 0.0;
+        if (t < nv)
+            for (unsigned c = tid & 7; c < ncl; c += 8) s += __ldcg(pp + (long)t * ncl + c);
+        s += __shfl_xor_sync(0xffffffffu, s, 4);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        if (t < nv && (tid & 7) == 0) out[t] = s;
+    }
+    __syncthreads();
+    return true;
+}
+
+// w - sum_{t <= j} h_t V_t on the CTA's rows, each handed to put(row, value); the vectors of a row are
+// spread over the warps when the rows are few.  `before` runs in the last warp first (scalar FP64 work
+// in the other warps' shadow); a block barrier orders it before the put calls.
+template <bool SM, typename Put, typename Work>
+__device__ __forceinline__ void subtract_basis_t(const FusedArnoldi &F, const double *ws, int rows, int r0, int j,
+                                                 const double *h, double *parts, Work before, Put put) {
+    const int rw = max(1, (rows + 31) >> 5), np = max(1, kFusedWarps / rw), width = rw * 32;
+    auto vec = [&](int t, int r) -> double {
+        if (SM) return asm_[t * F.ld + r];
+        return t < F.ks ? asm_[(size_t)t * F.ld + r] : F.V[(long)t * F.n + r0 + r];
+    };
+    if (threadIdx.x >= kFusedThreads - 32) before();
+    if (np == 1) {
+        __syncthreads();
+        for (int r = threadIdx.x; r < rows; r += kFusedThreads) {
+            double a0 = 0.0, a1 = 0.0;
+            int t = 0;
+            for (; t + 1 <= j; t += 2) {
+                a0 += vec(t, r) * h[t];
+                a1 += vec(t + 1, r) * h[t + 1];
+            }
+            if (t <= j) a0 += vec(t, r) * h[t];
+            put(r, ws[r] - (a0 + a1));
+        }
+        __syncthreads();
+        return;
+    }
+    const int part = threadIdx.x / width, r = threadIdx.x - part * width;
+    if (part < np && r < rows) {
+        double a0 = 0.0, a1 = 0.0;
+        int t = part;
+        for (; t + np <= j; t += 2 * np) {
+            a0 += vec(t, r) * h[t];
+            a1 += vec(t + np, r) * h[t + np];
+        }
+        if (t <= j) a0 += vec(t, r) * h[t];
+        parts[part * width + r] = a0 + a1;
+    }
+    __syncthreads();
+    if (threadIdx.x < rows) {
+        double a = 0.0, b = 0.0;
+        for (int p = 0; p < np; p += 2) {
+            a += parts[p * width + threadIdx.x];
+            if (p + 1 < np) b += parts[(p + 1) * width + threadIdx.x];
+        }
+        put((int)threadIdx.x, ws[threadIdx.x] - (a + b));
+    }
+    __syncthreads();
+}
+template <typename Put, typename Work>
+__device__ __forceinline__ void subtract_basis(const FusedArnoldi &F, const double *ws, int rows, int r0, int j,
+                                               const double *h, double *parts, Work before, Put put) {
+    if (j < F.ks) subtract_basis_t<true>(F, ws, rows, r0, j, h, parts, before, put);
+    else subtract_basis_t<false>(F, ws, rows, r0, j, h, parts, before, put);
+}
+
+__global__ void __launch_bounds__(kFusedThreads, 1) k_arnoldi_fused(FusedArnoldi F) {
+    __shared__ int s_bad, s_stop;
+    __shared__ double s_w2, s_inv;
+    const int n = F.n, m = F.m, ldh = m + 1, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    double *Vs = asm_;                                    // [ks][ld]
+    double *ws_s = Vs + (size_t)F.ks * F.ld;              // [ld]
+    double *h = ws_s + (F.w ? 0 : F.ld);                               // m + 2 each: this pass's sums, the column, rotations, g
+    double *hcol = h + m + 2, *cs = hcol + m + 2, *sn = cs + m + 2, *gv = sn + m + 2;
+    double *chunk = gv + m + 2;                           // [2 warps][8]
+    double *loc0 = chunk + 2 * kFusedWarps * 8, *loc1 = loc0 + m + 2;
+    double *parts = loc1 + m + 2;                         // [threads], then the RAS right-hand sides
+    float *vs = reinterpret_cast<float *>(parts + kFusedThreads) + warp * 128;
+    const unsigned rank = cluster_rank(), csize = cluster_size();
+    const unsigned cid = blockIdx.x / csize, ncl = gridDim.x / csize;
+    const int r0 = min(n, (int)blockIdx.x * F.per), rows = min(n, r0 + F.per) - r0;
+    double *ws = F.w ? F.w + r0 : ws_s;
+    const int iters0 = F.gs->iters;                       // written again only after the first grid-wide barrier
+    const double bnorm = F.gs->bnorm;
+    for (int i = tid; i <= m; i += kFusedThreads) gv[i] = F.g[i];
+    for (int r = tid; r < rows; r += kFusedThreads)
+        if (F.ks > 0) Vs[r] = F.V[r0 + r];
+    if (tid == 0) s_stop = F.gs->stop;
+    __syncthreads();
+    bool done = s_stop != 0;
+    for (int j = 0; j < m && !done; ++j) {
         const double *vj = F.V + (long)j * n;
         if (F.ras_P) {
-            // z_j = M^-1 v_j (Eq. 44): this block's subsets z_p = C_p^-1 (R_p v_j), then the gather of
-            // its own rows; w = C z_j below (right preconditioning, Eq. 45).  z_j is kept: the cycle
-            // ends with u += Z y (the flexible form, exact for the products actually taken, which the
-            // FP32 local solves make only nearly linear in v)
-            const int NP = F.ras_NP;
-            // four groups of 128 threads take four subsets at a time: group g of block b the subsets
-            // b + G (4 k + g); eight loads of C_p^-1 in flight per thread
-            const int grp = tid >> 7, gt = tid & 127;
-            for (int k0 = 0; b + G * k0 < F.ras_P; k0 += 4) {
-                const int p = b + G * (k0 + grp);
-                const bool has = p < F.ras_P;
-                const int wb = has ? F.ras_wptr[p] : 0, np_ = has ? F.ras_wptr[p + 1] - wb : 0;
-                if (gt < NP) vs[grp * 128 + gt] = gt < np_ ? (float)__ldcg(vj + F.ras_widx[wb + gt]) : 0.f;
-                __syncthreads();
-                if (has && gt < NP) {
-                    const float *ci = F.ras_cinvT + (long)p * NP * NP + gt;
-                    const float *vv = vs + grp * 128;
-                    float s = 0.f;
-                    for (int q0 = 0; q0 < np_; q0 += 8) {
-                        float c[8];
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) c[u] = q0 + u < np_ ? ci[(long)(q0 + u) * NP] : 0.f;
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) s = fmaf(c[u], vv[q0 + u < 128 ? q0 + u : 0], s);
-                    }
-                    F.ras_z[(long)p * NP + gt] = s;
-                }
-                __syncthreads();
+            // z_j is kept: the cycle ends with u += Z y (the flexible form, exact for the products actually
+            // taken, which the FP32 local solves make only nearly linear in v)
+            const int nwarps = (int)gridDim.x * kFusedWarps, rr = (F.ras_NP + 31) >> 5;
+            for (int p = (int)blockIdx.x + (int)gridDim.x * warp; p < F.ras_P; p += nwarps) {
+                if (rr == 1) ras_subset<1>(F, p, vj, vs, lane);
+                else if (rr == 2) ras_subset<2>(F, p, vj, vs, lane);
+                else ras_subset<4>(F, p, vj, vs, lane);
             }
-            if (!grid_barrier(F)) return;
+            if (!grid_barrier(F, ncl, rank, &s_bad)) break;
             double *zj = F.ras_Z + (long)j * n;
-            for (int r = r0 + tid; r < r1; r += kFusedThreads) {
+            for (int r = r0 + tid; r < r0 + rows; r += kFusedThreads) {
                 const int q2 = F.ras_p2[r];
-                const double a = (double)__ldcg(F.ras_z + (long)F.ras_p1[r] * NP + F.ras_l1[r]);
-                zj[r] = q2 >= 0 ? 0.5 * (a + (double)__ldcg(F.ras_z + (long)q2 * NP + F.ras_l2[r])) : a;
+                const double a = (double)__ldcg(F.ras_z + (long)F.ras_p1[r] * F.ras_NP + F.ras_l1[r]);
+                zj[r] = q2 >= 0 ? 0.5 * (a + (double)__ldcg(F.ras_z + (long)q2 * F.ras_NP + F.ras_l2[r])) : a;
             }
-            if (!grid_barrier(F)) return;
+            if (!grid_barrier(F, ncl, rank, &s_bad)) break;
             vj = zj;
         }
-        // (every lane of a warp runs the same number of slots: the shuffles below use the full mask);
-        // the row's column indices and values are loaded before the gathers
-        for (int base = r0; base < r1; base += kFusedThreads / 8) {
-            const int row = base + (tid >> 3), l = tid & 7;
-            double s = 0.0;
-            if (row < r1) {
-                const int ka = F.rowptr[row], kb = F.rowptr[row + 1];
-                for (int k0 = ka + l; k0 < kb; k0 += 32) {
-                    int c[4];
-                    double a[4];
+        // w = C v_j: four lanes per row (each FP64 instruction of a warp takes the SM's unit 16 cycles, so
+        // few shuffled additions and no empty rows), two rows of a lane group and 20 of their entries in
+        // flight
+        constexpr int U = 2, E = 5, RG = kFusedThreads / 4;
+        for (int base = 0; base < rows; base += RG * U) {
+            const int l = lane & 3;
+            int ka[U], kb[U], c[U][E];
+            double a[U][E], s[U];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int k = k0 + 8 * q;
-                        c[q] = k < kb ? F.col[k] : 0;
-                        a[q] = k < kb ? F.val[k] : 0.0;
-                    }
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) s += a[q] * __ldcg(vj + c[q]);
+            for (int u = 0; u < U; ++u) {
+                const int r = base + u * RG + (tid >> 2);
+                ka[u] = kb[u] = 0;
+                if (r < rows) {
+                    ka[u] = F.rowptr[r0 + r] + l;
+                    kb[u] = F.rowptr[r0 + r + 1];
                 }
             }
-            s += __shfl_xor_sync(0xffffffffu, s, 4);
-            s += __shfl_xor_sync(0xffffffffu, s, 2);
-            s += __shfl_xor_sync(0xffffffffu, s, 1);
-            if (row < r1 && l == 0) F.w[row] = s;
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const int k = ka[u] + 4 * e;
+                    c[u][e] = k < kb[u] ? F.col[k] : -1;
+                    a[u][e] = k < kb[u] ? F.val[k] : 0.0;
+                }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (base + u * RG + 8 * warp >= rows) break;          // none of the warp's eight rows
+                s[u] = 0.0;
+#pragma unroll
+                for (int e = 0; e < E; ++e)
+                    if (c[u][e] >= 0) s[u] += a[u][e] * __ldcg(vj + c[u][e]);
+                for (int k0 = ka[u] + 4 * E; k0 < kb[u]; k0 += 32) {
+                    int c2[8];
+                    double a2[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const int k = k0 + 4 * e;
+                        c2[e] = k < kb[u] ? F.col[k] : -1;
+                        a2[e] = k < kb[u] ? F.val[k] : 0.0;
+                    }
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        if (c2[e] >= 0) s[u] += a2[e] * __ldcg(vj + c2[e]);
+                }
+                __syncwarp();
+                s[u] += __shfl_xor_sync(0xffffffffu, s[u], 2);
+                s[u] += __shfl_xor_sync(0xffffffffu, s[u], 1);
+                const int r = base + u * RG + (tid >> 2);
+                if (r < rows && l == 0) ws[r] = s[u];
+            }
         }
         __syncthreads();
-        // two passes of classical Gram-Schmidt against v_0 .. v_j; eight loads in flight per lane
-        for (int pass = 0; pass < 2; ++pass) {
-            double *pp = F.part + (long)pass * kMaxDots * G;
-            for (int t = warp; t <= j; t += NW) {
-                const double *vt = F.V + (long)t * n;
-                double s = 0.0;
-                for (int rb = r0 + lane; rb < r1; rb += 256) {
-                    double v[8], x[8];
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        const int r = rb + 32 * q;
-                        v[q] = r < r1 ? vt[r] : 0.0;
-                        x[q] = r < r1 ? F.w[r] : 0.0;
-                    }
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) s += v[q] * x[q];
+        // two passes of classical Gram-Schmidt against v_0 .. v_j, the second with |w|^2
+        local_dots(F, ws, rows, r0, j, false, chunk, loc0, warp, lane);
+        if (!grid_sum(F, j + 1, loc0, F.part, h, ncl, cid, rank, csize, &s_bad)) break;
+        for (int t = tid; t <= j; t += kFusedThreads) hcol[t] = h[t];
+        subtract_basis(F, ws, rows, r0, j, h, parts, [] {}, [&](int r, double v) { ws[r] = v; });
+        local_dots(F, ws, rows, r0, j, true, chunk, loc1, warp, lane);
+        if (!grid_sum(F, j + 2, loc1, F.part + (long)kMaxDots * ncl, h, ncl, cid, rank, csize, &s_bad)) break;
+        // |w|^2 = |w1|^2 - |h2|^2 and its root's inverse, by the last warp while the others subtract; v_{j+1}
+        double *vn = F.V + (long)(j + 1) * n + r0;
+        subtract_basis(
+            F, ws, rows, r0, j, h, parts,
+            [&] {
+                double h2 = 0.0;
+                for (int t = lane; t <= j; t += 32) h2 += h[t] * h[t];
+                h2 = warp_sum(h2);
+                if (lane == 0) {
+                    const double w2 = h[j + 1] - h2;
+                    s_w2 = w2;
+                    s_inv = w2 > 0.5 * h[j + 1] ? 1.0 / sqrt(w2) : -1.0;      // -1: the second pass took much away
                 }
-                s = warp_sum(s);
-                if (lane == 0) pp[(long)t * G + b] = s;
-            }
-            if (!grid_barrier(F)) return;
-            for (int t = warp; t <= j; t += NW) {
-                double s = 0.0;
-                for (int qb = lane; qb < G; qb += 256) {
-                    double v[8];
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) v[q] = qb + 32 * q < G ? __ldcg(pp + (long)t * G + qb + 32 * q) : 0.0;
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) s += v[q];
+            },
+            [&](int r, double v) {
+                const double inv = s_inv;
+                if (inv < 0.0) {
+                    ws[r] = v;
+                } else {
+                    v *= inv;
+                    vn[r] = v;
+                    if (j + 1 < F.ks) Vs[(size_t)(j + 1) * F.ld + r] = v;
                 }
-                s = warp_sum(s);
-                if (lane == 0) h[t] = s;
-            }
-            __syncthreads();
-            if (b == 0)
-                for (int t = tid; t <= j; t += kFusedThreads) hcol[t] = pass ? hcol[t] + h[t] : h[t];
-            for (int r = r0 + tid; r < r1; r += kFusedThreads) {
-                double s = F.w[r];
-                for (int t0 = 0; t0 <= j; t0 += 8) {
-                    double v[8];
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) v[q] = t0 + q <= j ? F.V[(long)(t0 + q) * n + r] : 0.0;
-#pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        if (t0 + q <= j) s -= v[q] * h[t0 + q];
-                }
-                F.w[r] = s;
-            }
-            __syncthreads();
-        }
-        // |w|
-        {
-            double s = 0.0;
-            for (int r = r0 + tid; r < r1; r += kFusedThreads) s += F.w[r] * F.w[r];
-            s = warp_sum(s);
-            if (lane == 0) red[warp] = s;
-            __syncthreads();
+            });
+        for (int t = tid; t <= j; t += kFusedThreads) hcol[t] += h[t];
+        if (s_inv < 0.0) {                                // sum |w|^2 itself
+            local_dots(F, ws, rows, r0, -1, true, chunk, loc0, warp, lane);
+            if (!grid_sum(F, 1, loc0, F.part + 2L * kMaxDots * ncl, h, ncl, cid, rank, csize, &s_bad)) break;
             if (tid == 0) {
-                double t = 0.0;
-                for (int q = 0; q < NW; ++q) t += red[q];
-                F.part[2L * kMaxDots * G + b] = t;
+                s_w2 = h[0];
+                s_inv = h[0] > 0.0 ? 1.0 / sqrt(h[0]) : 0.0;
             }
-        }
-        if (!grid_barrier(F)) return;
-        if (warp == 0) {
-            const double s = warp_sum([&] {
-                double a = 0.0;
-                for (int q = lane; q < G; q += 32) a += __ldcg(F.part + 2L * kMaxDots * G + q);
-                return a;
-            }());
-            if (lane == 0) red[0] = s;
+            __syncthreads();
+            for (int r = tid; r < rows; r += kFusedThreads) {
+                const double v = ws[r] * s_inv;
+                vn[r] = v;
+                if (j + 1 < F.ks) Vs[(size_t)(j + 1) * F.ld + r] = v;
+            }
         }
         __syncthreads();
-        const double nrm = sqrt(red[0]);
-        const double inv = nrm > 0.0 ? 1.0 / nrm : 0.0;
-        double *vn = F.V + (long)(j + 1) * n;
-        for (int r = r0 + tid; r < r1; r += kFusedThreads) vn[r] = F.w[r] * inv;
-        if (b == 0 && tid == 0) {
-            // Givens: the previous rotations on column j, a new one, g and the stop flag
-            hcol[j + 1] = nrm;
+        // Givens, in the shadow of the barrier that completes v_{j+1}: the previous rotations on column j, a
+        // new one, g and the stop flag.  One lane walks the chain hi_{i+1} = c_i h_{i+1} - s_i hi_i (the
+        // products c_i h_{i+1} made by the others), then the lanes form the rotated entries.
+        auto givens = [&] {
+            if (warp != kFusedWarps - 1) return;
+            const double nrm = sqrt(s_w2);
             double hi = hcol[0];
-            for (int i = 0; i < j; ++i) {
-                const double hn = hcol[i + 1];
-                const double t = cs[i] * hi + sn[i] * hn;
-                hi = -sn[i] * hi + cs[i] * hn;
-                hcol[i] = t;
+            for (int i0 = 0; i0 < j; i0 += 32) {
+                const int i = i0 + lane;
+                const double hn = i < j ? hcol[i + 1] : 0.0, ci = i < j ? cs[i] : 0.0, si = i < j ? sn[i] : 0.0;
+                const double p = ci * hn;
+                double mine = 0.0;
+                const int cnt = min(32, j - i0);
+                for (int q = 0; q < cnt; ++q) {
+                    if (lane == q) mine = hi;
+                    hi = fma(-__shfl_sync(0xffffffffu, si, q), hi, __shfl_sync(0xffffffffu, p, q));
+                }
+                __syncwarp();
+                if (i < j) hcol[i] = ci * mine + si * hn;
             }
-            const double a = hi, bb = hcol[j + 1];
-            const double den = hypot(a, bb);
-            const double c = den > 0.0 ? a / den : 1.0, sv = den > 0.0 ? bb / den : 0.0;
-            cs[j] = c;
-            sn[j] = sv;
-            hcol[j] = den;
-            hcol[j + 1] = 0.0;
-            gv[j + 1] = -sv * gv[j];
-            gv[j] = c * gv[j];
-            GState *gs = F.gs;
-            gs->iters += 1;
-            gs->k_used = j + 1;
-            gs->res = fabs(gv[j + 1]);
-            if (gs->res <= F.rtol * gs->bnorm || gs->iters >= F.max_iters || bb == 0.0) gs->stop = 1;
-        }
-        if (b == 0) {
-            __syncthreads();
+            if (lane == 0) {
+                const double den = hypot(hi, nrm);
+                const double c = den > 0.0 ? hi / den : 1.0, sv = den > 0.0 ? nrm / den : 0.0;
+                cs[j] = c;
+                sn[j] = sv;
+                hcol[j] = den;
+                hcol[j + 1] = 0.0;
+                gv[j + 1] = -sv * gv[j];
+                gv[j] = c * gv[j];
+                const double res = fabs(gv[j + 1]);
+                const int iters = iters0 + j + 1;
+                s_stop = res <= F.rtol * bnorm || iters >= F.max_iters || nrm == 0.0;
+                if (blockIdx.x == 0) {
+                    F.gs->iters = iters;
+                    F.gs->k_used = j + 1;
+                    F.gs->res = res;
+                    if (s_stop) F.gs->stop = 1;
+                }
+            }
+            __syncwarp();
+        };
+        if (!grid_barrier(F, ncl, rank, &s_bad, givens)) break;       // v_{j+1} is complete
+        __syncthreads();
+        done = s_stop != 0;
+        if (blockIdx.x == 0) {
             double *Hc = F.H + (long)j * ldh;
             for (int i = tid; i <= j + 1; i += kFusedThreads) Hc[i] = hcol[i];
             for (int i = tid; i <= j + 1; i += kFusedThreads) F.g[i] = gv[i];
         }
-        if (!grid_barrier(F)) return;
     }
+    cluster_barrier();                                    // no CTA ends while another reads its shared memory
 }
 
 // buffers of one GMRES(m) solve; gmres_csr allocates them, the allocation-free entry point carves
 // them from its fixed array
 struct GmresBufs {
-    double *V, *w, *partial, *hsum, *H, *cs, *sn, *g, *y, *fpart;
+    double *V, *w, *partial, *H, *g, *y, *fpart;
     unsigned *cnt, *bar;
     GState *gs;
-    int *err;
 };
 
-// SM count of the current device (the occupancy check once per device: devices may differ)
-static int fused_grid(int n) {
+// clusters of the fused Arnoldi kernel that fit on the current device at once (asked once per device:
+// devices may differ)
+static int device_clusters() {
     static constexpr int kDevs = 64;
-    static int sms_of[kDevs] = {0};
+    static int clusters_of[kDevs] = {0};
     static std::mutex mu;
     int dev = 0;
     PDD_CUDA(cudaGetDevice(&dev));
     if (dev < 0 || dev >= kDevs) fail(PDD_EINVAL, "device ordinal out of range");
     std::lock_guard<std::mutex> lk(mu);
-    if (!sms_of[dev]) {
-        int sms = 0, per_sm = 0;
-        PDD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        PDD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_arnoldi_fused, kFusedThreads, 0));
-        if (per_sm < 1) fail(PDD_ECUDA, "the fused Arnoldi kernel does not fit on an SM");
-        sms_of[dev] = sms;
+    if (!clusters_of[dev]) {
+        PDD_CUDA(cudaFuncSetAttribute(k_arnoldi_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmem));
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = kClusterMax;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(kClusterMax * 64);
+        cfg.blockDim = dim3(kFusedThreads);
+        cfg.dynamicSmemBytes = kFusedSmem;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int nc = 0;
+        PDD_CUDA(cudaOccupancyMaxActiveClusters(&nc, k_arnoldi_fused, &cfg));
+        if (nc < 1) fail(PDD_ECUDA, "the fused Arnoldi kernel does not fit on the device");
+        clusters_of[dev] = nc;
     }
-    return std::max(1, std::min(sms_of[dev], cdiv(n, 64)));     // one block per SM: co-resident, cheap barriers
+    return clusters_of[dev];
+}
+
+// the launch shape of one solve: clusters, CTAs of a cluster, rows of a CTA.  One cluster (no grid-wide
+// barrier) up to 1,024 rows, where the FP64 work of 128 rows a CTA is below a barrier's 2 us; beyond
+// that as many clusters as give each CTA 64 rows, or the device has.
+struct FusedShape {
+    int clusters, csize, per, ld, ks;
+    bool w_global;               // more rows a CTA than shared memory holds (above 3.9 million in all)
+    size_t smem;
+};
+static FusedShape fused_shape(int n, int m) {
+    FusedShape S{};
+    S.clusters = n <= 1024 ? 1 : std::min(device_clusters(), cdiv(n, kClusterMax * kRowsPerCta));
+    S.csize = kClusterMax;
+    while (S.clusters == 1 && S.csize > 1 && (S.csize / 2) * 32 >= n) S.csize /= 2;
+    if (S.clusters == 1) device_clusters();                     // (the shared-memory attribute)
+    S.per = cdiv(n, S.clusters * S.csize);
+    S.ld = (S.per + 13) / 16 * 16 + 2;                          // 2 mod 16 and >= per: the dots' bank rule
+    size_t fixed = fused_fixed_doubles(m, S.ld) * sizeof(double);
+    S.w_global = fixed > kFusedSmem;
+    if (S.w_global) {
+        fixed = fused_fixed_doubles(m, 0) * sizeof(double);
+        S.ks = 0;
+        S.smem = fixed;
+        return S;
+    }
+    S.ks = (int)std::min<size_t>(m + 1, (kFusedSmem - fixed) / (S.ld * sizeof(double)));
+    S.smem = fixed + (size_t)S.ks * S.ld * sizeof(double);
+    return S;
+}
+
+static void launch_fused(const FusedShape &S, FusedArnoldi &F, cudaStream_t st) {
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = S.csize;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeCooperative;
+    at[1].val.cooperative = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(S.clusters * S.csize);
+    cfg.blockDim = dim3(kFusedThreads);
+    cfg.dynamicSmemBytes = S.smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    PDD_CUDA(cudaLaunchKernelEx(&cfg, k_arnoldi_fused, F));
+    count_launch();
 }
 
 // Failure injection on the host (tests): PDD_INJECT_BARRIER_TIMEOUT=1 makes every grid barrier
@@ -455,15 +785,13 @@ static SolveResult gmres_run(int n, const int *rowptr, const int *col, const dou
     PDD_CUDA(cudaMemsetAsync(B.gs, 0, sizeof(GState), st));
     PDD_CUDA(cudaMemsetAsync(B.cnt, 0, sizeof(unsigned) * kDotGroups, st));
     PDD_CUDA(cudaMemsetAsync(B.bar, 0, sizeof(unsigned) * 2, st));
-    PDD_CUDA(cudaMemsetAsync(B.err, 0, sizeof(int), st));
     PDD_CUDA(cudaMemsetAsync(u, 0, sizeof(double) * n, st));
-    PDD_CUDA(cudaMemsetAsync(B.H, 0, sizeof(double) * (m + 1) * m, st));
     const int vb = std::min(cdiv(n, 256), 2048);
     const int max_iters = std::max(1, o.max_iters);
-    const int Gf = fused_grid(n);
+    const FusedShape S = fused_shape(n, m);
     const bool inject = inject_barrier_timeout();
-    FusedArnoldi F{n, m, rowptr, col, val, B.V, B.w, B.fpart, B.H, B.cs, B.sn, B.g, B.gs, B.bar, B.err, o.rtol,
-                   max_iters, inject ? 1u : 0u, inject ? (1LL << 14) : kBarrierLimit, 0, 0, nullptr, nullptr, nullptr,
+    FusedArnoldi F{n, m, rowptr, col, val, B.V, B.fpart, S.w_global ? B.w : nullptr, B.H, B.g, B.gs, B.bar, o.rtol, max_iters, S.per, S.ld, S.ks,
+                   inject ? 1u : 0u, inject ? (1LL << 14) : kBarrierLimit, 0, 0, nullptr, nullptr, nullptr,
                    nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     if (Mr) {
         F.ras_P = Mr->P;
@@ -478,36 +806,31 @@ static SolveResult gmres_run(int n, const int *rowptr, const int *col, const dou
         F.ras_z = Mr->z.p;
         F.ras_Z = Z;
     }
+    double *rr = &B.gs->rr;                                // device address: the residual's squared norm
+    const size_t upper_smem = (size_t)kUpperCols * m * sizeof(double);
+    PDD_CUDA(cudaFuncSetAttribute(k_upper_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)upper_smem));
     SolveResult res;
     for (int cycle = 0;; ++cycle) {
-        // r = b - C u  (u = 0 on the first cycle)
-        PDD_LAUNCH(k_spmv, cdiv(n, kRowsPerBlock), 256, 0, st, n, rowptr, col, val, u, B.w, (const GState *)nullptr);
-        PDD_LAUNCH(k_residual_vec, vb, 256, 0, st, n, b, B.w);
-        PDD_LAUNCH(k_dots, dim3(G, 1), kDotThreads, 0, st, n, 1, B.w, B.w, B.partial, B.hsum, B.cnt,
-                   (const GState *)nullptr);
-        PDD_LAUNCH(k_cycle_start, 1, 32, 0, st, B.gs, B.hsum, B.g, m, o.rtol, max_iters, cycle == 0 ? 1 : 0);
-        PDD_LAUNCH(k_normalize, vb, kDotBlock, 0, st, n, B.w, B.V, B.hsum, (double *)nullptr, B.gs);
-        void *args[] = {&F};
-        PDD_CUDA(cudaLaunchCooperativeKernel((const void *)k_arnoldi_fused, dim3(Gf), dim3(kFusedThreads), args, 0,
-                                             st));
-        count_launch();
-        PDD_LAUNCH(k_upper_solve, 1, 1, 0, st, B.H, m + 1, B.g, B.y, B.gs);
+        // the residual: b on the first cycle (u = 0), what the previous cycle ended with after that
+        const double *r = cycle == 0 ? b : B.w;
+        if (cycle == 0)
+            PDD_LAUNCH(k_dots, dim3(G, 1), kDotThreads, 0, st, n, 1, r, r, B.partial, rr, B.cnt,
+                       (const GState *)nullptr);
+        PDD_LAUNCH(k_cycle_start, 1, 32, 0, st, B.gs, rr, B.g, m, o.rtol, max_iters, cycle == 0 ? 1 : 0);
+        PDD_LAUNCH(k_normalize, vb, kDotBlock, 0, st, n, r, B.V, rr, (double *)nullptr, B.gs);
+        launch_fused(S, F, st);
+        PDD_LAUNCH(k_upper_solve, 1, kUpperThreads, upper_smem, st, B.H, m + 1, B.g, B.y, B.gs);
         // u += Z y (preconditioned: the z_j = M^-1 v_j of the cycle) or V y
         PDD_LAUNCH(k_xupdate, vb, 256, 0, st, n, Mr ? Z : B.V, B.y, B.gs, u);
         // true residual
-        PDD_LAUNCH(k_spmv, cdiv(n, kRowsPerBlock), 256, 0, st, n, rowptr, col, val, u, B.w, (const GState *)nullptr);
-        PDD_LAUNCH(k_residual_vec, vb, 256, 0, st, n, b, B.w);
-        PDD_LAUNCH(k_dots, dim3(G, 1), kDotThreads, 0, st, n, 1, B.w, B.w, B.partial, B.hsum, B.cnt,
+        PDD_LAUNCH(k_spmv, cdiv(n, kRowsPerBlock), 256, 0, st, n, rowptr, col, val, u, B.w, b);
+        PDD_LAUNCH(k_dots, dim3(G, 1), kDotThreads, 0, st, n, 1, B.w, B.w, B.partial, rr, B.cnt,
                    (const GState *)nullptr);
         GState hg{};
-        double rs = 0.0;
-        int herr = 0;
-        PDD_CUDA(cudaMemcpyAsync(&rs, B.hsum, sizeof(double), cudaMemcpyDeviceToHost, st));
         PDD_CUDA(cudaMemcpyAsync(&hg, B.gs, sizeof(GState), cudaMemcpyDeviceToHost, st));
-        PDD_CUDA(cudaMemcpyAsync(&herr, B.err, sizeof(int), cudaMemcpyDeviceToHost, st));
         PDD_CUDA(cudaStreamSynchronize(st));
-        if (herr) fail(PDD_ECUDA, "GMRES grid barrier timed out");
-        const double rel = hg.bnorm > 0.0 ? std::sqrt(rs) / hg.bnorm : 0.0;
+        if (hg.err) fail(PDD_ECUDA, "GMRES grid barrier timed out");
+        const double rel = hg.bnorm > 0.0 ? std::sqrt(hg.rr) / hg.bnorm : 0.0;
         res.iters = hg.iters;
         res.rel = rel;
         if (hg.bnorm == 0.0 || rel <= o.rtol) {
@@ -523,26 +846,20 @@ SolveResult gmres_csr(int n, const int *rowptr, const int *col, const double *va
                       const pdd_solve_opts &o, cudaStream_t st, const RasPrecond *Mr) {
     const int m = std::max(1, std::min(256, o.restart));
     const int G = std::max(1, std::min(1024, cdiv(n, 2 * kDotThreads)));
-    const int Gf = fused_grid(n);
-    DevBuf<double> V, w, partial, hsum, H, cs, sn, g, y, fpart;
+    DevBuf<double> V, w, partial, H, g, y, fpart;
     DevBuf<unsigned> cnt, bar;
     DevBuf<GState> gs;
-    DevBuf<int> err;
     V.alloc((size_t)(m + 1) * n);
     w.alloc(n);
-    partial.alloc((size_t)(m + 1) * G);
-    hsum.alloc(m + 1);
+    partial.alloc(G);
     cnt.alloc(kDotGroups);
     H.alloc((size_t)(m + 1) * m);
-    cs.alloc(m);
-    sn.alloc(m);
     g.alloc(m + 1);
     y.alloc(m);
     gs.alloc(1);
-    fpart.alloc((size_t)3 * kMaxDots * Gf);
+    fpart.alloc((size_t)3 * kMaxDots * fused_shape(n, m).clusters);
     bar.alloc(2);
-    err.alloc(1);
-    const GmresBufs B{V.p, w.p, partial.p, hsum.p, H.p, cs.p, sn.p, g.p, y.p, fpart.p, cnt.p, bar.p, gs.p, err.p};
+    const GmresBufs B{V.p, w.p, partial.p, H.p, g.p, y.p, fpart.p, cnt.p, bar.p, gs.p};
     DevBuf<double> Z;
     if (Mr) Z.alloc((size_t)m * n);
     return gmres_run(n, rowptr, col, val, b, u, o, B, m, G, st, Mr, Z.p);
@@ -641,27 +958,23 @@ static void *noalloc_scratch(int dev) {
 }
 
 struct NoAllocLayout {
-    size_t V, w, partial, hsum, cnt, H, cs, sn, g, y, gs, fpart, bar, err, total;
+    size_t V, w, partial, cnt, H, g, y, gs, fpart, bar, total;
 };
 
-static NoAllocLayout noalloc_layout(int n, int m, int G, int Gf) {
+static NoAllocLayout noalloc_layout(int n, int m, int G, int clusters) {
     auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
     NoAllocLayout L{};
     size_t off = 0;
     L.V = off; off += up(sizeof(double) * (size_t)(m + 1) * n);
     L.w = off; off += up(sizeof(double) * (size_t)n);
-    L.partial = off; off += up(sizeof(double) * (size_t)(m + 1) * G);
-    L.hsum = off; off += up(sizeof(double) * (size_t)(m + 1));
+    L.partial = off; off += up(sizeof(double) * (size_t)G);
     L.cnt = off; off += up(sizeof(unsigned) * kDotGroups);
     L.H = off; off += up(sizeof(double) * (size_t)(m + 1) * m);
-    L.cs = off; off += up(sizeof(double) * (size_t)m);
-    L.sn = off; off += up(sizeof(double) * (size_t)m);
     L.g = off; off += up(sizeof(double) * (size_t)(m + 1));
     L.y = off; off += up(sizeof(double) * (size_t)m);
     L.gs = off; off += up(sizeof(GState));
-    L.fpart = off; off += up(sizeof(double) * (size_t)3 * kMaxDots * Gf);
+    L.fpart = off; off += up(sizeof(double) * (size_t)3 * kMaxDots * clusters);
     L.bar = off; off += up(sizeof(unsigned) * 2);
-    L.err = off; off += up(sizeof(int));
     L.total = off;
     return L;
 }
@@ -671,10 +984,9 @@ static SolveResult gmres_csr_fixed(int n, const int *rowptr, const int *col, con
                                    const double *b, double *u, const pdd_solve_opts &o, unsigned char *base,
                                    const NoAllocLayout &L, int m, int G, cudaStream_t st) {
     const GmresBufs B{(double *)(base + L.V), (double *)(base + L.w), (double *)(base + L.partial),
-                      (double *)(base + L.hsum), (double *)(base + L.H), (double *)(base + L.cs),
-                      (double *)(base + L.sn), (double *)(base + L.g), (double *)(base + L.y),
+                      (double *)(base + L.H), (double *)(base + L.g), (double *)(base + L.y),
                       (double *)(base + L.fpart), (unsigned *)(base + L.cnt), (unsigned *)(base + L.bar),
-                      (GState *)(base + L.gs), (int *)(base + L.err)};
+                      (GState *)(base + L.gs)};
     return gmres_run(n, rowptr, col, val, b, u, o, B, m, G, st);
 }
 
@@ -693,7 +1005,7 @@ extern "C" pdd_status pdd_solve_csr_noalloc(int n, const int *rowptr, const int 
         if (n <= 0 || !rowptr || !col || !val || !b || !u) fail(PDD_EINVAL, "null array or n <= 0");
         const int m = opts->restart;
         const int G = std::max(1, std::min(1024, cdiv(n, 2 * kDotThreads)));
-        const NoAllocLayout L = noalloc_layout(n, m, G, fused_grid(n));
+        const NoAllocLayout L = noalloc_layout(n, m, G, fused_shape(n, m).clusters);
         if (L.total > kNoAllocBytes)
             fail(PDD_EINVAL, "workspace of " + std::to_string(L.total) + " bytes exceeds the fixed " +
                                  std::to_string(kNoAllocBytes) + "-byte array: (restart + 2) * n * 8 bytes "
