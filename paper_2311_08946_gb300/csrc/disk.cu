@@ -4,8 +4,8 @@
 //   a6  k_node_coef + k_fill_operator: per-node FP64 coefficients and row
 //       scales (one thread per node), the right-hand sides [A_IB H, -f], then
 //       the rows of the row-equilibrated collocation matrix of L + c.
-//   a7  FP64 form: k_lu, right-looking blocked LU with partial pivoting, one
-//       CTA per disk, panel in shared memory.  Mixed form: the recursive FP32
+//   a7  FP64 form: lu64.cu, blocked LU with partial pivoting over the whole
+//       device (k_lu, one CTA per disk, where its panel does not fit).  Mixed form: the recursive FP32
 //       LU of lu_rec.cu (tensor-core Schur updates) or the blocked one, chosen
 //       by tune_lu.  The paper factors by QR (Eq. 41); LU solves the same
 //       systems.
@@ -444,28 +444,31 @@ __global__ void __launch_bounds__(256) k_lu(T *Aall, int n, long strideA, int *p
 // (plain form) or X += W with a per-disk convergence test (refinement).
 // Row blocks of TB: the off-diagonal part of each block is a small GEMM
 // staged through shared memory (QB-wide tiles of the factor and of the
-// solved rows), the TB x TB diagonal block is solved column by column.
+// solved rows); in the TB x TB diagonal block a warp takes a column, lane r row r.
+// blockIdx.y takes a group of ncg columns (one group when conv is given): the
+// FP64 pipe of an SM is the bound, so the columns of few disks go to many SMs.
 // ---------------------------------------------------------------------------
 static constexpr int kSolveTB = 32, kSolveQB = 64, kSolveMaxOut = 12;   // nrhs <= 96
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_lu_solve(const T *LUall, int n, long strideA, const int *permAll,
-                                                  const double *Rall, int nrhs, long strideR,
+                                                  const double *Rall, int nrhs, int ncg, long strideR,
                                                   T *Wall, double *Xall, int accumulate, int *conv,
                                                   int *sweeps, double tol) {
     extern __shared__ __align__(16) unsigned char ssm[];
+    constexpr int TB = kSolveTB, QB = kSolveQB;
+    const int c0 = blockIdx.y * ncg, nc = min(ncg, nrhs - c0);
     T *Ls = reinterpret_cast<T *>(ssm);                     // kSolveTB x kSolveQB (factor tile)
-    T *Ys = Ls + kSolveTB * kSolveQB;                       // kSolveQB x nrhs (solved rows)
-    T *Dg = Ys + kSolveQB * nrhs;                           // kSolveTB x kSolveTB diagonal block
-    T *Xs = Dg + kSolveTB * kSolveTB;                       // kSolveTB x nrhs rows being solved
-    const int disk = blockIdx.x, tid = threadIdx.x;
+    T *Ys = Ls + kSolveTB * kSolveQB;                       // kSolveQB x nc (solved rows)
+    T *Dg = Ys + kSolveQB * nc;                             // kSolveTB x (kSolveTB + 1) diagonal block
+    T *Xs = Dg + kSolveTB * (kSolveTB + 1);                 // kSolveTB x nc rows being solved
+    const int disk = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (conv && conv[disk]) return;
     const T *LU = LUall + disk * strideA;
     const int *perm = permAll + (long)disk * n;
-    const double *R = Rall + disk * strideR;
-    T *W = Wall + disk * strideR;
-    double *X = Xall + disk * strideR;
-    constexpr int TB = kSolveTB, QB = kSolveQB;
+    const double *R = Rall + disk * strideR + c0;
+    T *W = Wall + disk * strideR + c0;
+    double *X = Xall + disk * strideR + c0;
     for (int pass = 0; pass < 2; ++pass) {                  // 0: L (unit lower), 1: U (upper)
         const int nblk = (n + TB - 1) / TB;
         for (int bi = 0; bi < nblk; ++bi) {
@@ -481,19 +484,19 @@ __global__ void __launch_bounds__(256) k_lu_solve(const T *LUall, int n, long st
                     const int r = e / QB, q = e - r * QB;
                     Ls[e] = (r < tb && q < qn) ? LU[(long)(i0 + r) * n + q0 + q] : (T)0;
                 }
-                for (int e = tid; e < QB * nrhs; e += 256) {
-                    const int q = e / nrhs, c = e - q * nrhs;
+                for (int e = tid; e < QB * nc; e += 256) {
+                    const int q = e / nc, c = e - q * nc;
                     Ys[e] = (q < qn) ? W[(long)(q0 + q) * nrhs + c] : (T)0;
                 }
                 __syncthreads();
 #pragma unroll
                 for (int o = 0; o < kSolveMaxOut; ++o) {
                     const int e = tid + o * 256;
-                    if (e < tb * nrhs) {
-                        const int r = e / nrhs, c = e - r * nrhs;
+                    if (e < tb * nc) {
+                        const int r = e / nc, c = e - r * nc;
                         T a = acc[o];
                         const T *lr = Ls + r * QB;
-                        for (int q = 0; q < qn; ++q) a += lr[q] * Ys[q * nrhs + c];
+                        for (int q = 0; q < qn; ++q) a += lr[q] * Ys[q * nc + c];
                         acc[o] = a;
                     }
                 }
@@ -501,42 +504,44 @@ __global__ void __launch_bounds__(256) k_lu_solve(const T *LUall, int n, long st
             }
             for (int e = tid; e < tb * tb; e += 256) {
                 const int r = e / tb, c = e - r * tb;
-                Dg[r * TB + c] = LU[(long)(i0 + r) * n + i0 + c];
+                Dg[r * (TB + 1) + c] = LU[(long)(i0 + r) * n + i0 + c];
             }
 #pragma unroll
             for (int o = 0; o < kSolveMaxOut; ++o) {
                 const int e = tid + o * 256;
-                if (e < tb * nrhs) {
-                    const int r = e / nrhs, c = e - r * nrhs;
+                if (e < tb * nc) {
+                    const int r = e / nc, c = e - r * nc;
                     const T rhs = pass == 0 ? (T)R[(long)perm[i0 + r] * nrhs + c] : W[(long)(i0 + r) * nrhs + c];
-                    Xs[r * nrhs + c] = rhs - acc[o];
+                    Xs[r * nc + c] = rhs - acc[o];
                 }
             }
             __syncthreads();
-            // the diagonal block, in shared memory
-            for (int c = tid; c < nrhs; c += 256) {
+            // the diagonal block
+            const T dinv = (pass == 1 && lane < tb) ? (T)1 / Dg[lane * (TB + 1) + lane] : (T)1;
+            for (int c = warp; c < nc; c += 8) {
+                T x = lane < tb ? Xs[lane * nc + c] : (T)0;
                 if (pass == 0) {
-                    for (int ii = 1; ii < tb; ++ii) {
-                        T v = Xs[ii * nrhs + c];
-                        for (int t = 0; t < ii; ++t) v -= Dg[ii * TB + t] * Xs[t * nrhs + c];
-                        Xs[ii * nrhs + c] = v;
+                    for (int t = 0; t < tb - 1; ++t) {
+                        const T xt = __shfl_sync(0xffffffffu, x, t);
+                        if (lane > t && lane < tb) x -= Dg[lane * (TB + 1) + t] * xt;
                     }
                 } else {
-                    for (int ii = tb - 1; ii >= 0; --ii) {
-                        T v = Xs[ii * nrhs + c];
-                        for (int t = ii + 1; t < tb; ++t) v -= Dg[ii * TB + t] * Xs[t * nrhs + c];
-                        Xs[ii * nrhs + c] = v / Dg[ii * TB + ii];
+                    for (int t = tb - 1; t >= 0; --t) {
+                        const T xt = __shfl_sync(0xffffffffu, x * dinv, t);
+                        if (lane == t) x = xt;
+                        if (lane < t) x -= Dg[lane * (TB + 1) + t] * xt;
                     }
                 }
+                if (lane < tb) W[(long)(i0 + lane) * nrhs + c] = x;
             }
-            __syncthreads();
-            for (int e = tid; e < tb * nrhs; e += 256) W[(long)i0 * nrhs + e] = Xs[e];
             __syncthreads();
         }
     }
     // X = W or X += W; refinement test max|W| <= tol max|X|
     double dmax = 0.0, xmax = 0.0;
-    for (long o = tid; o < (long)n * nrhs; o += 256) {
+    for (int e = tid; e < n * nc; e += 256) {
+        const int r = e / nc;
+        const long o = (long)r * nrhs + (e - r * nc);
         const double w = (double)W[o];
         const double xv = accumulate ? X[o] + w : w;
         X[o] = xv;
@@ -550,7 +555,7 @@ __global__ void __launch_bounds__(256) k_lu_solve(const T *LUall, int n, long st
         dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
         xmax = fmax(xmax, __shfl_xor_sync(0xffffffffu, xmax, o));
     }
-    if ((tid & 31) == 0) { sd[tid >> 5] = dmax; sx[tid >> 5] = xmax; }
+    if (lane == 0) { sd[warp] = dmax; sx[warp] = xmax; }
     __syncthreads();
     if (tid == 0) {
         double d = 0.0, x = 0.0;
@@ -562,7 +567,7 @@ __global__ void __launch_bounds__(256) k_lu_solve(const T *LUall, int n, long st
 
 template <typename T>
 static size_t solve_smem(int nrhs) {
-    return sizeof(T) * ((size_t)kSolveTB * kSolveQB + (size_t)kSolveQB * nrhs + (size_t)kSolveTB * kSolveTB +
+    return sizeof(T) * ((size_t)kSolveTB * kSolveQB + (size_t)kSolveQB * nrhs + (size_t)kSolveTB * (kSolveTB + 1) +
                         (size_t)kSolveTB * nrhs);
 }
 
@@ -570,9 +575,15 @@ template <typename T>
 static void launch_solve(const T *LU, int n, long sA, const int *perm, const double *R, int nrhs, long sR, T *W,
                          double *X, int accumulate, int *conv, int *sweeps, double tol, int nd, cudaStream_t st) {
     if (nrhs > 96) fail(PDD_EINVAL, "more than 95 knots per circle");
-    const size_t sm = solve_smem<T>(nrhs);
+    // groups of columns (at least four each: 128 outputs of a row block) until the device has two CTAs per SM
+    int dev = 0, sms = 0, groups = 1;
+    PDD_CUDA(cudaGetDevice(&dev));
+    PDD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    if (!conv) groups = std::max(1, std::min(cdiv(2L * sms, nd), nrhs / 4));
+    const int ncg = cdiv(nrhs, groups);
+    const size_t sm = solve_smem<T>(ncg);
     PDD_CUDA(cudaFuncSetAttribute(k_lu_solve<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    PDD_LAUNCH(k_lu_solve<T>, nd, 256, sm, st, LU, n, sA, perm, R, nrhs, sR, W, X, accumulate, conv, sweeps, tol);
+    PDD_LAUNCH(k_lu_solve<T>, dim3(nd, cdiv(nrhs, ncg)), 256, sm, st, LU, n, sA, perm, R, nrhs, ncg, sR, W, X, accumulate, conv, sweeps, tol);
 }
 
 // ---------------------------------------------------------------------------
@@ -1425,6 +1436,8 @@ static int lu_nb(int n, size_t elem) {
 
 template <typename T>
 static void launch_lu(T *A, int n, long strideA, int *perm, int *info, int nd, cudaStream_t st) {
+    if constexpr (sizeof(T) == 8)
+        if (lu_f64(A, n, strideA, perm, info, nd, st)) return;
     const int nb = lu_nb(n, sizeof(T));
     const size_t smem = ((size_t)n * (nb + 1) + (size_t)nb * 64) * sizeof(T);
     switch (nb) {

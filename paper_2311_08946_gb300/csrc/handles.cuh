@@ -173,6 +173,9 @@ void grad_impl(const pdd_cover &cov, const Problem &P, const pdd_assembly_opts &
 void lu_recursive_f32(float *A, int n, long strideA, int *perm, int *info, int nd, cudaStream_t st, int W,
                       int tensor_min, float *ms_gemm = nullptr, double *gemm_flop = nullptr);
 
+// blocked LU of a batch of FP64 matrices (lu64.cu); false: n or nd beyond its launches
+bool lu_f64(double *A, int n, long strideA, int *perm, int *info, int nd, cudaStream_t st);
+
 // batched split-TF32 tensor-core GEMM C_b (-)= A_b B_b (tc_gemm.cu); `alias` states how C meets
 // the operands, scratch holds pre-split tiles for the cases the fused kernel does not take
 enum { TC_ALIAS_NONE = 0, TC_ALIAS_A = 1, TC_ALIAS_B = 2, TC_ALIAS_UNKNOWN = 3 };
