@@ -174,7 +174,7 @@ void spmv_csr(int n, const int *rowptr, const int *col, const double *val, const
 }
 
 // ---------------------------------------------------------------------------
-// One restart cycle's Arnoldi iterations in a single cooperative launch of clusters of eight CTAs.
+// One restart cycle's Arnoldi iterations in a single cooperative launch of clusters of CTAs.
 // Each CTA owns `per` rows: it computes w = C v_j on them, keeps w and (as far as shared memory goes:
 // 64 vectors of 400 rows) its part of the basis in shared memory, and takes part in two passes of
 // classical Gram-Schmidt.  Dot products are added over a CTA's warps, then over the cluster through
@@ -184,11 +184,11 @@ void spmv_csr(int n, const int *rowptr, const int *col, const double *val, const
 // by itself from the same sums, so an iteration has three grid-wide barriers.
 // Why: four barriers, basis slices read from L2 by latency-bound loops, 152 partial sums per vector
 // read by every CTA and a serial rotation on the critical path cost 22 us an iteration at n = 204 and
-// 52 us at n = 32,768; what is left is the FP64 pipe (4 n j products an iteration) and the barriers: 13 and 37 us.
+// 52 us at n = 32,768; what is left is the FP64 pipe (4 n j products an iteration) and the barriers: 13 and 35 us.
 // With RAS (Eq. 44-45) z_j = M^-1 v_j comes first (two more barriers), one warp per subset.
 // ---------------------------------------------------------------------------
 static constexpr int kFusedThreads = 512, kFusedWarps = kFusedThreads / 32;
-static constexpr int kClusterMax = 8;
+static constexpr int kClusterMax = 8, kClusterMany = 4;     // CTAs of a lone cluster, of each of several
 static constexpr int kRowsPerCta = 64;                  // fewer clusters than the device holds below this
 static constexpr size_t kFusedSmem = 222 * 1024;
 static constexpr long long kBarrierLimit = 1LL << 22;   // polls (an L2 read each, ~0.2 us) before giving up
@@ -653,8 +653,10 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_arnoldi_fused(FusedArnoldi
                 if (i < j) hcol[i] = ci * mine + si * hn;
             }
             if (lane == 0) {
-                const double den = hypot(hi, nrm);
-                const double c = den > 0.0 ? hi / den : 1.0, sv = den > 0.0 ? nrm / den : 0.0;
+                const double top = fmax(fabs(hi), nrm);
+                const double den = top > 1e-140 && top < 1e140 ? sqrt(hi * hi + nrm * nrm) : hypot(hi, nrm);
+                const double rd = 1.0 / den;
+                const double c = den > 0.0 ? hi * rd : 1.0, sv = den > 0.0 ? nrm * rd : 0.0;
                 cs[j] = c;
                 sn[j] = sv;
                 hcol[j] = den;
@@ -707,10 +709,10 @@ static int device_clusters() {
         PDD_CUDA(cudaFuncSetAttribute(k_arnoldi_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmem));
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = kClusterMax;
+        at[0].val.clusterDim.x = kClusterMany;
         at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
         cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(kClusterMax * 64);
+        cfg.gridDim = dim3(kClusterMany * 64);
         cfg.blockDim = dim3(kFusedThreads);
         cfg.dynamicSmemBytes = kFusedSmem;
         cfg.attrs = at;
@@ -725,7 +727,8 @@ static int device_clusters() {
 
 // the launch shape of one solve: clusters, CTAs of a cluster, rows of a CTA.  One cluster (no grid-wide
 // barrier) up to 1,024 rows, where the FP64 work of 128 rows a CTA is below a barrier's 2 us; beyond
-// that as many clusters as give each CTA 64 rows, or the device has.
+// that as many clusters as give each CTA 64 rows, or the device has: clusters of four, which fill its
+// SMs (clusters of eight fit 15 times, on 120 of 152).
 struct FusedShape {
     int clusters, csize, per, ld, ks;
     bool w_global;               // more rows a CTA than shared memory holds (above 3.9 million in all)
@@ -733,8 +736,8 @@ struct FusedShape {
 };
 static FusedShape fused_shape(int n, int m) {
     FusedShape S{};
-    S.clusters = n <= 1024 ? 1 : std::min(device_clusters(), cdiv(n, kClusterMax * kRowsPerCta));
-    S.csize = kClusterMax;
+    S.clusters = n <= 1024 ? 1 : std::min(device_clusters(), cdiv(n, kClusterMany * kRowsPerCta));
+    S.csize = S.clusters == 1 ? kClusterMax : kClusterMany;
     while (S.clusters == 1 && S.csize > 1 && (S.csize / 2) * 32 >= n) S.csize /= 2;
     if (S.clusters == 1) device_clusters();                     // (the shared-memory attribute)
     S.per = cdiv(n, S.clusters * S.csize);
