@@ -431,35 +431,7 @@ static void build_grid(Grid G, int n, const double *x, const double *y, DevBuf<i
     if (n) PDD_LAUNCH(k_cell_fill, cdiv(n, 256), 256, 0, st, n, cell.p, ptr.p, cursor.p, items.p);
 }
 
-// ---------------------------------------------------------------------------
-// Eq. 5 (left) on a sample grid of pitch min(r)/4
-// ---------------------------------------------------------------------------
-__global__ void k_coverage(Problem P, Grid G, int sx, int sy, double bx0, double by0, double bx1,
-                           double by1, const int *cptr, const int *citems, const double *cx,
-                           const double *cy, const double *r, int *uncovered) {
-    int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= sx * sy) return;
-    int i = idx % sx, j = idx / sx;
-    double x = bx0 + (i + 0.5) * (bx1 - bx0) / sx;
-    double y = by0 + (j + 0.5) * (by1 - by0) / sy;
-    if (!inside_domain(P, x, y)) return;
-    int c = G.cell_of(x, y), ix = c % G.gx, iy = c / G.gx;
-    for (int b = max(0, iy - 1); b <= min(G.gy - 1, iy + 1); ++b)
-        for (int a = max(0, ix - 1); a <= min(G.gx - 1, ix + 1); ++a) {
-            int cc = b * G.gx + a;
-            for (int q = cptr[cc]; q < cptr[cc + 1]; ++q) {
-                int m = citems[q];
-                double dx = x - cx[m], dy = y - cy[m];
-                if (dx * dx + dy * dy < r[m] * r[m]) return;
-            }
-        }
-    atomicAdd(uncovered, 1);
-}
-
-// ---------------------------------------------------------------------------
-// a4: row assignment
-// ---------------------------------------------------------------------------
-// circles in cell order as FP32 (x, y, r), for the tests that rule a circle out
+// circles in cell order as FP32 (x, y, r), for the tests that FP32 can decide
 __global__ void k_cell_circles(int M, const int *citems, const double *cx, const double *cy, const double *r,
                                float4 *c32) {
     int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -468,6 +440,47 @@ __global__ void k_cell_circles(int M, const int *citems, const double *cx, const
     c32[q] = make_float4((float)cx[m], (float)cy[m], (float)r[m], 0.f);
 }
 
+// Whether circle f holds (x, y): 1 surely, -1 surely not, 0 for the FP64 test to say.  FP32 coordinates
+// are off by 2^-24 of their size; `slack` is 16 times that (1e-6 of |x| + |y| + the cells' pitch), and
+// 1e-5 of the radius is to spare on either side.
+__device__ __forceinline__ int holds32(float4 f, float x, float y, float slack) {
+    const float dx = x - f.x, dy = y - f.y, d2 = dx * dx + dy * dy;
+    const float out = f.z * 1.00001f + slack, in = f.z * 0.99999f - slack;
+    if (d2 > out * out) return -1;
+    return in > 0.f && d2 < in * in ? 1 : 0;
+}
+
+// ---------------------------------------------------------------------------
+// Eq. 5 (left) on a sample grid of pitch min(r)/4
+// ---------------------------------------------------------------------------
+__global__ void k_coverage(Problem P, Grid G, int sx, int sy, double bx0, double by0, double bx1,
+                           double by1, const int *cptr, const int *citems, const float4 *c32, const double *cx,
+                           const double *cy, const double *r, int *uncovered) {
+    int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= sx * sy) return;
+    int i = idx % sx, j = idx / sx;
+    double x = bx0 + (i + 0.5) * (bx1 - bx0) / sx;
+    double y = by0 + (j + 0.5) * (by1 - by0) / sy;
+    if (!inside_domain(P, x, y)) return;
+    const float xf = (float)x, yf = (float)y, slack = 1e-6f * (fabsf(xf) + fabsf(yf) + (float)G.h);
+    int c = G.cell_of(x, y), ix = c % G.gx, iy = c / G.gx;
+    for (int b = max(0, iy - 1); b <= min(G.gy - 1, iy + 1); ++b) {
+        const int q0 = cptr[b * G.gx + max(0, ix - 1)], q1 = cptr[b * G.gx + min(G.gx - 1, ix + 1) + 1];
+        for (int q = q0; q < q1; ++q) {
+            const int in = holds32(c32[q], xf, yf, slack);
+            if (in < 0) continue;
+            if (in > 0) return;
+            const int m = citems[q];
+            double dx = x - cx[m], dy = y - cy[m];
+            if (dx * dx + dy * dy < r[m] * r[m]) return;
+        }
+    }
+    atomicAdd(uncovered, 1);
+}
+
+// ---------------------------------------------------------------------------
+// a4: row assignment
+// ---------------------------------------------------------------------------
 // Every knot looks at the circles of the 3 x 3 cells around it (pitch: the largest radius), hundreds
 // when the radii are uneven, and lies inside a few.  The FP64 score (a square root) was the bound
 // (2.3 ms for 127 thousand knots of the 7,108-circle cover); an FP32 distance test that can only rule
@@ -485,41 +498,52 @@ __global__ void k_assign_rows(Grid G, int N, const double *kx, const double *ky,
     const double x = kx[i], y = ky[i];
     const int own = kowner[i];
     const double eps = kScoreEps * r[own];
-    const float xf = (float)x, yf = (float)y;
-    // FP32 coordinates are off by 2^-24 of their size; 16 times that and 1e-5 of the radius to spare
-    const float slack = 1e-6f * (fabsf(xf) + fabsf(yf) + (float)G.h);
+    const float xf = (float)x, yf = (float)y, slack = 1e-6f * (fabsf(xf) + fabsf(yf) + (float)G.h);
     int c = G.cell_of(x, y), ix = c % G.gx, iy = c / G.gx;
-    double best = -1.0;
-    bool any = false;
+    // first pass: the best score, and the circles that hold the knot while they are few; the owner is the
+    // lowest index within eps of the best, from that list or a second pass
+    constexpr int kList = 6;
+    int lm[kList], n = 0;
+    double ls[kList], best = -1.0;
+    int pick = 0x7fffffff;
     for (int pass = 0; pass < 2; ++pass) {
-        int pick = 0x7fffffff;
         for (int b = max(0, iy - 1); b <= min(G.gy - 1, iy + 1); ++b) {
             // the cells of a row of cells are consecutive, and so are their circles
             const int q0 = cptr[b * G.gx + max(0, ix - 1)], q1 = cptr[b * G.gx + min(G.gx - 1, ix + 1) + 1];
             for (int q = q0; q < q1; ++q) {
-                const float4 f = c32[q];
-                const float dxf = xf - f.x, dyf = yf - f.y, rf = f.z * 1.00001f + slack;
-                if (dxf * dxf + dyf * dyf > rf * rf) continue;
+                if (holds32(c32[q], xf, yf, slack) < 0) continue;
                 int m = citems[q];
                 if (m == own) continue;
                 double dx = x - cx[m], dy = y - cy[m];
                 double s = r[m] - sqrt(dx * dx + dy * dy);
                 if (!(s > eps)) continue;
                 if (pass == 0) {
-                    if (!any || s > best) best = s;
-                    any = true;
+                    if (!n || s > best) best = s;
+#pragma unroll
+                    for (int k = 0; k < kList; ++k)
+                        if (k == n) {
+                            lm[k] = m;
+                            ls[k] = s;
+                        }
+                    ++n;
                 } else if (s >= best - eps && m < pick) {
                     pick = m;
                 }
             }
         }
-        if (pass == 0 && !any) {
+        if (n == 0) {
             row_sub[i] = -2;
             atomicAdd(uncovered, 1);
             return;
         }
-        if (pass == 1) row_sub[i] = pick;
+        if (n <= kList) {
+#pragma unroll
+            for (int k = 0; k < kList; ++k)
+                if (k < n && ls[k] >= best - eps && lm[k] < pick) pick = lm[k];
+            break;
+        }
     }
+    row_sub[i] = pick;
 }
 
 // ---------------------------------------------------------------------------
@@ -834,6 +858,10 @@ void build_cover_impl(const pdd_domain &dom, const pdd_cover_spec &spec, pdd_cov
     err.alloc(8);
     PDD_CUDA(cudaMemsetAsync(err.p, 0, 8 * sizeof(int), st));
 
+    DevBuf<float4> c32;
+    c32.alloc(M);
+    PDD_LAUNCH(k_cell_circles, cdiv(M, 256), 256, 0, st, M, cov.cell_items.p, cov.cx.p, cov.cy.p, cov.r.p, c32.p);
+
     // Eq. 5 (left): sampled coverage
     {
         double x0, y0, x1, y1;
@@ -847,7 +875,7 @@ void build_cover_impl(const pdd_domain &dom, const pdd_cover_spec &spec, pdd_cov
         int sx = (int)std::ceil((x1 - x0) / h), sy = (int)std::ceil((y1 - y0) / h);
         if ((double)sx * sy > 4e8) fail(PDD_EINVAL, "coverage sample grid too large");
         PDD_LAUNCH(k_coverage, cdiv((long)sx * sy, 256), 256, 0, st, P, G, sx, sy, x0, y0, x1, y1,
-                   cov.cell_ptr.p, cov.cell_items.p, cov.cx.p, cov.cy.p, cov.r.p, err.p + 3);
+                   cov.cell_ptr.p, cov.cell_items.p, c32.p, cov.cx.p, cov.cy.p, cov.r.p, err.p + 3);
     }
 
     // a2-a3: knots
@@ -882,9 +910,6 @@ void build_cover_impl(const pdd_domain &dom, const pdd_cover_spec &spec, pdd_cov
                    err.p + 2);
     }
     // a4: rows
-    DevBuf<float4> c32;
-    c32.alloc(M);
-    PDD_LAUNCH(k_cell_circles, cdiv(M, 256), 256, 0, st, M, cov.cell_items.p, cov.cx.p, cov.cy.p, cov.r.p, c32.p);
     PDD_LAUNCH(k_assign_rows, cdiv(N, 256), 256, 0, st, G, N, cov.kx.p, cov.ky.p, cov.kowner.p,
                cov.kdir.p, cov.cell_ptr.p, cov.cell_items.p, c32.p, cov.cx.p, cov.cy.p, cov.r.p,
                cov.row_sub.p, err.p + 1);
