@@ -275,9 +275,288 @@ __device__ __forceinline__ void cv_accumulate(R (&cq)[kMaxCv], int D, R xr, R yr
     }
 }
 
-// mixed form: positions, drift and normals in FP32, weights in FP64
-template <bool KILL, bool SRC, bool CV>
-__global__ void __launch_bounds__(256) k_paths(Problem P, PathArgs A) {
+// a / b rounded to nearest, rb = 1 / b: quotient and residual corrected twice by FMAs (P. Markstein, IBM
+// J. Res. Dev. 34, 1990), where the compiler's division takes a dozen instructions and a branch
+__device__ __forceinline__ float quotient(float a, float b, float rb) {
+    float q = __fmul_rn(a, rb);
+    q = fmaf(fmaf(-q, b, a), rb, q);
+    return fmaf(fmaf(-q, b, a), rb, q);
+}
+
+// packed FP32 pairs, each lane of the pair rounded like the scalar operation
+__device__ __forceinline__ unsigned long long pack2(float a, float b) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(unsigned long long r, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long fma2p(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// Gaussians in shared memory, two by two: (-x0, -x1, -y0, -y1) and (w0, w1), a missing second one with
+// weight 0.  The sum of killing32 and source32_given, term by term and rounding by rounding; per pair two
+// shared loads and five packed operations where the global form takes six loads and ten.
+struct GaussTab {
+    const float4 *xy;
+    const float2 *w;
+    int pairs;
+    float ninv;              // -1 / (2 sigma^2)
+};
+__device__ __forceinline__ float gauss_sum(const GaussTab &G, float x, float y) {
+    const unsigned long long x2 = pack2(x, x), y2 = pack2(y, y), n2 = pack2(G.ninv, G.ninv);
+    float s = 0.f;
+#pragma unroll 4
+    for (int q = 0; q < G.pairs; ++q) {
+        const float4 c = G.xy[q];
+        const float2 w = G.w[q];
+        const unsigned long long dx = add2(x2, pack2(c.x, c.y)), dy = add2(y2, pack2(c.z, c.w));
+        float a0, a1;
+        unpack2(mul2(fma2p(dx, dx, mul2(dy, dy)), n2), a0, a1);
+        s = fmaf(w.x, __expf(a0), s);
+        s = fmaf(w.y, __expf(a1), s);
+    }
+    return s;
+}
+
+// ---------------------------------------------------------------------------
+// Mixed form: positions, drift and normals in FP32, weights in FP64.  Instruction issue bounds it
+// (Philox, Box-Muller and the coefficients, some 150 instructions a step).
+//   k_paths       one CTA per row, whose constants are the block's: starting a path takes a few
+//                 instructions, for short paths (62 steps on the variable-coefficient cover).
+//   k_paths_long  resident warps take the launch's records 256 at a time and hand them to the lanes
+//                 that are free: no lanes idle while the last paths of a row finish, no part-filled last
+//                 wave of CTAs; exit points by k_exit32, one thread per record.  Starting a path takes some
+//                 eighty instructions (its row's constants), so it is for paths of kLongSteps steps and
+//                 more on average.
+// Control variate of degree 4, boundary shift (1,000 rows x 5,000 paths of 1,684 steps): 179 -> 141 ms in
+// k_paths_long; drift, killing and source (2,276 rows x 10^4 paths): 16.5 ms in k_paths, 31 in
+// k_paths_long; killing by 64 Gaussians (3,000 rows), read from shared memory two at a time: 68 -> 49 ms.
+// ---------------------------------------------------------------------------
+struct alignas(16) Slot32 {          // what a path reads when it starts
+    float cx, cy, r2, rs, x0, y0, rad, ts;      // r2, rs: of the disk shrunk by the boundary shift
+    long rbase;
+    int i, max_steps;
+    uint32_t kw;
+    int pad[3];
+};
+struct Pool32 {
+    const Slot32 *slots;
+    int nslots;
+    long total;                      // records of the launch
+    unsigned *next;                  // chunks taken
+    float4 *seg;                     // per record: the last step's segment (x, y, nx, ny)
+    int nc, nf;                      // Gaussians of c and f kept in shared memory (0: none)
+};
+static constexpr int kP32Threads = 128, kP32Chunk = 256, kRowThreads = 256;
+static constexpr double kLongSteps = 500.0;
+static constexpr int kP32Staged = 1024;          // most Gaussians of c or f kept in shared memory (24 KB each)
+
+__global__ void k_slots32(int n, PathArgs A, Slot32 *out) {
+    const int slot = blockIdx.x * blockDim.x + threadIdx.x;
+    if (slot >= n) return;
+    const int gsl = A.gslot ? A.gslot[slot] : slot;
+    const int i = A.rows[slot], m = A.subs[gsl];
+    const double rad = A.cr[m], rs = rad - A.shift;
+    Slot32 s;
+    s.cx = (float)A.ccx[m];
+    s.cy = (float)A.ccy[m];
+    s.r2 = (float)(rs * rs);
+    s.rs = (float)rs;
+    s.x0 = (float)A.kx[i];
+    s.y0 = (float)A.ky[i];
+    s.rad = (float)rad;
+    s.ts = (float)A.theta_s[m];
+    s.rbase = A.rec_off ? A.rec_off[slot] : (long)slot * A.paths;
+    s.i = i;
+    s.max_steps = A.max_steps > 0 ? A.max_steps : (int)fmin(2147483647.0, ceil(50.0 * rad * rad / A.h));
+    s.kw = A.kword ? (uint32_t)A.kword[gsl] : 0u;
+    s.pad[0] = s.pad[1] = s.pad[2] = 0;
+    out[slot] = s;
+}
+
+// the slot of record g (the records of the slots are contiguous and in slot order)
+template <typename SlotT>
+__device__ __forceinline__ int slot_of(const PathArgs &A, const SlotT *slots, int nslots, long g) {
+    if (!A.rec_off) return (int)((unsigned)g / (unsigned)A.paths);      // at most 2^31 records per launch
+    int lo = 0, hi = nslots - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (slots[mid].rbase <= g) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
+// a Gaussian family into shared memory (see GaussTab), by the block
+__device__ __forceinline__ GaussTab stage_gauss(float4 *smem, const float *src, int n, float inv2s2) {
+    GaussTab G;
+    G.pairs = (n + 1) >> 1;
+    G.ninv = -inv2s2;
+    float2 *w = reinterpret_cast<float2 *>(smem + G.pairs);
+    for (int q = threadIdx.x; q < G.pairs; q += blockDim.x) {
+        const int a = 2 * q, b = 2 * q + 1 < n ? 2 * q + 1 : a;
+        smem[q] = make_float4(-src[a], -src[b], -src[n + a], -src[n + b]);
+        w[q] = make_float2(src[2 * n + a], 2 * q + 1 < n ? src[2 * n + b] : 0.f);
+    }
+    G.xy = smem;
+    G.w = w;
+    return G;
+}
+__host__ __device__ constexpr size_t gauss_smem(int n) { return (((size_t)(n + 1) / 2) * 24 + 15) / 16 * 16; }
+
+// constants of a launch
+struct Env32 {
+    GaussTab gc, gf;
+    float h, sh, d0, d1, d2, d3, dr2;
+    bool sq_dom;
+};
+template <bool KILL, bool SRC>
+__device__ __forceinline__ Env32 env32(const Problem &P, const PathArgs &A, const Pool32 &Q, unsigned char *smem) {
+    Env32 E{};
+    if (KILL && Q.nc) E.gc = stage_gauss(reinterpret_cast<float4 *>(smem), P.rbf32, Q.nc, P.rbf_inv2s2);
+    if (SRC && Q.nf)
+        E.gf = stage_gauss(reinterpret_cast<float4 *>(smem + (Q.nc ? gauss_smem(Q.nc) : 0)), P.frbf32, Q.nf,
+                           P.frbf_inv2s2);
+    const double sft = A.shift;
+    E.sq_dom = P.dom_kind == 0;
+    E.h = (float)A.h;
+    E.sh = sqrtf((float)A.h);
+    E.d0 = (float)(E.sq_dom ? P.dom[0] + sft : P.dom[0]);
+    E.d1 = (float)(E.sq_dom ? P.dom[1] + sft : P.dom[1]);
+    E.d2 = (float)(P.dom[2] - sft);
+    E.d3 = (float)(P.dom[3] - sft);
+    E.dr2 = (float)((P.dom[2] - sft) * (P.dom[2] - sft));
+    return E;
+}
+
+// a path: position, weights Y = Yv (1 + e) and Z = Zv + Yv z (e, z: FP32 increments), step count
+struct Path32 {
+    float x, y, e, z;
+    double Yv, Zv;
+    int k;
+};
+
+// One Euler-Maruyama step of path S (of knot, on the circle (cx, cy) with squared radius r2): moves it, or
+// returns true when its end point (nx, ny) is outside, the weights then being those after the step.
+// `fold`: the iterations that fold the FP32 increments into the FP64 weights.
+// CVD: control-variate degree, 0 (none), 4, or -1 (A.cvd at run time)
+template <bool KILL, bool SRC, int CVD>
+__device__ __forceinline__ bool step32(const Problem &P, const PathArgs &A, const Pool32 &Q, const Env32 &E, Path32 &S,
+                                       int knot, uint32_t kw, int p, float cx, float cy, float r2, float crad,
+                                       float rcrad, float *cq, bool fold, float &nx, float &ny) {
+    float xi0, xi1;
+    normals32(A.seed, (uint32_t)knot, kw, (uint32_t)S.k, (uint32_t)p, xi0, xi1);
+    if constexpr (CVD != 0) {
+        // Y_k sqrt(h) grad psi(X_k) . xi_k / r, with Y_k the weight before this step
+        const float yk = (float)S.Yv * (1.0f + S.e);
+        cv_accumulate<float>(*reinterpret_cast<float(*)[kMaxCv]>(cq), CVD > 0 ? CVD : A.cvd,
+                             quotient(S.x - cx, crad, rcrad), quotient(S.y - cy, crad, rcrad),
+                             quotient(yk * E.sh, crad, rcrad), xi0, xi1);
+    }
+    float bx, by;
+    Num<float>::drift(P, S.x, S.y, bx, by);
+    float cv = 0.f;
+    if (KILL) {
+        if (Q.nc) {
+            const float s = gauss_sum(E.gc, S.x, S.y);
+            cv = s < 0.f ? s : 0.f;
+        } else {
+            cv = killing32(P, S.x, S.y);
+        }
+    }
+    // Z_{k+1} = Z_k + f_k h Y_k and Y_{k+1} = Y_k (1 + c_k h), with Y_k = Yv (1 + e)
+    const float e = S.e;
+    if (SRC) {
+        const float fv = Q.nf ? gauss_sum(E.gf, S.x, S.y) : source32_given(P, S.x, S.y, bx, by, cv);
+        S.z = fmaf(fv * E.h, 1.0f + e, S.z);
+    }
+    if (KILL) S.e = fmaf(cv * E.h, 1.0f + e, e);
+    nx = S.x + bx * E.h + E.sh * xi0;
+    ny = S.y + by * E.h + E.sh * xi1;
+    ++S.k;
+    const float ddx = nx - cx, ddy = ny - cy;
+    bool out = !(ddx * ddx + ddy * ddy < r2);
+    if (E.sq_dom) {
+        out = out || !(nx > E.d0 && nx < E.d2 && ny > E.d1 && ny < E.d3);
+    } else {
+        const float ex0 = nx - E.d0, ey0 = ny - E.d1;
+        out = out || !(ex0 * ex0 + ey0 * ey0 < E.dr2);
+    }
+    if (fold) {
+        S.Zv = fma(S.Yv, (double)S.z, S.Zv);
+        S.Yv = fma(S.Yv, (double)S.e, S.Yv);
+        S.e = 0.f;
+        S.z = 0.f;
+    }
+    if (!out) {
+        S.x = nx;
+        S.y = ny;
+    }
+    return out;
+}
+
+// the record of a path that left (k_exit32 finds the side and the exit point) or reached the step cap
+template <bool CV>
+__device__ __forceinline__ void record_exit(const PathArgs &A, const Pool32 &Q, long rec, const Path32 &S, float nx,
+                                            float ny, const float *cq) {
+    A.side[rec] = 3;
+    Q.seg[rec] = make_float4(S.x, S.y, nx, ny);
+    A.Y[rec] = S.Yv;
+    A.Z[rec] = S.Zv;
+    A.ez[rec] = make_float2(S.e, S.z);
+    if constexpr (CV) {
+#pragma unroll
+        for (int q = 0; q < kMaxCv; ++q)
+            if (q < A.ncv) A.cvq[rec * A.ncv + q] = (double)cq[q];
+    }
+}
+template <bool CV>
+__device__ __forceinline__ void record_capped(const PathArgs &A, long rec) {
+    A.side[rec] = 2;
+    A.su[rec] = 0.0;
+    A.Y[rec] = 0.0;
+    A.Z[rec] = 0.0;
+    A.ez[rec] = make_float2(0.f, 0.f);
+    if constexpr (CV)
+        for (int q = 0; q < A.ncv; ++q) A.cvq[rec * A.ncv + q] = 0.0;
+}
+
+__device__ __forceinline__ void add_totals(const PathArgs &A, unsigned long long steps, int capped) {
+    for (int o = 16; o; o >>= 1) {
+        steps += __shfl_xor_sync(0xffffffffu, steps, o);
+        capped += __shfl_xor_sync(0xffffffffu, capped, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        if (steps) atomicAdd(A.steps, steps);
+        if (capped) atomicAdd(A.capped, capped);
+    }
+}
+
+// one CTA per row; GAUSS: nc, nf Gaussians of c and f are kept in shared memory (a form of its own: the
+// unused branches alone cost the variable-coefficient paths 4 of 16 ms; 4, 3 and 2 CTAs an SM take 49.0,
+// 48.8 and 51.9 ms on the Gaussians' case)
+template <bool KILL, bool SRC, bool CV, bool GAUSS>
+__global__ void __launch_bounds__(kRowThreads, GAUSS ? 3 : 0) k_paths(Problem P, PathArgs A, int nc, int nf) {
+    extern __shared__ __align__(16) unsigned char psm32[];
+    GaussTab gc{}, gf{};
+    if (GAUSS && KILL && nc) gc = stage_gauss(reinterpret_cast<float4 *>(psm32), P.rbf32, nc, P.rbf_inv2s2);
+    if (GAUSS && SRC && nf)
+        gf = stage_gauss(reinterpret_cast<float4 *>(psm32 + (nc ? gauss_smem(nc) : 0)), P.frbf32, nf, P.frbf_inv2s2);
     using R = float;
     __shared__ int next_path;
     const int slot = blockIdx.x;
@@ -361,9 +640,17 @@ __global__ void __launch_bounds__(256) k_paths(Problem P, PathArgs A) {
             Num<R>::drift(P, x, y, bx, by);
             double Yn = Yv, Zn = Zv;
             float en = e, zn = z;
-            const float cv = KILL ? killing32(P, x, y) : 0.f;
+            float cv = 0.f;
+            if (KILL) {
+                if (GAUSS && nc) {
+                    const float s = gauss_sum(gc, x, y);
+                    cv = s < 0.f ? s : 0.f;
+                } else {
+                    cv = killing32(P, x, y);
+                }
+            }
             // Z_{k+1} = Z_k + f_k h Y_k and Y_{k+1} = Y_k (1 + c_k h), with Y_k = Yv (1 + e)
-            if (SRC) zn = fmaf(source32_given(P, x, y, bx, by, cv) * hf, 1.0f + e, z);
+            if (SRC) zn = fmaf((GAUSS && nf ? gauss_sum(gf, x, y) : source32_given(P, x, y, bx, by, cv)) * hf, 1.0f + e, z);
             if (KILL) en = fmaf(cv * hf, 1.0f + e, e);
             const R nx = x + bx * h + sh * xi0;
             const R ny = y + by * h + sh * xi1;
@@ -494,6 +781,166 @@ __global__ void __launch_bounds__(256) k_paths(Problem P, PathArgs A) {
     }
 }
 
+template <bool KILL, bool SRC, int CVD>
+__global__ void __launch_bounds__(kP32Threads) k_paths_long(Problem P, PathArgs A, Pool32 Q) {
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr bool CV = CVD != 0;
+    extern __shared__ __align__(16) unsigned char psm32[];
+    const Env32 E = env32<KILL, SRC>(P, A, Q, psm32);
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    const unsigned nchunks = (unsigned)((Q.total + kP32Chunk - 1) / kP32Chunk);
+    unsigned long long my_steps = 0;
+    int my_capped = 0;
+    // this warp's records still to start: [q_next, q_end), the first of them in slot q_slot
+    long q_next = 0, q_end = 0;
+    int q_slot = 0;
+    bool drained = false, have = false;
+    long rec = 0;
+    int p = 0, knot = 0, max_steps = 0;
+    uint32_t kw = 0;
+    float cx = 0.f, cy = 0.f, r2 = 0.f, crad = 1.f, rcrad = 1.f;
+    Path32 S{0.f, 0.f, 0.f, 0.f, 1.0, 0.0, 0};
+    float cq[CV ? kMaxCv : 1];
+    unsigned it = 0;           // loop iterations, equal in all lanes
+    for (;;) {
+        // free lanes take the next records, in lane order
+        unsigned idle = __ballot_sync(kAll, !have);
+        while (idle) {
+            if (q_next >= q_end) {
+                if (drained) break;
+                unsigned c = 0;
+                int sl = 0;
+                if (lane == 0) {
+                    c = atomicAdd(Q.next, 1u);
+                    if (c < nchunks) sl = slot_of(A, Q.slots, Q.nslots, (long)c * kP32Chunk);
+                }
+                c = __shfl_sync(kAll, c, 0);
+                q_slot = __shfl_sync(kAll, sl, 0);
+                if (c >= nchunks) {
+                    drained = true;
+                    break;
+                }
+                q_next = (long)c * kP32Chunk;
+                q_end = min(Q.total, q_next + kP32Chunk);
+            }
+            const long g = q_next + __popc(idle & below);
+            if (!have && g < q_end) {
+                int sl = q_slot;
+                while (sl + 1 < Q.nslots && Q.slots[sl + 1].rbase <= g) ++sl;
+                const Slot32 *L = Q.slots + sl;
+                have = true;
+                rec = g;
+                p = (int)(g - L->rbase);
+                S = Path32{L->x0, L->y0, 0.f, 0.f, 1.0, 0.0, 0};
+                cx = L->cx;
+                cy = L->cy;
+                r2 = L->r2;
+                knot = L->i;
+                max_steps = L->max_steps;
+                kw = L->kw;
+                if constexpr (CV) {
+                    crad = L->rad;
+                    rcrad = 1.0f / crad;
+#pragma unroll
+                    for (int q = 0; q < kMaxCv; ++q) cq[q] = 0.f;
+                }
+            }
+            q_next = min(q_end, q_next + __popc(idle));
+            idle = __ballot_sync(kAll, !have);
+        }
+        if (idle == kAll) break;
+        ++it;
+        if (!have) continue;
+        if (S.k >= max_steps) {
+            record_capped<CV>(A, rec);
+            ++my_capped;
+            have = false;
+        } else {
+            float nx, ny;
+            if (step32<KILL, SRC, CVD>(P, A, Q, E, S, knot, kw, p, cx, cy, r2, crad, rcrad, cq, (it & 7) == 0, nx, ny)) {
+                record_exit<CV>(A, Q, rec, S, nx, ny, cq);
+                have = false;
+            }
+        }
+        if (!have) my_steps += (unsigned long long)S.k;
+    }
+    add_totals(A, my_steps, my_capped);
+}
+
+// The exit point of every record's last segment, in FP32: the first crossing with the circle or the
+// domain's boundary (both shrunk by the boundary shift); with the shift the piece crossed first is
+// scored at the projection of the first point outside onto the true boundary
+__global__ void __launch_bounds__(256) k_exit32(Problem P, PathArgs A, Pool32 Q) {
+    const long rec = blockIdx.x * 256L + threadIdx.x;
+    if (rec >= Q.total || A.side[rec] != 3) return;
+    const int slot = slot_of(A, Q.slots, Q.nslots, rec);
+    const Slot32 *S = Q.slots + slot;
+    const bool sq_dom = P.dom_kind == 0;
+    const double sft = A.shift;
+    const float d0 = (float)(sq_dom ? P.dom[0] + sft : P.dom[0]), d1 = (float)(sq_dom ? P.dom[1] + sft : P.dom[1]);
+    const float d2 = (float)(P.dom[2] - sft), d3 = (float)(P.dom[3] - sft);
+    const float dr2 = (float)((P.dom[2] - sft) * (P.dom[2] - sft));
+    const float rcx = S->cx, rcy = S->cy, r2 = S->r2;
+    const float4 s = Q.seg[rec];
+    const float x = s.x, y = s.y, nx = s.z, ny = s.w;
+    const float ddx = nx - rcx, ddy = ny - rcy;
+    const bool out_c = !(ddx * ddx + ddy * ddy < r2);
+    bool out_d;
+    if (sq_dom) {
+        out_d = !(nx > d0 && nx < d2 && ny > d1 && ny < d3);
+    } else {
+        const float ex0 = nx - d0, ey0 = ny - d1;
+        out_d = !(ex0 * ex0 + ey0 * ey0 < dr2);
+    }
+    const float dx = nx - x, dy = ny - y;
+    float tc = 2.f, td = 2.f;
+    int ed = -1;
+    if (out_c) tc = circle_exit_tr<float>(x, y, dx, dy, rcx, rcy, S->rs);
+    if (out_d) {
+        if (sq_dom) {
+            float t;
+            if (nx <= d0) { t = (d0 - x) / dx; if (t < td) { td = t; ed = 3; } }
+            if (nx >= d2) { t = (d2 - x) / dx; if (t < td) { td = t; ed = 1; } }
+            if (ny <= d1) { t = (d1 - y) / dy; if (t < td) { td = t; ed = 0; } }
+            if (ny >= d3) { t = (d3 - y) / dy; if (t < td) { td = t; ed = 2; } }
+        } else {
+            td = circle_exit_tr<float>(x, y, dx, dy, d0, d1, d2);
+            ed = 0;
+        }
+    }
+    const bool proj = A.shift > 0.0;
+    if (td <= tc) {
+        float ex = x + td * dx, ey = y + td * dy;
+        if (proj) {
+            ex = nx;
+            ey = ny;
+            if (sq_dom) {
+                const float x0 = (float)P.dom[0], y0 = (float)P.dom[1], x1 = (float)P.dom[2], y1 = (float)P.dom[3];
+                ex = ex < x0 ? x0 : (ex > x1 ? x1 : ex);
+                ey = ey < y0 ? y0 : (ey > y1 ? y1 : ey);
+                if (ed == 0) ey = y0;
+                else if (ed == 1) ex = x1;
+                else if (ed == 2) ey = y1;
+                else ex = x0;
+            }                                             // disk domain: the arclength is the angle's
+        }
+        A.side[rec] = 1;
+        A.su[rec] = boundary_s(P, (double)ex, (double)ey, ed);
+    } else {
+        const float ex = proj ? nx : x + tc * dx, ey = proj ? ny : y + tc * dy;
+        float th = atan2f(ey - rcy, ex - rcx);
+        const float two_pi = (float)PDD_TWO_PI;
+        if (th < 0.f) th += two_pi;
+        float u = th - S->ts;
+        if (u < 0.f) u += two_pi;
+        if (u >= two_pi) u -= two_pi;
+        A.side[rec] = 0;
+        A.su[rec] = (double)u;
+    }
+}
+
 // ---------------------------------------------------------------------------
 // FP64 form.  The FP64 pipe bounds it (1/64 of the FP32 rate: a warp instruction occupies an SM's
 // unit for 16 cycles whatever the number of its lanes in use), so the design keeps the lanes full
@@ -559,18 +1006,6 @@ __global__ void k_slots64(int n, PathArgs A, Slot64 *out) {
     s.max_steps = A.max_steps > 0 ? A.max_steps : (int)fmin(2147483647.0, ceil(50.0 * rad * rad / A.h));
     s.kw = A.kword ? (uint32_t)A.kword[gsl] : 0u;
     out[slot] = s;
-}
-
-// the slot of record g (the records of the slots are contiguous and in slot order)
-__device__ __forceinline__ int slot_of(const PathArgs &A, const Slot64 *slots, int nslots, unsigned long long g) {
-    if (!A.rec_off) return (int)((unsigned)g / (unsigned)A.paths);      // at most 2^31 records per launch
-    int lo = 0, hi = nslots - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if ((unsigned long long)slots[mid].rbase <= g) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
 }
 
 // an order-preserving integer of a double (-0 below +0; no NaN)
@@ -640,7 +1075,7 @@ __global__ void __launch_bounds__(kP64Threads) k_paths64(Problem P, PathArgs A, 
                     Yv = s.Y;
                     Zv = s.Z;
                 } else {
-                    slot = slot_of(A, Q.slots, Q.nslots, g);
+                    slot = slot_of(A, Q.slots, Q.nslots, (long)g);
                     p = (int)(g - (unsigned long long)Q.slots[slot].rbase);
                     k = 0;
                     x = Q.slots[slot].x0;
@@ -763,7 +1198,7 @@ __global__ void __launch_bounds__(kP64Threads) k_paths64(Problem P, PathArgs A, 
 __global__ void __launch_bounds__(256) k_exit64(Problem P, PathArgs A, PathPool Q) {
     const unsigned long long rec = blockIdx.x * 256ULL + threadIdx.x;
     if (rec >= Q.total || A.side[rec] != 3) return;
-    const int slot = slot_of(A, Q.slots, Q.nslots, rec);
+    const int slot = slot_of(A, Q.slots, Q.nslots, (long)rec);
     const int m = A.subs[A.gslot ? A.gslot[slot] : slot];
     const bool sq_dom = P.dom_kind == 0;
     const double sft = A.shift;
@@ -1473,18 +1908,59 @@ __global__ void k_need(int nmc, const int *rows, const int *subs, const int *spo
     need[slot] = w > Pmax ? Pmax : w;
 }
 
+// buffers of the mixed form, kept over the waves of one assembly
+struct Paths32Bufs {
+    DevBuf<Slot32> slots;
+    DevBuf<float4> seg;
+    DevBuf<unsigned> next;
+};
+
+template <int CVD>
+static const void *paths_long_kernel(bool kill, bool src) {
+    return kill ? (src ? (const void *)k_paths_long<true, true, CVD> : (const void *)k_paths_long<true, false, CVD>)
+                : (src ? (const void *)k_paths_long<false, true, CVD> : (const void *)k_paths_long<false, false, CVD>);
+}
 template <bool CV>
-static void launch_paths_cv(const Problem &P, const PathArgs &A, int nrows, cudaStream_t st) {
+static void launch_paths(const Problem &P, const PathArgs &A, int nrows, int nc, int nf, size_t sm, cudaStream_t st) {
     const bool kill = P.c_kind != PDD_C_ZERO, src = P.f_kind != PDD_F_ZERO;
-    if (kill && src) PDD_LAUNCH((k_paths<true, true, CV>), nrows, 256, 0, st, P, A);
-    else if (kill) PDD_LAUNCH((k_paths<true, false, CV>), nrows, 256, 0, st, P, A);
-    else if (src) PDD_LAUNCH((k_paths<false, true, CV>), nrows, 256, 0, st, P, A);
-    else PDD_LAUNCH((k_paths<false, false, CV>), nrows, 256, 0, st, P, A);
+    auto kern = kill ? (src ? k_paths<true, true, CV, false> : k_paths<true, false, CV, false>)
+                     : (src ? k_paths<false, true, CV, false> : k_paths<false, false, CV, false>);
+    if (nc || nf)
+        kern = kill ? (src ? k_paths<true, true, CV, true> : k_paths<true, false, CV, true>) : k_paths<false, true, CV, true>;
+    PDD_LAUNCH(kern, nrows, kRowThreads, sm, st, P, A, nc, nf);
 }
 
-static void launch_paths(const Problem &P, const PathArgs &A, int nrows, cudaStream_t st) {
-    if (A.cvd > 0) launch_paths_cv<true>(P, A, nrows, st);
-    else launch_paths_cv<false>(P, A, nrows, st);
+// nrows slots with `total` paths in all, their records contiguous in slot order
+static void run_paths32(const Problem &P, const PathArgs &A, int nrows, long total, double max_r, Paths32Bufs &B,
+                        cudaStream_t st) {
+    const int nc = P.c_kind == PDD_C_RBF && P.n_rbf <= kP32Staged ? P.n_rbf : 0;
+    const int nf = P.f_kind == PDD_F_RBF && P.n_frbf <= kP32Staged ? P.n_frbf : 0;
+    const size_t sm = (nc ? gauss_smem(nc) : 0) + (nf ? gauss_smem(nf) : 0);
+    if (max_r * max_r / (4.0 * A.h) < kLongSteps) {        // mean steps of a path of the largest circle
+        if (A.cvd > 0) launch_paths<true>(P, A, nrows, nc, nf, sm, st);
+        else launch_paths<false>(P, A, nrows, nc, nf, sm, st);
+        return;
+    }
+    int dev = 0, sms = 0, per_sm = 0;
+    PDD_CUDA(cudaGetDevice(&dev));
+    PDD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    if (B.slots.n < (size_t)nrows) B.slots.alloc(nrows);
+    if (B.seg.n < (size_t)total) B.seg.alloc(total);
+    if (!B.next.n) B.next.alloc(1);
+    PDD_CUDA(cudaMemsetAsync(B.next.p, 0, sizeof(unsigned), st));
+    PDD_LAUNCH(k_slots32, cdiv(nrows, 128), 128, 0, st, nrows, A, B.slots.p);
+    Pool32 Q{B.slots.p, nrows, total, B.next.p, B.seg.p, nc, nf};
+    const bool kill = P.c_kind != PDD_C_ZERO, src = P.f_kind != PDD_F_ZERO;
+    const void *kern = A.cvd == 0 ? paths_long_kernel<0>(kill, src)
+                                  : (A.cvd == 4 ? paths_long_kernel<4>(kill, src) : paths_long_kernel<-1>(kill, src));
+    PDD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kP32Threads, sm));
+    const int grid = (int)std::max<long>(1, std::min<long>((long)sms * std::max(per_sm, 1), cdiv(total, kP32Threads)));
+    Problem Pv = P;
+    PathArgs Av = A;
+    void *args[] = {&Pv, &Av, &Q};
+    PDD_CUDA(cudaLaunchKernel(kern, dim3(grid), dim3(kP32Threads), args, sm, st));
+    count_launch();
+    PDD_LAUNCH(k_exit32, cdiv(total, 256), 256, 0, st, P, A, Q);
 }
 
 // buffers of the FP64 form's passes, kept over the waves of one assembly
@@ -1587,7 +2063,8 @@ McStats assemble_mc(const pdd_cover &cov, const Problem &P, const pdd_assembly_o
     const int cvd = o.cv_degree, ncv = cvd * (cvd + 3) / 2;          // control-variate features per path
     const int cv_stride = cov.max_stencil + 1;
     const size_t rec_bytes =
-        1 + 3 * sizeof(double) + (mixed ? sizeof(float2) : sizeof(Seg64)) + (size_t)ncv * sizeof(double);
+        1 + 3 * sizeof(double) + (mixed ? sizeof(float2) + sizeof(float4) : sizeof(Seg64)) +
+        (size_t)ncv * sizeof(double);
     const size_t per_row = (size_t)P_ * rec_bytes;
     const int wave = (int)std::max<size_t>(1, std::min<size_t>(nmc, ((size_t)8 << 30) / per_row));
     DevBuf<int8_t> side;
@@ -1622,6 +2099,7 @@ McStats assemble_mc(const pdd_cover &cov, const Problem &P, const pdd_assembly_o
     // per-slot arrays (subs, spos, kword, momp, bmean) are indexed like the global slot gs: offset to
     // the wave's first slot when gsl is null, or the whole arrays with gsl
     Paths64Bufs p64;
+    Paths32Bufs p32;
     auto run_wave = [&](const int *rows, int nr, long nrec, const int *np, const long *roff, const int *gsl,
                         const int *momp, double *bmean, size_t w0) {
         const int *subs = sys.mc_subs.p + w0, *spos = sys.mc_spos.p + w0, *kword = sys.mc_kword.p + w0;
@@ -1629,7 +2107,7 @@ McStats assemble_mc(const pdd_cover &cov, const Problem &P, const pdd_assembly_o
                    cov.theta_s.p, o.paths, o.h, o.seed, side.p, su.p, Y.p, Z.p, steps.p, capped.p, np, roff, ez.p,
                    o.boundary_shift ? kGmC0 * sqrt(o.h) : 0.0, gsl, o.max_steps, cvd, ncv, cvq.p};
         PDD_CUDA(cudaEventRecord(e0, st));
-        if (mixed) launch_paths(P, A, nr, st);
+        if (mixed) run_paths32(P, A, nr, nrec, cov.max_r, p32, st);
         else run_paths64(P, A, nr, nrec, p64, st);
         PDD_CUDA(cudaEventRecord(e1, st));
         FinalArgs F{rows, subs, spos, cov.sub_off.p, cov.knot_ptr.p, cov.rowptr.p, cov.floating.p,
