@@ -304,6 +304,25 @@ __device__ __forceinline__ float2 df_split(double v) {
     return make_float2(h, (float)(v - (double)h));
 }
 
+// v = hi + lo with hi = v truncated to 24 significant bits and lo the rest rounded to FP32, built
+// from the bit fields by integer operations (the FP64 pipe of this part is 1/64 of the FP32 rate).
+// |v| < 2^-126 gives (0, 0) and |v| < 2^-74 drops lo (relative error up to 2^-23 there); above
+// that the split is within 2^-47 relative (an emulation over 2e4 values per decade); the Monte Carlo
+// weights and exit angles are far from either.
+__device__ __forceinline__ float2 split_df_bits(double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
+    const int e = (int)((b >> 52) & 0x7FF);
+    const int eh = e - 896;                                 // FP32 biased exponent of hi
+    if (eh >= 255) return make_float2((float)v, 0.f);       // beyond FP32 range (not reached)
+    if (eh <= 0) return make_float2(__uint_as_float(sign), 0.f);
+    const float hi = __uint_as_float(sign | ((unsigned)eh << 23) | (unsigned)((b >> 29) & 0x7FFFFFu));
+    const int el = e - 948;                                 // FP32 biased exponent of 2^(e - 1075)
+    float lo = 0.f;
+    if (el > 0) lo = __fmul_rn(__uint2float_rn((unsigned)(b & 0x1FFFFFFFull)), __uint_as_float((unsigned)el << 23));
+    return make_float2(hi, __uint_as_float(__float_as_uint(lo) | sign));
+}
+
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     s = a + b;
     const float bb = s - a;

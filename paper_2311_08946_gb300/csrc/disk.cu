@@ -40,6 +40,9 @@ struct Shape {
     double *x, *D, *D2, *F1, *F2, *Hg;   // device tables
     float2 *Dhl, *D2hl, *F1hl, *F2hl;    // the same tables as FP32 (hi, lo) pairs
     float2 *Hghl;
+    // without drift: the operator over the angle pairs (j, j + nt/2), see k_residual_sym
+    double *SE, *SO, *RA, *RB, *RG;
+    float2 *SEhl, *SOhl, *RAhl, *RBhl, *RGhl;
 };
 
 struct DiskDesc {
@@ -104,6 +107,28 @@ __global__ void k_matmul_sq(const double *A, double *C, int np) {
     double s = 0.0;
     for (int k = 0; k < np; ++k) s += A[i * np + k] * A[k * np + j];
     C[idx] = s;
+}
+
+// SE/SO[l][k] = half the sum / difference of the weights that the node's own line and its mirror give
+// ring l at ring k, over alpha; RA/RB[delta + nt/2] the same of the ring's weights of the angles at
+// distance delta and delta + nt/2, over gamma; RG[k] = gamma / alpha
+__global__ void k_shape_sym(int nr, int nt, const double *x, const double *D, const double *D2, const double *F2,
+                            double *SE, double *SO, double *RA, double *RB, double *RG) {
+    const int nc = 2 * nr + 1, np = nc + 1, half = nt / 2;
+    const int id = blockIdx.x * blockDim.x + threadIdx.x;
+    if (id < nr * nr) {
+        const int l = id / nr + 1, k = id % nr + 1;
+        const double w = D2[k * np + l] + D[k * np + l] / x[k], wm = D2[k * np + nc - l] + D[k * np + nc - l] / x[k];
+        SE[id] = 0.5 * (w + wm);
+        SO[id] = 0.5 * (w - wm);
+    }
+    if (id < nr) RG[id] = 1.0 / (x[id + 1] * x[id + 1]);
+    if (id < nt) {
+        const int d = id - half;
+        const double a = F2[(d + nt) % nt], b = F2[(d + half + nt) % nt];
+        RA[id] = 0.5 * (a + b);
+        RB[id] = 0.5 * (a - b);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1218,6 +1243,168 @@ __global__ void __launch_bounds__(256) k_residual_df(Shape S, const NodeCoef *co
     }
 }
 
+// The same residuals where the operator has no drift (its coefficients then depend on the ring alone,
+// but for c).  With e = u_j + u_{j+nt/2} and o = u_j - u_{j+nt/2} the radial lines of a pair of nodes and
+// their mirrors, and the ring, each split into a part on e and a part on o, which the two nodes add and
+// subtract: half the products, and the weights are tables of the grid shape.  A block takes a disk and up
+// to four columns, e and o of which it keeps in shared memory; a warp takes 32 (column, angle) pairs and
+// eight rings, so that a loaded weight or value feeds eight sums (the node-by-node form loads two
+// operands a product).  The FP64 form is bound by the FP64 pipe, the double-float one by issue.
+// 600 disks of 48 x 64 nodes, 17 columns: FP64 9.6 -> 4.9 ms, double-float 4.5 -> 1.4 ms.
+struct SymF64 {
+    using T = double;
+    __device__ static T zero() { return 0.0; }
+    __device__ static void acc(T &a, T w, T x) { a = fma(w, x, a); }
+    __device__ static T sum(T a) { return a; }
+    __device__ static T add(T a, T b) { return a + b; }
+    __device__ static T sub(T a, T b) { return a - b; }
+    __device__ static T mul(T a, T b) { return a * b; }
+    __device__ static T from(double v) { return v; }
+};
+struct SymDf {
+    using T = float2;
+    __device__ static T zero() { return make_float2(0.f, 0.f); }
+    __device__ static void acc(T &a, T w, T x) { df_acc(a.x, a.y, w, x); }
+    __device__ static T sum(T a) {                        // the unnormalised accumulator
+        const float h = a.x + a.y;
+        return make_float2(h, a.y - (h - a.x));
+    }
+    __device__ static T add(T a, T b) { return df_add(a, b); }
+    __device__ static T sub(T a, T b) { return df_add(a, make_float2(-b.x, -b.y)); }
+    __device__ static T mul(T a, T b) { return df_mul(a, b); }
+    __device__ static T from(double v) { return df_split(v); }
+};
+static constexpr int kSymThreads = 384, kSymK = 8;
+
+template <typename T>
+static size_t sym_smem(const Shape &S, int cg) {
+    const size_t nrp = (S.nr + kSymK - 1) / kSymK * kSymK;
+    return sizeof(T) * ((size_t)S.n * cg + 2 * (size_t)S.nr * nrp + 2 * S.nt);
+}
+
+// DF: R = R1 - A D (rounded to FP32) from the double-float pairs R1, D; else R = RHS - A X and R1 its split
+template <bool DF>
+__global__ void __launch_bounds__(kSymThreads, 1) k_residual_sym(Shape S, const NodeCoef *coefAll, long strideC,
+                                                              const double *RHSall, const double *Xall,
+                                                              const float2 *Dall, double *Rall, float2 *R1all,
+                                                              long strideR, const int *conv, int cgmax) {
+    using Pol = typename std::conditional<DF, SymDf, SymF64>::type;
+    using T = typename Pol::T;
+    const int disk = blockIdx.y;
+    if (conv[disk]) return;
+    extern __shared__ __align__(16) double ysm[];
+    const int c0 = blockIdx.x * cgmax, cg = min(cgmax, S.nrhs - c0);
+    const int nr = S.nr, nt = S.nt, half = nt >> 1, n = S.n, nrp = (nr + kSymK - 1) / kSymK * kSymK;
+    T *eo = reinterpret_cast<T *>(ysm);                   // [column][ring][e of half angles, o of half angles]
+    T *we = eo + (size_t)n * cgmax, *wo = we + (size_t)nr * nrp, *ra = wo + (size_t)nr * nrp, *rb = ra + nt;
+    const T *gse, *gso, *gra, *grb, *grg, *U;
+    if constexpr (DF) {
+        gse = S.SEhl;
+        gso = S.SOhl;
+        gra = S.RAhl;
+        grb = S.RBhl;
+        grg = S.RGhl;
+        U = Dall + disk * strideR;
+    } else {
+        gse = S.SE;
+        gso = S.SO;
+        gra = S.RA;
+        grb = S.RB;
+        grg = S.RG;
+        U = Xall + disk * strideR;
+    }
+    for (int q = threadIdx.x; q < nr * nrp; q += blockDim.x) {
+        const int l = q / nrp, k = q - l * nrp;
+        we[q] = k < nr ? gse[l * nr + k] : Pol::zero();
+        wo[q] = k < nr ? gso[l * nr + k] : Pol::zero();
+    }
+    for (int q = threadIdx.x; q < nt; q += blockDim.x) {
+        ra[q] = gra[q];
+        rb[q] = grb[q];
+    }
+    for (int q = threadIdx.x; q < (n >> 1) * cg; q += blockDim.x) {
+        const int pr = q / cg, c = q - pr * cg, l = pr / half, j = pr - l * half;
+        const T u = U[(long)(l * nt + j) * S.nrhs + c0 + c], v = U[(long)(l * nt + j + half) * S.nrhs + c0 + c];
+        T *row = eo + (size_t)c * n + l * nt;
+        row[j] = Pol::add(u, v);
+        row[half + j] = Pol::sub(u, v);
+    }
+    __syncthreads();
+    const T al = Pol::from(coefAll[disk * strideC].alpha);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int items = cg * half, its = (items + 31) >> 5, kbs = nrp / kSymK, units = kbs * its;
+    for (int un = warp; un < units; un += blockDim.x >> 5) {
+        const int it = (un % its) * 32 + lane, ic = min(it, items - 1), c = ic / half, jc = ic - c * half;
+        const int k0 = un / its * kSymK;
+        const T *col = eo + (size_t)c * n;
+        T ae[kSymK], ao[kSymK];
+#pragma unroll
+        for (int q = 0; q < kSymK; ++q) ae[q] = ao[q] = Pol::zero();
+        // the ring, over gamma
+        for (int jp = 0; jp < half; ++jp) {
+            const T wa = ra[jc - jp + half], wb = rb[jc - jp + half];
+#pragma unroll
+            for (int q = 0; q < kSymK; ++q) {
+                const T *row = col + min(k0 + q, nr - 1) * nt + jp;
+                Pol::acc(ae[q], wa, row[0]);
+                Pol::acc(ao[q], wb, row[half]);
+            }
+        }
+        // gamma / alpha = 1 / rho^2 onto the radial sums
+#pragma unroll
+        for (int q = 0; q < kSymK; ++q) {
+            const T g = grg[min(k0 + q, nr - 1)];
+            ae[q] = Pol::mul(Pol::sum(ae[q]), g);
+            ao[q] = Pol::mul(Pol::sum(ao[q]), g);
+        }
+        for (int l = 0; l < nr; ++l) {
+            const T e = col[l * nt + jc], o = col[l * nt + half + jc];
+            const T *pe = we + l * nrp + k0, *po = wo + l * nrp + k0;
+#pragma unroll
+            for (int q = 0; q < kSymK; ++q) {
+                Pol::acc(ae[q], pe[q], e);
+                Pol::acc(ao[q], po[q], o);
+            }
+        }
+        if (it >= items) continue;
+#pragma unroll
+        for (int q = 0; q < kSymK; ++q) {
+            if (k0 + q >= nr) continue;
+            const T E = Pol::sum(ae[q]), O = Pol::sum(ao[q]);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int p = (k0 + q) * nt + jc + h * half;
+                const NodeCoef cf = coefAll[disk * strideC + p];
+                const long o = (long)p * S.nrhs + c0 + c;
+                const T t = h ? Pol::sub(E, O) : Pol::add(E, O);
+                if constexpr (DF) {
+                    const float2 au = df_add(df_mul(al, t), df_mul(split_df_bits(cf.c), U[o]));
+                    const float2 v = df_mul(split_df_bits(cf.s), au);
+                    Rall[disk * strideR + o] = (double)df_add(R1all[disk * strideR + o], make_float2(-v.x, -v.y)).x;
+                } else {
+                    const double r = RHSall[disk * strideR + o] - cf.s * (al * t + cf.c * U[o]);
+                    Rall[disk * strideR + o] = r;
+                    if (R1all) R1all[disk * strideR + o] = df_split(r);
+                }
+            }
+        }
+    }
+}
+
+// threads of a block: twelve warps, fewer where its units of work leave some of them idle
+static int sym_threads(const Shape &S, int cg) {
+    const int units = cdiv(S.nr, kSymK) * cdiv(cg * (S.nt / 2), 32), rounds = cdiv(units, kSymThreads / 32);
+    return 32 * cdiv(units, rounds);
+}
+
+// columns of a block: as many as fit (four at most), 0 when not one does
+template <typename T>
+static int sym_columns(const Shape &S) {
+    for (int cg = 4; cg >= 1; --cg)
+        if (sym_smem<T>(S, cg) <= (size_t)220 * 1024) return std::min(cg, S.nrhs);
+    return 0;
+}
+
 // ---------------------------------------------------------------------------
 // a9: evaluate at the disk's knots and scatter into C and r
 // ---------------------------------------------------------------------------
@@ -1400,6 +1587,8 @@ __global__ void __launch_bounds__(256) k_disk_eval_df(Shape S, const DiskDesc *d
 struct ShapeTables {
     DevBuf<double> x, D, D2, F1, F2, Hg;
     DevBuf<float2> Dhl, D2hl, F1hl, F2hl, Hghl;
+    DevBuf<double> SE, SO, RA, RB, RG;
+    DevBuf<float2> SEhl, SOhl, RAhl, RBhl, RGhl;
     Shape S{};
     void build(int nr, int nt, int nk, cudaStream_t st) {
         const int nc = 2 * nr + 1, np = nc + 1;
@@ -1422,8 +1611,27 @@ struct ShapeTables {
         PDD_LAUNCH(k_split_df, cdiv(nt, 256), 256, 0, st, F2.p, F2hl.p, nt);
         Hghl.alloc((size_t)nt * nk);
         PDD_LAUNCH(k_split_df, cdiv(nt * nk, 256), 256, 0, st, Hg.p, Hghl.p, nt * nk);
+        const int ns = nr * nr;
+        SE.alloc(ns);
+        SO.alloc(ns);
+        RA.alloc(nt);
+        RB.alloc(nt);
+        SEhl.alloc(ns);
+        SOhl.alloc(ns);
+        RAhl.alloc(nt);
+        RBhl.alloc(nt);
+        RG.alloc(nr);
+        RGhl.alloc(nr);
+        PDD_LAUNCH(k_shape_sym, cdiv(std::max(ns, nt), 256), 256, 0, st, nr, nt, x.p, D.p, D2.p, F2.p, SE.p, SO.p, RA.p,
+                   RB.p, RG.p);
+        PDD_LAUNCH(k_split_df, cdiv(ns, 256), 256, 0, st, SE.p, SEhl.p, ns);
+        PDD_LAUNCH(k_split_df, cdiv(ns, 256), 256, 0, st, SO.p, SOhl.p, ns);
+        PDD_LAUNCH(k_split_df, cdiv(nt, 256), 256, 0, st, RA.p, RAhl.p, nt);
+        PDD_LAUNCH(k_split_df, cdiv(nt, 256), 256, 0, st, RB.p, RBhl.p, nt);
+        PDD_LAUNCH(k_split_df, cdiv(nr, 256), 256, 0, st, RG.p, RGhl.p, nr);
         S = Shape{nr, nt, nk, nc, nr * nt, nk + 1, x.p, D.p, D2.p, F1.p, F2.p, Hg.p,
-                  Dhl.p, D2hl.p, F1hl.p, F2hl.p, Hghl.p};
+                  Dhl.p, D2hl.p, F1hl.p, F2hl.p, Hghl.p,
+                  SE.p, SO.p, RA.p, RB.p, RG.p, SEhl.p, SOhl.p, RAhl.p, RBhl.p, RGhl.p};
     }
 };
 
@@ -1683,6 +1891,22 @@ static DiskStats run_group(const pdd_cover &cov, const Problem &P, const pdd_ass
             PDD_CUDA(cudaFuncSetAttribute(k_residual, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm));
             PDD_CUDA(cudaFuncSetAttribute(k_residual_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm_df));
             dim3 g_res(cdiv(S.n, kResNP), nd), g_res_df(cdiv(S.n, kResNPdf), nd);
+            // without drift, the forms over angle pairs (nd <= 65535 is the grid's limit for both)
+            const int cg1 = P.b_kind == PDD_B_ZERO ? sym_columns<double>(S) : 0;
+            const size_t sm1 = cg1 ? sym_smem<double>(S, cg1) : 0;
+            if (cg1) {
+                PDD_CUDA(cudaFuncSetAttribute(k_residual_sym<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1));
+                PDD_CUDA(cudaFuncSetAttribute(k_residual_sym<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1));
+            }
+            const int th1 = cg1 ? sym_threads(S, cg1) : 32;
+            const dim3 g_sym(cg1 ? cdiv(S.nrhs, cg1) : 1, nd);
+            auto first_residual = [&](float2 *r1) {
+                if (cg1)
+                    PDD_LAUNCH(k_residual_sym<false>, g_sym, th1, sm1, st, S, coef.p, sC, RHS.p, X.p, nullptr,
+                               Rr.p, r1, sR, conv.p, cg1);
+                else
+                    PDD_LAUNCH(k_residual, g_res, 256, rsm, st, S, coef.p, sC, RHS.p, X.p, Rr.p, sR, conv.p, r1);
+            };
             std::vector<cudaEvent_t> sev(rlW ? 2 * maxs : 0);
             for (cudaEvent_t &e : sev) PDD_CUDA(cudaEventCreate(&e));
             struct EvFree {
@@ -1708,8 +1932,10 @@ static DiskStats run_group(const pdd_cover &cov, const Problem &P, const pdd_ass
                                tol);
                     if (s + 1 < maxs) {
                         if (s == 0)
-                            PDD_LAUNCH(k_residual, g_res, 256, rsm, st, S, coef.p, sC, RHS.p, X.p, Rr.p, sR, conv.p,
-                                       R1hl.p);
+                            first_residual(R1hl.p);
+                        else if (cg1)
+                            PDD_LAUNCH(k_residual_sym<true>, g_sym, th1, sm1, st, S, coef.p, sC, nullptr, nullptr,
+                                       Dhl.p, Rr.p, R1hl.p, sR, conv.p, cg1);
                         else
                             PDD_LAUNCH(k_residual_df, g_res_df, 256, rsm_df, st, S, coef.p, sC, R1hl.p, Dhl.p, Rr.p, sR,
                                        conv.p);
@@ -1717,9 +1943,7 @@ static DiskStats run_group(const pdd_cover &cov, const Problem &P, const pdd_ass
                 } else {
                     launch_solve<T>(A.p, S.n, sA, perm.p, rhs_now, S.nrhs, sR, W.p, X.p, 1, conv.p, sweeps.p, tol,
                                     nd, st);
-                    if (s + 1 < maxs)
-                        PDD_LAUNCH(k_residual, g_res, 256, rsm, st, S, coef.p, sC, RHS.p, X.p, Rr.p, sR, conv.p,
-                                   (float2 *)nullptr);
+                    if (s + 1 < maxs) first_residual(nullptr);
                 }
             }
             tm.mark(3);
