@@ -620,7 +620,7 @@ static void launch_solve(const T *LU, int n, long sA, const int *perm, const dou
 // solve, and the row updates are independent FP32 FMA chains (broadcast
 // shared-memory reads of the solved panel rows).
 // ---------------------------------------------------------------------------
-static constexpr int kRlTB = 32, kRlThreads = 512;
+static constexpr int kRlTB = 32, kRlThreads = 512, kRlNarrow = 256;
 static constexpr size_t kRlSmemMax = 225 * 1024;        // 227 KB per CTA, less the static arrays
 
 // inverses of the unit-lower and upper 32x32 diagonal blocks of each LU:
@@ -686,15 +686,17 @@ static size_t rl_smem_bytes(int n, int CG) {
 
 // X += inv(LU) P R for the columns [blockIdx.y CG, ...) of every disk not yet
 // converged; the largest |correction| and |X| of each disk go to dmaxb/xmaxb
-// (bit patterns of non-negative doubles, ordered like the values)
-template <int CG>
-__global__ void __launch_bounds__(kRlThreads, 1) k_lu_solve_rl(const float *LUTall, int n, long strideA,
+// (bit patterns of non-negative doubles, ordered like the values).  NT = 512 threads, or 256 for small
+// disks, where two CTAs share an SM and work while the other waits at a panel's barriers; blocks of one
+// disk's column groups are neighbours, so that the factors come from L2 for all but the first
+template <int CG, int NT>
+__global__ void __launch_bounds__(NT, kRlThreads / NT) k_lu_solve_rl(const float *LUTall, int n, long strideA,
                                                                const int *permAll, const float *DinvAll,
                                                                const double *Rall, int nrhs, long strideR,
                                                                double *Xall, const int *conv,
                                                                unsigned long long *dmaxb, unsigned long long *xmaxb,
-                                                               float2 *Dall, int dmode) {
-    constexpr int NT = kRlThreads, TB = kRlTB;
+                                                               float2 *Dall, int dmode, int groups) {
+    constexpr int TB = kRlTB, HN = (TB * TB + NT - 1) / NT;
     constexpr bool VEC = (CG % 4) == 0;                // 16-byte shared-memory access to the columns
     constexpr int PD = (CG <= 20) ? 32 : (CG <= 36 ? 8 : 2);   // factor entries per row in flight
     constexpr int CGP = rl_cgp(CG);
@@ -703,9 +705,10 @@ __global__ void __launch_bounds__(kRlThreads, 1) k_lu_solve_rl(const float *LUTa
     float *Xp = rsm;                                   // TB x CGP: the panel's solved rows, 16-byte rows
     float *Ds = Xp + TB * CGP;                         // TB x (TB + 1) diagonal-block inverse (padded rows)
     float *Bs = Ds + TB * (TB + 1);                    // n x CG: right-hand sides, then solutions
-    const int disk = blockIdx.x, tid = threadIdx.x;
+    constexpr bool NARROW = NT != kRlThreads;          // grid: disk x group, else (disk, group)
+    const int disk = NARROW ? blockIdx.x / groups : blockIdx.x, tid = threadIdx.x;
     if (conv[disk]) return;
-    const int c0 = blockIdx.y * CG, cg = min(CG, nrhs - c0);
+    const int c0 = (NARROW ? blockIdx.x - disk * groups : blockIdx.y) * CG, cg = min(CG, nrhs - c0);
     const float *LUT = LUTall + disk * strideA;      // the factors transposed
     const int *perm = permAll + (long)disk * n;
     const double *R = Rall + disk * strideR;
@@ -717,11 +720,10 @@ __global__ void __launch_bounds__(kRlThreads, 1) k_lu_solve_rl(const float *LUTa
         Bs[e] = (c < cg) ? (float)R[(long)perm[p] * nrhs + c0 + c] : 0.f;
     }
     for (int e = tid; e < TB * CGP; e += NT) Xp[e] = 0.f;
-    // each panel's diagonal-block inverse is loaded into registers one panel ahead (NT >= TB TB / 2)
-    static_assert(2 * NT >= TB * TB, "two inverse entries per thread");
-    float dnext[2];
+    // each panel's diagonal-block inverse is loaded into registers one panel ahead
+    float dnext[HN];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < HN; ++h) {
         const int e = tid + h * NT;
         dnext[h] = e < TB * TB ? Dv[e] : 0.f;                       // pass 0, block 0
     }
@@ -736,7 +738,7 @@ __global__ void __launch_bounds__(kRlThreads, 1) k_lu_solve_rl(const float *LUTa
             // memory and the panel's right-hand sides are read as broadcasts
             const int warp = tid >> 5, lane = tid & 31;
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
+            for (int h = 0; h < HN; ++h) {
                 const int e = tid + h * NT;
                 if (e < TB * TB) Ds[(e >> 5) * (TB + 1) + (e & 31)] = dnext[h];
             }
@@ -745,11 +747,12 @@ __global__ void __launch_bounds__(kRlThreads, 1) k_lu_solve_rl(const float *LUTa
                 const int npass = last_l ? 1 : pass;
                 const int nblk_i = last_l ? nblk - 1 : (pass == 0 ? blk + 1 : blk - 1);
                 if (npass == 1 && nblk_i < 0) {
-                    dnext[0] = dnext[1] = 0.f;
+#pragma unroll
+                    for (int h = 0; h < HN; ++h) dnext[h] = 0.f;
                 } else {
                     const float *Dn = Dv + ((long)nblk_i * 2 + npass) * (TB * TB);
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
+                    for (int h = 0; h < HN; ++h) {
                         const int e = tid + h * NT;
                         if (e < TB * TB) dnext[h] = Dn[e];
                     }
@@ -1004,9 +1007,19 @@ __global__ void k_refine_conv(int nd, int *conv, int *sweeps, unsigned long long
 }
 
 // column-group width of the right-looking solve for n rows and nrhs columns
-// (0: the shared-memory block does not fit; the tiled solve is used)
-static int rl_width(int n, int nrhs, int &groups) {
+// (0: the shared-memory block does not fit; the tiled solve is used).  narrow: groups of 17 columns at
+// most, two CTAs of 256 threads an SM, where both blocks fit (n <= 1,500): 864 disks of n = 1,024 with 33
+// columns take 0.71 ms a solve so and 0.94 in one group of 36
+static int rl_width(int n, int nrhs, int &groups, bool &narrow) {
     static const int widths[] = {8, 12, 17, 20, 36, 52};     // 17: all 17 columns of 16-knot disks at n = 3072
+    const int few = (nrhs + 16) / 17, cgn = (nrhs + few - 1) / few;
+    for (int w : {8, 12, 17})
+        if (w >= cgn && rl_smem_bytes(n, w) <= kRlSmemMax / 2 - 1024) {
+            narrow = true;
+            groups = (nrhs + w - 1) / w;
+            return w;
+        }
+    narrow = false;
     for (int g = 1; g <= nrhs; ++g) {
         const int cg = (nrhs + g - 1) / g;
         int W = 0;
@@ -1043,15 +1056,22 @@ struct RlArgs {
     int dmode, nd, groups;
 };
 
-template <int CG>
+template <int CG, int NT = kRlThreads>
 static void launch_rl_cg(const RlArgs &a, cudaStream_t st) {
     const size_t sm = rl_smem_bytes(a.n, CG);
-    PDD_CUDA(cudaFuncSetAttribute(k_lu_solve_rl<CG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    PDD_LAUNCH(k_lu_solve_rl<CG>, dim3(a.nd, a.groups), kRlThreads, sm, st, a.LU, a.n, a.sA, a.perm, a.Dinv, a.R,
-               a.nrhs, a.sR, a.X, a.conv, a.dmb, a.xmb, a.D, a.dmode);
+    auto kern = k_lu_solve_rl<CG, NT>;
+    PDD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    PDD_LAUNCH(kern, NT == kRlThreads ? dim3(a.nd, a.groups) : dim3(a.nd * a.groups), NT, sm, st, a.LU, a.n, a.sA, a.perm, a.Dinv, a.R, a.nrhs, a.sR, a.X, a.conv,
+               a.dmb, a.xmb, a.D, a.dmode, a.groups);
 }
 
-static void launch_rl(int W, const RlArgs &a, cudaStream_t st) {
+static void launch_rl(int W, bool narrow, const RlArgs &a, cudaStream_t st) {
+    if (narrow) {
+        if (W == 8) launch_rl_cg<8, kRlNarrow>(a, st);
+        else if (W == 12) launch_rl_cg<12, kRlNarrow>(a, st);
+        else launch_rl_cg<17, kRlNarrow>(a, st);
+        return;
+    }
     switch (W) {
         case 8: launch_rl_cg<8>(a, st); break;
         case 12: launch_rl_cg<12>(a, st); break;
@@ -1759,7 +1779,8 @@ static DiskStats run_group(const pdd_cover &cov, const Problem &P, const pdd_ass
     const size_t perA = (size_t)S.n * S.n * sizeof(T);
     const size_t perR = (size_t)S.n * S.nrhs * sizeof(double);
     int rl_groups = 0;
-    const int rlW = mixed ? rl_width(S.n, S.nrhs, rl_groups) : 0;
+    bool rl_narrow = false;
+    const int rlW = mixed ? rl_width(S.n, S.nrhs, rl_groups, rl_narrow) : 0;
     const int nblk = (S.n + kRlTB - 1) / kRlTB;
     const size_t perDinv = rlW ? (size_t)nblk * 2 * kRlTB * kRlTB * sizeof(float) + 2 * perR + perA : 0;
     const bool use_np = mixed && o.factor == PDD_FACTOR_RECURSIVE_TC && o.lu_leaf_width == 0 && S.n > 64;
@@ -1950,7 +1971,7 @@ static DiskStats run_group(const pdd_cover &cov, const Problem &P, const pdd_ass
                                     X.p, conv.p, dmaxb.p, xmaxb.p, Dhl.p, s == 0 ? 0 : (s == 1 ? 1 : 2), nd,
                                     rl_groups};
                     PDD_CUDA(cudaEventRecord(sev[2 * s], st));
-                    launch_rl(rlW, ra, st);
+                    launch_rl(rlW, rl_narrow, ra, st);
                     PDD_CUDA(cudaEventRecord(sev[2 * s + 1], st));
                     PDD_LAUNCH(k_refine_conv, cdiv(nd, 256), 256, 0, st, nd, conv.p, sweeps.p, dmaxb.p, xmaxb.p, dprev.p,
                                tol);
