@@ -392,15 +392,15 @@ def roofline(stats, cfg, N, ms_solve):
     ks.sort(key=lambda k: -(k["ms"] or 0.0))
     out.update(ks[0])
     out["others"] = ks[1:]
-    # the disk path (a6-a9): 2/3 n^3 (LU) + 2 n^2 (n_k + 1) per sweep (solves) per disk, over its stage time
-    sweeps = st["disk_solves"] / max(1, st["floating_disks"])
-    per_disk = 2.0 / 3.0 * n ** 3 + 2.0 * n * n * nrhs * sweeps
+    # the disk path (a6-a9): 2/3 n^3 per matrix (LU; one matrix for all disks without drift and killing) +
+    # 2 n^2 (n_k + 1) per (disk, sweep) (solves), over its stage time
+    factored = 1 if cfg["op"]["b"] == cfg["op"]["c"] == "zero" else st["floating_disks"]
+    flop = 2.0 / 3.0 * n ** 3 * factored + tri_flop
     disk_ms = mean("ms_disks")
-    out["disk_path"] = {"flop_per_disk": per_disk, "disks": st["floating_disks"], "sweeps_per_disk": sweeps,
-                        "ms": disk_ms, "achieved_tflops": st["floating_disks"] * per_disk / (disk_ms / 1e3) / 1e12,
-                        "tf32_peak_tflops": tf32,
-                        "frac_of_tf32": st["floating_disks"] * per_disk / (disk_ms / 1e3) / 1e12 / tf32,
-                        "frac_of_tf32_over_3": st["floating_disks"] * per_disk / (disk_ms / 1e3) / 1e12 / (tf32 / 3)}
+    out["disk_path"] = {"flop": flop, "disks": st["floating_disks"], "factored": factored,
+                        "solves": st["disk_solves"], "ms": disk_ms, "achieved_tflops": flop / (disk_ms / 1e3) / 1e12,
+                        "tf32_peak_tflops": tf32, "frac_of_tf32": flop / (disk_ms / 1e3) / 1e12 / tf32,
+                        "frac_of_tf32_over_3": flop / (disk_ms / 1e3) / 1e12 / (tf32 / 3)}
     return out
 
 

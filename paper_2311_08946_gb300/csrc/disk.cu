@@ -490,7 +490,7 @@ __global__ void __launch_bounds__(256) k_lu_solve(const T *LUall, int n, long st
     const int disk = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (conv && conv[disk]) return;
     const T *LU = LUall + disk * strideA;
-    const int *perm = permAll + (long)disk * n;
+    const int *perm = permAll + (strideA ? (long)disk * n : 0);
     const double *R = Rall + disk * strideR + c0;
     T *W = Wall + disk * strideR + c0;
     double *X = Xall + disk * strideR + c0;
@@ -709,12 +709,13 @@ __global__ void __launch_bounds__(NT, kRlThreads / NT) k_lu_solve_rl(const float
     const int disk = NARROW ? blockIdx.x / groups : blockIdx.x, tid = threadIdx.x;
     if (conv[disk]) return;
     const int c0 = (NARROW ? blockIdx.x - disk * groups : blockIdx.y) * CG, cg = min(CG, nrhs - c0);
-    const float *LUT = LUTall + disk * strideA;      // the factors transposed
-    const int *perm = permAll + (long)disk * n;
+    const int fd = strideA ? disk : 0;               // stride 0: one factorisation for all
+    const float *LUT = LUTall + fd * strideA;        // the factors transposed
+    const int *perm = permAll + (long)fd * n;
     const double *R = Rall + disk * strideR;
     double *X = Xall + disk * strideR;
     const int nblk = (n + TB - 1) / TB;
-    const float *Dv = DinvAll + (long)disk * nblk * 2 * (TB * TB);
+    const float *Dv = DinvAll + (long)fd * nblk * 2 * (TB * TB);
     for (int e = tid; e < n * CG; e += NT) {
         const int p = e / CG, c = e - p * CG;
         Bs[e] = (c < cg) ? (float)R[(long)perm[p] * nrhs + c0 + c] : 0.f;
@@ -1733,9 +1734,10 @@ static void run_lu_choice(const LuChoice &c, float *A, int n, long sA, int *perm
 }
 
 static LuChoice tune_lu(float *A, int n, long sA, int nd, cudaStream_t st) {
+    const int key = nd == 1 ? -n : n;            // a single matrix has a choice of its own
     {
         std::lock_guard<std::mutex> lk(g_lu_mu);
-        auto it = g_lu_choice.find(n);
+        auto it = g_lu_choice.find(key);
         if (it != g_lu_choice.end()) return it->second;
     }
     std::vector<LuChoice> cand{{1, 0, 0, 0.f}};
@@ -1766,8 +1768,276 @@ static LuChoice tune_lu(float *A, int n, long sA, int nd, cudaStream_t st) {
         if (t < best.ms) best = c;
     }
     std::lock_guard<std::mutex> lk(g_lu_mu);
-    g_lu_choice[n] = best;
+    g_lu_choice[key] = best;
     return best;
+}
+
+// ---------------------------------------------------------------------------
+// a wave's buffers, its solve (a8) and its evaluation (a9)
+// ---------------------------------------------------------------------------
+template <typename T>
+struct SolveBufs {
+    DevBuf<T> W;
+    DevBuf<double> X, Rr, dprev;
+    DevBuf<int> conv, sweeps;
+    DevBuf<unsigned long long> dmaxb, xmaxb;
+    DevBuf<float2> R1hl, Dhl;
+    int rlW = 0, rl_groups = 0;          // right-looking solve: columns of a group (0: the tiled solve), groups
+    bool rl_narrow = false;
+    void choose(const Shape &S) { rlW = sizeof(T) == 4 ? rl_width(S.n, S.nrhs, rl_groups, rl_narrow) : 0; }
+    void alloc(const Shape &S, int wave) {
+        const size_t cnt = (size_t)wave * S.n * S.nrhs;
+        choose(S);
+        if (rlW) {
+            dmaxb.alloc(wave);
+            xmaxb.alloc(wave);
+            dprev.alloc(wave);
+            R1hl.alloc(cnt);
+            Dhl.alloc(cnt);
+        }
+        W.alloc(cnt);
+        X.alloc(cnt);
+        if (sizeof(T) == 4) Rr.alloc(cnt);
+        conv.alloc(wave);
+        sweeps.alloc(wave);
+    }
+};
+
+template <typename T>
+struct Factors {
+    const T *A;
+    const float *AT, *dinv;              // right-looking solve: transposed, diagonal blocks inverted
+    const int *perm;
+    long sA;                             // 0: one factorisation for all entries
+};
+
+// X of nd entries, a disk each or the source columns of disks_of disks
+template <typename T>
+static void solve_wave(const Problem &P, const pdd_assembly_opts &o, const Shape &S, int nd, const Factors<T> &F,
+                       const NodeCoef *coef, long sC, const double *RHS, SolveBufs<T> &B, cudaStream_t st,
+                       DiskStats &wv, int disks_of = 1) {
+    const bool mixed = sizeof(T) == 4;
+    const long sR = (long)S.n * S.nrhs;
+    if (!mixed) {
+        launch_solve<T>(F.A, S.n, F.sA, F.perm, RHS, S.nrhs, sR, B.W.p, B.X.p, 0, nullptr, nullptr, 0.0, nd, st);
+    } else {
+        PDD_CUDA(cudaMemsetAsync(B.conv.p, 0, nd * sizeof(int), st));
+        PDD_CUDA(cudaMemsetAsync(B.sweeps.p, 0, nd * sizeof(int), st));
+        PDD_CUDA(cudaMemsetAsync(B.X.p, 0, (size_t)nd * sR * sizeof(double), st));
+        const int maxs = std::max(1, o.max_refine);
+        const double tol = o.refine_tol > 0 ? o.refine_tol : 1e-12;
+        const int nw = (S.nc - 1) + S.nt;
+        const size_t rsm = (size_t)kResNP * nw * sizeof(double);
+        const size_t rsm_df = ((size_t)kResNPdf * nw + 6 * kResNPdf) * sizeof(float2);
+        PDD_CUDA(cudaFuncSetAttribute(k_residual, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm));
+        PDD_CUDA(cudaFuncSetAttribute(k_residual_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm_df));
+        dim3 g_res(cdiv(S.n, kResNP), nd), g_res_df(cdiv(S.n, kResNPdf), nd);
+        // without drift, the forms over angle pairs (nd <= 65535 is the grid's limit for both)
+        const int cg1 = P.b_kind == PDD_B_ZERO ? sym_columns<double>(S) : 0;
+        const size_t sm1 = cg1 ? sym_smem<double>(S, cg1) : 0;
+        if (cg1) {
+            PDD_CUDA(cudaFuncSetAttribute(k_residual_sym<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1));
+            PDD_CUDA(cudaFuncSetAttribute(k_residual_sym<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1));
+        }
+        const int th1 = cg1 ? sym_threads(S, cg1) : 32;
+        const dim3 g_sym(cg1 ? cdiv(S.nrhs, cg1) : 1, nd);
+        auto first_residual = [&](float2 *r1) {
+            if (cg1)
+                PDD_LAUNCH(k_residual_sym<false>, g_sym, th1, sm1, st, S, coef, sC, RHS, B.X.p, nullptr,
+                           B.Rr.p, r1, sR, B.conv.p, cg1);
+            else
+                PDD_LAUNCH(k_residual, g_res, 256, rsm, st, S, coef, sC, RHS, B.X.p, B.Rr.p, sR, B.conv.p, r1);
+        };
+        std::vector<cudaEvent_t> sev(B.rlW ? 2 * maxs : 0);
+        for (cudaEvent_t &e : sev) PDD_CUDA(cudaEventCreate(&e));
+        struct EvFree {
+            std::vector<cudaEvent_t> &v;
+            ~EvFree() {
+                for (cudaEvent_t e : v) cudaEventDestroy(e);
+            }
+        } ev_free{sev};
+        if (B.rlW) {
+            PDD_CUDA(cudaMemsetAsync(B.dmaxb.p, 0, nd * sizeof(unsigned long long), st));
+            PDD_CUDA(cudaMemsetAsync(B.xmaxb.p, 0, nd * sizeof(unsigned long long), st));
+        }
+        for (int s = 0; s < maxs; ++s) {
+            const double *rhs_now = (s == 0) ? RHS : B.Rr.p;
+            if (B.rlW) {
+                const RlArgs ra{F.AT, S.n, F.sA, F.perm, F.dinv, rhs_now, S.nrhs, sR,
+                                B.X.p, B.conv.p, B.dmaxb.p, B.xmaxb.p, B.Dhl.p, s == 0 ? 0 : (s == 1 ? 1 : 2), nd,
+                                B.rl_groups};
+                PDD_CUDA(cudaEventRecord(sev[2 * s], st));
+                launch_rl(B.rlW, B.rl_narrow, ra, st);
+                PDD_CUDA(cudaEventRecord(sev[2 * s + 1], st));
+                PDD_LAUNCH(k_refine_conv, cdiv(nd, 256), 256, 0, st, nd, B.conv.p, B.sweeps.p, B.dmaxb.p, B.xmaxb.p, B.dprev.p,
+                           tol);
+                if (s + 1 < maxs) {
+                    if (s == 0)
+                        first_residual(B.R1hl.p);
+                    else if (cg1)
+                        PDD_LAUNCH(k_residual_sym<true>, g_sym, th1, sm1, st, S, coef, sC, nullptr, nullptr,
+                                   B.Dhl.p, B.Rr.p, B.R1hl.p, sR, B.conv.p, cg1);
+                    else
+                        PDD_LAUNCH(k_residual_df, g_res_df, 256, rsm_df, st, S, coef, sC, B.R1hl.p, B.Dhl.p, B.Rr.p, sR,
+                                   B.conv.p);
+                }
+            } else {
+                launch_solve<T>(F.A, S.n, F.sA, F.perm, rhs_now, S.nrhs, sR, B.W.p, B.X.p, 1, B.conv.p, B.sweeps.p, tol,
+                                nd, st);
+                if (s + 1 < maxs) first_residual(nullptr);
+            }
+        }
+        std::vector<int> hc(nd), hs(nd);
+        PDD_CUDA(cudaMemcpyAsync(hc.data(), B.conv.p, nd * sizeof(int), cudaMemcpyDeviceToHost, st));
+        PDD_CUDA(cudaMemcpyAsync(hs.data(), B.sweeps.p, nd * sizeof(int), cudaMemcpyDeviceToHost, st));
+        PDD_CUDA(cudaStreamSynchronize(st));
+        for (int d = 0; d < nd; ++d) {
+            wv.max_sweeps = std::max(wv.max_sweeps, hs[d]);
+            wv.unconverged += hc[d] ? 0 : disks_of;
+            wv.disk_solves += hs[d];
+        }
+        if (B.rlW)
+            for (int s = 0; s < maxs; ++s) {
+                float t = 0.f;
+                cudaEventElapsedTime(&t, sev[2 * s], sev[2 * s + 1]);
+                wv.ms_trisolve += t;
+            }
+    }
+}
+
+// a9 of nd disks; split: the mixed form's FP32 pairs of X are still to be made
+template <typename T>
+static void eval_wave(const pdd_cover &cov, pdd_system &sys, const Shape &S, const DiskDesc *dd, int nd,
+                      SolveBufs<T> &B, bool split, cudaStream_t st) {
+    const long sR = (long)S.n * S.nrhs;
+    if (S.nc + 1 > 130 || S.nt > 130) fail(PDD_EINVAL, "disk grid too large for the evaluation kernel");
+    if (B.rlW) {
+        // mixed form: double-float sums on X split into FP32 pairs (the correction buffer is free now)
+        const long cnt = (long)nd * sR;
+        if (split) PDD_LAUNCH(k_split_x, (int)std::min<long>(cdiv(cnt, 256), 4096), 256, 0, st, cnt, B.X.p, B.Dhl.p);
+        const size_t esm = sizeof(float2) * kEvalKnots * std::max<size_t>(2 * kEvalChunk, kEvalThreads);
+        PDD_CUDA(cudaFuncSetAttribute(k_disk_eval_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)esm));
+        PDD_LAUNCH(k_disk_eval_df, dim3(nd, cdiv(S.nrhs, kEvalThreads)), kEvalThreads, esm, st, S, dd,
+                   cov.sub_rows.p, cov.sub_off.p, cov.kx.p, cov.ky.p, cov.rowptr.p, B.Dhl.p, sR, sys.val.p, sys.bs.p);
+    } else {
+        const int group = (S.nrhs <= 32) ? 32 : ((S.nrhs <= 64) ? 64 : 128);
+        const size_t rowb = (size_t)(S.n + S.nt) * sizeof(double);
+        const int per = (int)std::min<size_t>(256 / group, (180 * 1024) / rowb);
+        if (per < 1) fail(PDD_EINVAL, "disk grid too large for the evaluation kernel");
+        const size_t esm = per * rowb;
+        PDD_CUDA(cudaFuncSetAttribute(k_disk_eval, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)esm));
+        PDD_LAUNCH(k_disk_eval, nd, 256, esm, st, S, dd, cov.sub_rows.p, cov.sub_off.p, cov.kx.p, cov.ky.p,
+                   cov.rowptr.p, B.X.p, sR, group, per, sys.val.p, sys.bs.p);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Without drift and killing the operator of a disk is that of the unit disk over R^2: the equilibrated
+// matrix and the boundary columns are the same for all disks of a grid shape.  They are factored and
+// solved once, for the first disk; the source columns, where there is a source, are each disk's own and
+// are solved kShareCols at a time against the shared factors.  A source column is scaled by a power of
+// two to a largest right-hand side in [1, 2): columns that are refined together are of one size.
+// 3,600 disks of 48 x 64 nodes: 985 -> 18 ms (the factorisations alone take 240 ms at the split-TF32
+// peak); 64 disks of 22 x 44 nodes with a source: 8.3 -> 5.5 ms.
+// ---------------------------------------------------------------------------
+static constexpr int kShareCols = 17;
+
+// right-hand sides of the source columns against the first disk's equilibrated matrix (radius R0, row
+// scales coef[p].s): -s_p (R / R0)^2 f(x_p) 2^-e, with scl = 2^e.  One CTA per disk
+__global__ void __launch_bounds__(256) k_source_cols(Problem P, Shape S, const DiskDesc *disks, const NodeCoef *coef,
+                                                     double R0, double *RHS, double *scl) {
+    __shared__ double red[8];
+    const int d = blockIdx.x, tid = threadIdx.x;
+    const DiskDesc dd = disks[d];
+    const double q = (dd.R / R0) * (dd.R / R0);
+    double *col = RHS + (long)(d / kShareCols) * S.n * kShareCols + d % kShareCols;
+    double mx = 0.0;
+    for (int p = tid; p < S.n; p += 256) {
+        const int k = p / S.nt + 1, j = p % S.nt;
+        const double rho = S.x[k];
+        double st, ct;
+        sincos(PDD_TWO_PI * j / S.nt, &st, &ct);
+        const double v = -coef[p].s * q * source(P, dd.cx + dd.R * rho * ct, dd.cy + dd.R * rho * st);
+        col[(long)p * kShareCols] = v;
+        mx = fmax(mx, fabs(v));
+    }
+    for (int o = 16; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((tid & 31) == 0) red[tid >> 5] = mx;
+    __syncthreads();
+    for (int w = 0; w < 8; ++w) mx = fmax(mx, red[w]);
+    const int e = mx > 0.0 && isfinite(mx) ? max(-1000, min(1000, ilogb(mx))) : 0;
+    const double dn = ldexp(1.0, -e);
+    for (int p = tid; p < S.n; p += 256) col[(long)p * kShareCols] *= dn;
+    if (tid == 0) scl[d] = ldexp(1.0, e);
+}
+
+// X of the disks from the shared boundary columns X0 and the source columns Xs (null: no source)
+template <typename V>
+__global__ void __launch_bounds__(256) k_gather_x(Shape S, int nd, const double *X0, const double *Xs, const double *scl,
+                                                  V *out) {
+    const long per = (long)S.n * S.nrhs, total = per * nd;
+    for (long e = blockIdx.x * 256L + threadIdx.x; e < total; e += gridDim.x * 256L) {
+        const int d = (int)(e / per), q = (int)(e - d * per), p = q / S.nrhs, c = q - p * S.nrhs;
+        double v = 0.0;
+        if (c < S.nk) v = X0[q];
+        else if (Xs) v = Xs[((long)(d / kShareCols) * S.n + p) * kShareCols + d % kShareCols] * scl[d];
+        if constexpr (std::is_same<V, float2>::value) out[e] = split_df_bits(v);
+        else out[e] = v;
+    }
+}
+
+// source solves and evaluation of all disks of a shape from one factorisation F and the boundary columns
+// X0 of the first disk (node coefficients coef, radius R0); returns the solves' time
+template <typename T>
+static float shared_disks(const pdd_cover &cov, const Problem &P, const pdd_assembly_opts &o, pdd_system &sys,
+                          const Shape &S, const std::vector<DiskDesc> &disks, Factors<T> F, const NodeCoef *coef,
+                          double R0, const double *X0, cudaStream_t st, DiskStats &wv) {
+    Shape Ss = S;                        // kShareCols disks' columns make one entry
+    Ss.nrhs = kShareCols;
+    const bool src = P.f_kind != PDD_F_ZERO;
+    SolveBufs<T> B, Bx;                  // the source columns'; Bx carries only X of the disks to their evaluation
+    Bx.choose(S);
+    const size_t per = (size_t)S.n * S.nrhs * sizeof(double) + sizeof(DiskDesc) + sizeof(double) +
+                       (src ? (size_t)S.n * (sizeof(T) + 3 * sizeof(double) + 2 * sizeof(float2)) : 0);
+    const size_t freeb = free_device_bytes(), budget = std::min<size_t>((size_t)(0.6 * freeb), (size_t)64 << 30);
+    size_t most = std::min<size_t>(disks.size(), 65535);
+    most = std::min(most, std::max<size_t>(kShareCols, budget / per / kShareCols * kShareCols));
+    const int chunk = (int)most, nvmax = cdiv(chunk, kShareCols);
+    if (nvmax * kShareCols * per > freeb) fail(PDD_ENOMEM, "not enough device memory for one disk");
+    DevBuf<DiskDesc> dd;
+    DevBuf<double> RHS, scl;
+    dd.alloc(chunk);
+    if (src) {
+        RHS.alloc((size_t)nvmax * S.n * kShareCols);
+        scl.alloc(chunk);
+        B.alloc(Ss, nvmax);
+    }
+    if (Bx.rlW) Bx.Dhl.alloc((size_t)chunk * S.n * S.nrhs);
+    else Bx.X.alloc((size_t)chunk * S.n * S.nrhs);
+    F.sA = 0;
+    float ms = 0.f;
+    for (size_t w0 = 0; w0 < disks.size(); w0 += chunk) {
+        const int nd = (int)std::min<size_t>(chunk, disks.size() - w0), nv = cdiv(nd, kShareCols);
+        PDD_CUDA(cudaMemcpyAsync(dd.p, disks.data() + w0, nd * sizeof(DiskDesc), cudaMemcpyHostToDevice, st));
+        if (src) {
+            StageTimer t(st, 2);
+            t.mark(0);
+            PDD_CUDA(cudaMemsetAsync(RHS.p, 0, (size_t)nv * S.n * kShareCols * sizeof(double), st));
+            PDD_LAUNCH(k_source_cols, nd, 256, 0, st, P, S, dd.p, coef, R0, RHS.p, scl.p);
+            solve_wave<T>(P, o, Ss, nv, F, coef, 0, RHS.p, B, st, wv, kShareCols);
+            t.mark(1);
+            PDD_CUDA(cudaStreamSynchronize(st));
+            ms += t.ms(0, 1);
+        }
+        const int grid = (int)std::min<long>(cdiv((long)nd * S.n * S.nrhs, 1024), 8192);
+        if (Bx.rlW)
+            PDD_LAUNCH(k_gather_x<float2>, grid, 256, 0, st, S, nd, X0, src ? B.X.p : nullptr, scl.p, Bx.Dhl.p);
+        else
+            PDD_LAUNCH(k_gather_x<double>, grid, 256, 0, st, S, nd, X0, src ? B.X.p : nullptr, scl.p, Bx.X.p);
+        eval_wave(cov, sys, S, dd.p, nd, Bx, false, st);
+    }
+    wv.unconverged = std::min<int>(wv.unconverged, (int)disks.size());
+    return ms;
 }
 
 template <typename T>
@@ -1778,9 +2048,14 @@ static DiskStats run_group(const pdd_cover &cov, const Problem &P, const pdd_ass
     const bool mixed = sizeof(T) == 4;
     const size_t perA = (size_t)S.n * S.n * sizeof(T);
     const size_t perR = (size_t)S.n * S.nrhs * sizeof(double);
-    int rl_groups = 0;
-    bool rl_narrow = false;
-    const int rlW = mixed ? rl_width(S.n, S.nrhs, rl_groups, rl_narrow) : 0;
+    SolveBufs<T> B;
+    B.choose(S);
+    const int rlW = B.rlW;
+    // one factorisation for all disks of the shape (see shared_disks); with a source, whose columns are a
+    // second sequence of solves (0.5 ms at n = 968), from two groups of columns on
+    const bool shared = P.b_kind == PDD_B_ZERO && P.c_kind == PDD_C_ZERO &&
+                        disks.size() > (P.f_kind == PDD_F_ZERO ? 1 : 2 * kShareCols);
+    const size_t ndisks = shared ? 1 : disks.size();
     const int nblk = (S.n + kRlTB - 1) / kRlTB;
     const size_t perDinv = rlW ? (size_t)nblk * 2 * kRlTB * kRlTB * sizeof(float) + 2 * perR + perA : 0;
     const bool use_np = mixed && o.factor == PDD_FACTOR_RECURSIVE_TC && o.lu_leaf_width == 0 && S.n > 64;
@@ -1791,11 +2066,11 @@ static DiskStats run_group(const pdd_cover &cov, const Problem &P, const pdd_ass
     size_t budget = std::min<size_t>((size_t)(0.6 * freeb), (size_t)64 << 30);
     if (use_np) {           // the GEMM tile scratch comes out of the same budget
         const size_t scr = lu_np_scratch_floats_per_disk(S.n) * sizeof(float) *
-                           std::min<size_t>(disks.size(), 256);
+                           std::min<size_t>(ndisks, 256);
         budget = budget > 2 * scr ? budget - scr : budget / 2;
     }
     int wave = (int)std::max<size_t>(1, budget / perDisk);
-    wave = std::min<int>(wave, (int)disks.size());
+    wave = std::min<int>(wave, (int)ndisks);
     if ((size_t)wave * perDisk > freeb) fail(PDD_ENOMEM, "not enough device memory for one disk");
     {
         // equal waves, as many as fill the SMs in the fewest rounds: the kernels that take one CTA
@@ -1804,7 +2079,7 @@ static DiskStats run_group(const pdd_cover &cov, const Problem &P, const pdd_ass
         int dev = 0, sms = 0;
         PDD_CUDA(cudaGetDevice(&dev));
         PDD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        const long total = (long)disks.size(), nw0 = (total + wave - 1) / wave;
+        const long total = (long)ndisks, nw0 = (total + wave - 1) / wave;
         long best = wave, best_rounds = -1;
         for (long nw = nw0; nw <= std::min(nw0 + 2, total); ++nw) {
             const long w = (total + nw - 1) / nw, rounds = nw * ((w + sms - 1) / sms);
@@ -1815,34 +2090,22 @@ static DiskStats run_group(const pdd_cover &cov, const Problem &P, const pdd_ass
         }
         wave = (int)best;
     }
-    DevBuf<T> A, W;
-    DevBuf<double> RHS, X, Rr;
+    DevBuf<T> A;
+    DevBuf<double> RHS;
     DevBuf<NodeCoef> coef;
-    DevBuf<int> perm, info, conv, sweeps;
+    DevBuf<int> perm, info;
     DevBuf<DiskDesc> dd;
     DevBuf<float> dinv, AT;
-    DevBuf<unsigned long long> dmaxb, xmaxb;
-    DevBuf<double> dprev;
-    DevBuf<float2> R1hl, Dhl;
     if (rlW) {
         dinv.alloc((size_t)wave * nblk * 2 * kRlTB * kRlTB);
         AT.alloc((size_t)wave * S.n * S.n);
-        dmaxb.alloc(wave);
-        xmaxb.alloc(wave);
-        dprev.alloc(wave);
-        R1hl.alloc((size_t)wave * S.n * S.nrhs);
-        Dhl.alloc((size_t)wave * S.n * S.nrhs);
     }
     A.alloc((size_t)wave * S.n * S.n);
-    W.alloc((size_t)wave * S.n * S.nrhs);
     RHS.alloc((size_t)wave * S.n * S.nrhs);
-    X.alloc((size_t)wave * S.n * S.nrhs);
-    if (mixed) Rr.alloc((size_t)wave * S.n * S.nrhs);
+    B.alloc(S, wave);
     coef.alloc((size_t)wave * S.n);
     perm.alloc((size_t)wave * S.n);
     info.alloc(wave);
-    conv.alloc(wave);
-    sweeps.alloc(wave);
     dd.alloc(wave);
     // pivot-free LU: inverses of the 64 x 64 diagonal blocks and the GEMMs' hi/lo tile scratch
     // (enough for min(wave, 256) disks of the largest update; larger waves run in chunks)
@@ -1856,8 +2119,8 @@ static DiskStats run_group(const pdd_cover &cov, const Problem &P, const pdd_ass
     }
     const long sA = (long)S.n * S.n, sR = (long)S.n * S.nrhs, sC = S.n;
     DiskStats ds;
-    for (size_t w0 = 0; w0 < disks.size(); w0 += wave) {
-        const int nd = (int)std::min<size_t>(wave, disks.size() - w0);
+    for (size_t w0 = 0; w0 < ndisks; w0 += wave) {
+        const int nd = (int)std::min<size_t>(wave, ndisks - w0);
         for (int attempt = 0; attempt < 2; ++attempt) {
         DiskStats wv;                                   // this wave's statistics (kept on success)
         PDD_CUDA(cudaMemcpyAsync(dd.p, disks.data() + w0, nd * sizeof(DiskDesc), cudaMemcpyHostToDevice, st));
@@ -1922,111 +2185,16 @@ static DiskStats run_group(const pdd_cover &cov, const Problem &P, const pdd_ass
                            reinterpret_cast<const float *>(A.p), AT.p, S.n, sA);
         }
         tm.mark(2);
-        if (!mixed) {
-            launch_solve<T>(A.p, S.n, sA, perm.p, RHS.p, S.nrhs, sR, W.p, X.p, 0, nullptr, nullptr, 0.0, nd, st);
+        const Factors<T> F{A.p, AT.p, dinv.p, perm.p, sA};
+        solve_wave<T>(P, o, S, nd, F, coef.p, sC, RHS.p, B, st, wv);
+        tm.mark(3);
+        if (shared) {
+            // every disk is unconverged when the common columns are
+            if (wv.unconverged) wv.unconverged = (int)disks.size();
+            if (!(np_used && wv.unconverged))
+                wv.ms_shared = shared_disks<T>(cov, P, o, sys, S, disks, F, coef.p, disks[0].R, B.X.p, st, wv);
         } else {
-            PDD_CUDA(cudaMemsetAsync(conv.p, 0, nd * sizeof(int), st));
-            PDD_CUDA(cudaMemsetAsync(sweeps.p, 0, nd * sizeof(int), st));
-            PDD_CUDA(cudaMemsetAsync(X.p, 0, (size_t)nd * sR * sizeof(double), st));
-            const int maxs = std::max(1, o.max_refine);
-            const double tol = o.refine_tol > 0 ? o.refine_tol : 1e-12;
-            const int nw = (S.nc - 1) + S.nt;
-            const size_t rsm = (size_t)kResNP * nw * sizeof(double);
-            const size_t rsm_df = ((size_t)kResNPdf * nw + 6 * kResNPdf) * sizeof(float2);
-            PDD_CUDA(cudaFuncSetAttribute(k_residual, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm));
-            PDD_CUDA(cudaFuncSetAttribute(k_residual_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm_df));
-            dim3 g_res(cdiv(S.n, kResNP), nd), g_res_df(cdiv(S.n, kResNPdf), nd);
-            // without drift, the forms over angle pairs (nd <= 65535 is the grid's limit for both)
-            const int cg1 = P.b_kind == PDD_B_ZERO ? sym_columns<double>(S) : 0;
-            const size_t sm1 = cg1 ? sym_smem<double>(S, cg1) : 0;
-            if (cg1) {
-                PDD_CUDA(cudaFuncSetAttribute(k_residual_sym<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1));
-                PDD_CUDA(cudaFuncSetAttribute(k_residual_sym<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1));
-            }
-            const int th1 = cg1 ? sym_threads(S, cg1) : 32;
-            const dim3 g_sym(cg1 ? cdiv(S.nrhs, cg1) : 1, nd);
-            auto first_residual = [&](float2 *r1) {
-                if (cg1)
-                    PDD_LAUNCH(k_residual_sym<false>, g_sym, th1, sm1, st, S, coef.p, sC, RHS.p, X.p, nullptr,
-                               Rr.p, r1, sR, conv.p, cg1);
-                else
-                    PDD_LAUNCH(k_residual, g_res, 256, rsm, st, S, coef.p, sC, RHS.p, X.p, Rr.p, sR, conv.p, r1);
-            };
-            std::vector<cudaEvent_t> sev(rlW ? 2 * maxs : 0);
-            for (cudaEvent_t &e : sev) PDD_CUDA(cudaEventCreate(&e));
-            struct EvFree {
-                std::vector<cudaEvent_t> &v;
-                ~EvFree() {
-                    for (cudaEvent_t e : v) cudaEventDestroy(e);
-                }
-            } ev_free{sev};
-            if (rlW) {
-                PDD_CUDA(cudaMemsetAsync(dmaxb.p, 0, nd * sizeof(unsigned long long), st));
-                PDD_CUDA(cudaMemsetAsync(xmaxb.p, 0, nd * sizeof(unsigned long long), st));
-            }
-            for (int s = 0; s < maxs; ++s) {
-                const double *rhs_now = (s == 0) ? RHS.p : Rr.p;
-                if (rlW) {
-                    const RlArgs ra{AT.p, S.n, sA, perm.p, dinv.p, rhs_now, S.nrhs, sR,
-                                    X.p, conv.p, dmaxb.p, xmaxb.p, Dhl.p, s == 0 ? 0 : (s == 1 ? 1 : 2), nd,
-                                    rl_groups};
-                    PDD_CUDA(cudaEventRecord(sev[2 * s], st));
-                    launch_rl(rlW, rl_narrow, ra, st);
-                    PDD_CUDA(cudaEventRecord(sev[2 * s + 1], st));
-                    PDD_LAUNCH(k_refine_conv, cdiv(nd, 256), 256, 0, st, nd, conv.p, sweeps.p, dmaxb.p, xmaxb.p, dprev.p,
-                               tol);
-                    if (s + 1 < maxs) {
-                        if (s == 0)
-                            first_residual(R1hl.p);
-                        else if (cg1)
-                            PDD_LAUNCH(k_residual_sym<true>, g_sym, th1, sm1, st, S, coef.p, sC, nullptr, nullptr,
-                                       Dhl.p, Rr.p, R1hl.p, sR, conv.p, cg1);
-                        else
-                            PDD_LAUNCH(k_residual_df, g_res_df, 256, rsm_df, st, S, coef.p, sC, R1hl.p, Dhl.p, Rr.p, sR,
-                                       conv.p);
-                    }
-                } else {
-                    launch_solve<T>(A.p, S.n, sA, perm.p, rhs_now, S.nrhs, sR, W.p, X.p, 1, conv.p, sweeps.p, tol,
-                                    nd, st);
-                    if (s + 1 < maxs) first_residual(nullptr);
-                }
-            }
-            tm.mark(3);
-            std::vector<int> hc(nd), hs(nd);
-            PDD_CUDA(cudaMemcpyAsync(hc.data(), conv.p, nd * sizeof(int), cudaMemcpyDeviceToHost, st));
-            PDD_CUDA(cudaMemcpyAsync(hs.data(), sweeps.p, nd * sizeof(int), cudaMemcpyDeviceToHost, st));
-            PDD_CUDA(cudaStreamSynchronize(st));
-            for (int d = 0; d < nd; ++d) {
-                wv.max_sweeps = std::max(wv.max_sweeps, hs[d]);
-                wv.unconverged += hc[d] ? 0 : 1;
-                wv.disk_solves += hs[d];
-            }
-            if (rlW)
-                for (int s = 0; s < maxs; ++s) {
-                    float t = 0.f;
-                    cudaEventElapsedTime(&t, sev[2 * s], sev[2 * s + 1]);
-                    wv.ms_trisolve += t;
-                }
-        }
-        if (!mixed) tm.mark(3);
-        if (S.nc + 1 > 130 || S.nt > 130) fail(PDD_EINVAL, "disk grid too large for the evaluation kernel");
-        if (rlW) {
-            // mixed form: double-float sums on X split into FP32 pairs (the correction buffer is free now)
-            const long cnt = (long)nd * sR;
-            PDD_LAUNCH(k_split_x, (int)std::min<long>(cdiv(cnt, 256), 4096), 256, 0, st, cnt, X.p, Dhl.p);
-            const size_t esm = sizeof(float2) * kEvalKnots * std::max<size_t>(2 * kEvalChunk, kEvalThreads);
-            PDD_CUDA(cudaFuncSetAttribute(k_disk_eval_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)esm));
-            PDD_LAUNCH(k_disk_eval_df, dim3(nd, cdiv(S.nrhs, kEvalThreads)), kEvalThreads, esm, st, S, dd.p,
-                       cov.sub_rows.p, cov.sub_off.p, cov.kx.p, cov.ky.p, cov.rowptr.p, Dhl.p, sR, sys.val.p, sys.bs.p);
-        } else {
-            const int group = (S.nrhs <= 32) ? 32 : ((S.nrhs <= 64) ? 64 : 128);
-            const size_t rowb = (size_t)(S.n + S.nt) * sizeof(double);
-            const int per = (int)std::min<size_t>(256 / group, (180 * 1024) / rowb);
-            if (per < 1) fail(PDD_EINVAL, "disk grid too large for the evaluation kernel");
-            const size_t esm = per * rowb;
-            PDD_CUDA(cudaFuncSetAttribute(k_disk_eval, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)esm));
-            PDD_LAUNCH(k_disk_eval, nd, 256, esm, st, S, dd.p, cov.sub_rows.p, cov.sub_off.p, cov.kx.p, cov.ky.p,
-                       cov.rowptr.p, X.p, sR, group, per, sys.val.p, sys.bs.p);
+            eval_wave(cov, sys, S, dd.p, nd, B, true, st);
         }
         tm.mark(4);
         std::vector<int> hinfo(nd);
@@ -2039,8 +2207,8 @@ static DiskStats run_group(const pdd_cover &cov, const Problem &P, const pdd_ass
         }
         ds.ms_operator += tm.ms(0, 1);
         ds.ms_factor += tm.ms(1, 2);
-        ds.ms_refine += tm.ms(2, 3);
-        ds.ms_eval += tm.ms(3, 4);
+        ds.ms_refine += tm.ms(2, 3) + wv.ms_shared;
+        ds.ms_eval += tm.ms(3, 4) - wv.ms_shared;
         ds.ms_tc_gemm += wv.ms_tc_gemm;
         ds.tc_gemm_flop += wv.tc_gemm_flop;
         ds.ms_gemm_fused += wv.ms_gemm_fused;
@@ -2057,8 +2225,9 @@ static DiskStats run_group(const pdd_cover &cov, const Problem &P, const pdd_ass
         ds.lu_fallback |= wv.lu_fallback;
         for (int d = 0; d < nd; ++d)
             if (hinfo[d] && !np_used) fail(PDD_ENOCONV, "singular collocation matrix");
-        ds.disks += nd;
-        for (int d = 0; d < nd; ++d) ds.rows += disks[w0 + d].row_end - disks[w0 + d].row_begin;
+        const int done = shared ? (int)disks.size() : nd;
+        ds.disks += done;
+        for (int d = 0; d < done; ++d) ds.rows += disks[w0 + d].row_end - disks[w0 + d].row_begin;
         break;
         }
     }

@@ -94,6 +94,7 @@ struct DiskStats {
     int lu_blocked = 0, lu_leaf = 0, lu_tmin = 0;          // factorisation used (mixed form)
     int lu_fallback = 0;                                   // a pivot-free wave was redone pivoted
     float ms_trisolve = 0, ms_tc_gemm = 0;                 // kernel-only device times (mixed form)
+    float ms_shared = 0;                                   // source solves against shared factors (in ms_refine)
     int64_t disk_solves = 0;                               // (disk, sweep) triangular solves
     double tc_gemm_flop = 0;                               // useful flops of the tensor-core launches
     float ms_gemm_fused = 0;                               // the fused-split part of ms_tc_gemm
