@@ -1011,7 +1011,16 @@ __global__ void k_refine_conv(int nd, int *conv, int *sweeps, unsigned long long
 // (0: the shared-memory block does not fit; the tiled solve is used).  narrow: groups of 17 columns at
 // most, two CTAs of 256 threads an SM, where both blocks fit (n <= 1,500): 864 disks of n = 1,024 with 33
 // columns take 0.71 ms a solve so and 0.94 in one group of 36
-static int rl_width(int n, int nrhs, int &groups, bool &narrow) {
+//
+// Few entries (nd, with their groups at most one a SM): groups of 4 or 8 columns, which spread an entry's
+// columns over more SMs; one entry of n = 3,072 with 17 columns: 0.50 -> 0.19 ms a solve.
+static int rl_width(int n, int nrhs, long nd, int &groups, bool &narrow) {
+    for (int w : {4, 8})
+        if (w < nrhs && nd * cdiv(nrhs, w) <= sm_count() && rl_smem_bytes(n, w) <= kRlSmemMax) {
+            narrow = false;
+            groups = cdiv(nrhs, w);
+            return w;
+        }
     static const int widths[] = {8, 12, 17, 20, 36, 52};     // 17: all 17 columns of 16-knot disks at n = 3072
     const int few = (nrhs + 16) / 17, cgn = (nrhs + few - 1) / few;
     for (int w : {8, 12, 17})
@@ -1074,6 +1083,7 @@ static void launch_rl(int W, bool narrow, const RlArgs &a, cudaStream_t st) {
         return;
     }
     switch (W) {
+        case 4: launch_rl_cg<4>(a, st); break;
         case 8: launch_rl_cg<8>(a, st); break;
         case 12: launch_rl_cg<12>(a, st); break;
         case 17: launch_rl_cg<17>(a, st); break;
@@ -1784,10 +1794,9 @@ struct SolveBufs {
     DevBuf<float2> R1hl, Dhl;
     int rlW = 0, rl_groups = 0;          // right-looking solve: columns of a group (0: the tiled solve), groups
     bool rl_narrow = false;
-    void choose(const Shape &S) { rlW = sizeof(T) == 4 ? rl_width(S.n, S.nrhs, rl_groups, rl_narrow) : 0; }
+    void choose(const Shape &S, long nd) { rlW = sizeof(T) == 4 ? rl_width(S.n, S.nrhs, nd, rl_groups, rl_narrow) : 0; }
     void alloc(const Shape &S, int wave) {
         const size_t cnt = (size_t)wave * S.n * S.nrhs;
-        choose(S);
         if (rlW) {
             dmaxb.alloc(wave);
             xmaxb.alloc(wave);
@@ -1996,7 +2005,7 @@ static float shared_disks(const pdd_cover &cov, const Problem &P, const pdd_asse
     Ss.nrhs = kShareCols;
     const bool src = P.f_kind != PDD_F_ZERO;
     SolveBufs<T> B, Bx;                  // the source columns'; Bx carries only X of the disks to their evaluation
-    Bx.choose(S);
+    Bx.choose(S, disks.size());
     const size_t per = (size_t)S.n * S.nrhs * sizeof(double) + sizeof(DiskDesc) + sizeof(double) +
                        (src ? (size_t)S.n * (sizeof(T) + 3 * sizeof(double) + 2 * sizeof(float2)) : 0);
     const size_t freeb = free_device_bytes(), budget = std::min<size_t>((size_t)(0.6 * freeb), (size_t)64 << 30);
@@ -2010,6 +2019,7 @@ static float shared_disks(const pdd_cover &cov, const Problem &P, const pdd_asse
     if (src) {
         RHS.alloc((size_t)nvmax * S.n * kShareCols);
         scl.alloc(chunk);
+        B.choose(Ss, nvmax);
         B.alloc(Ss, nvmax);
     }
     if (Bx.rlW) Bx.Dhl.alloc((size_t)chunk * S.n * S.nrhs);
@@ -2048,14 +2058,14 @@ static DiskStats run_group(const pdd_cover &cov, const Problem &P, const pdd_ass
     const bool mixed = sizeof(T) == 4;
     const size_t perA = (size_t)S.n * S.n * sizeof(T);
     const size_t perR = (size_t)S.n * S.nrhs * sizeof(double);
-    SolveBufs<T> B;
-    B.choose(S);
-    const int rlW = B.rlW;
     // one factorisation for all disks of the shape (see shared_disks); with a source, whose columns are a
     // second sequence of solves (0.5 ms at n = 968), from two groups of columns on
     const bool shared = P.b_kind == PDD_B_ZERO && P.c_kind == PDD_C_ZERO &&
                         disks.size() > (P.f_kind == PDD_F_ZERO ? 1 : 2 * kShareCols);
     const size_t ndisks = shared ? 1 : disks.size();
+    SolveBufs<T> B;
+    B.choose(S, ndisks);
+    const int rlW = B.rlW;
     const int nblk = (S.n + kRlTB - 1) / kRlTB;
     const size_t perDinv = rlW ? (size_t)nblk * 2 * kRlTB * kRlTB * sizeof(float) + 2 * perR + perA : 0;
     const bool use_np = mixed && o.factor == PDD_FACTOR_RECURSIVE_TC && o.lu_leaf_width == 0 && S.n > 64;

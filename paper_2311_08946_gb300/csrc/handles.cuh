@@ -161,6 +161,9 @@ void grad_disks(const pdd_cover &cov, const Problem &P, const double *u, const d
 void grad_mc(const pdd_cover &cov, const Problem &P, const pdd_assembly_opts &o, const pdd_system &sys,
              const double *u, const double *lambda, DevBuf<double> &partial, int &n_part,
              cudaStream_t st);
+// SMs of the current device
+int sm_count();
+
 // K^-1 of every perimeter stencil (offsets per circle, -1 when none)
 void build_imq_inverses(const pdd_cover &cov, double c2, DevBuf<double> &kinv, DevBuf<long> &koff_m,
                         DevBuf<double> &kcond, cudaStream_t st);

@@ -1104,7 +1104,7 @@ __global__ void __launch_bounds__(kFzThreads, fz_ctas(TN)) k_tc_gemm_fused(FzArg
 
 static int g_sms[64] = {0};
 
-static int sm_count() {
+int sm_count() {
     int dev = 0;
     PDD_CUDA(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) fail(PDD_EINVAL, "device ordinal out of range");
