@@ -5,10 +5,11 @@
 //       scales (one thread per node), the right-hand sides [A_IB H, -f], then
 //       the rows of the row-equilibrated collocation matrix of L + c.
 //   a7  FP64 form: lu64.cu, blocked LU with partial pivoting over the whole
-//       device (k_lu, one CTA per disk, where its panel does not fit).  Mixed form: the recursive FP32
-//       LU of lu_rec.cu (tensor-core Schur updates) or the blocked one, chosen
-//       by tune_lu.  The paper factors by QR (Eq. 41); LU solves the same
-//       systems.
+//       device (k_lu, one CTA per disk, where its panel does not fit).  Mixed
+//       form: the pivot-free FP32 LU of lu_np.cu on the tensor cores, or the
+//       pivoted ones (lu_rec.cu or blocked, chosen by tune_lu).  The paper
+//       factors by QR (Eq. 41); LU solves the same systems.  Without drift and
+//       killing one factorisation serves all disks of a grid (shared_disks).
 //   a8  FP64 form: k_lu_solve.  Mixed form: k_lu_solve_rl on the transposed
 //       FP32 factors, refined in FP64 (first residual k_residual in FP64,
 //       later ones k_residual_df in double-float delta form) until the
@@ -1305,7 +1306,7 @@ struct SymDf {
     __device__ static T mul(T a, T b) { return df_mul(a, b); }
     __device__ static T from(double v) { return df_split(v); }
 };
-static constexpr int kSymThreads = 384, kSymK = 8;
+static constexpr int kSymThreads = 384, kSymK = 8, kSymSmem = 220 * 1024;
 
 template <typename T>
 static size_t sym_smem(const Shape &S, int cg) {
@@ -1432,7 +1433,7 @@ static int sym_threads(const Shape &S, int cg) {
 template <typename T>
 static int sym_columns(const Shape &S) {
     for (int cg = 4; cg >= 1; --cg)
-        if (sym_smem<T>(S, cg) <= (size_t)220 * 1024) return std::min(cg, S.nrhs);
+        if (sym_smem<T>(S, cg) <= (size_t)kSymSmem) return std::min(cg, S.nrhs);
     return 0;
 }
 
@@ -1845,8 +1846,8 @@ static void solve_wave(const Problem &P, const pdd_assembly_opts &o, const Shape
         const int cg1 = P.b_kind == PDD_B_ZERO ? sym_columns<double>(S) : 0;
         const size_t sm1 = cg1 ? sym_smem<double>(S, cg1) : 0;
         if (cg1) {
-            PDD_CUDA(cudaFuncSetAttribute(k_residual_sym<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1));
-            PDD_CUDA(cudaFuncSetAttribute(k_residual_sym<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1));
+            PDD_CUDA(cudaFuncSetAttribute(k_residual_sym<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSymSmem));
+            PDD_CUDA(cudaFuncSetAttribute(k_residual_sym<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSymSmem));
         }
         const int th1 = cg1 ? sym_threads(S, cg1) : 32;
         const dim3 g_sym(cg1 ? cdiv(S.nrhs, cg1) : 1, nd);

@@ -242,14 +242,15 @@ __global__ void k_lu64_init(int n, int nd, int *perm, int *info) {
     if (i < nd) info[i] = 0;
 }
 
+static constexpr int kPanelSmem = 226 * 1024;        // 227 KB per CTA, less the static arrays
+
 template <int NB>
 static void lu64_run(double *A, int n, long sA, int *perm, int *info, int nd, int sms, cudaStream_t st) {
     DevBuf<int2> moves;
     DevBuf<int> nmoves;
     moves.alloc((size_t)nd * 2 * NB);
     nmoves.alloc(nd);
-    PDD_CUDA(cudaFuncSetAttribute(k_lu64_panel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)lu64_panel_smem<NB>(n)));
+    PDD_CUDA(cudaFuncSetAttribute(k_lu64_panel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPanelSmem));
     for (int k0 = 0; k0 < n; k0 += NB) {
         const int kb = std::min(NB, n - k0), rem = n - k0 - kb;
         PDD_LAUNCH(k_lu64_panel<NB>, nd, kPanelThreads, lu64_panel_smem<NB>(n - k0), st, A, n, sA, k0, perm, info,
@@ -271,7 +272,7 @@ static void lu64_run(double *A, int n, long sA, int *perm, int *info, int nd, in
 // false when the panel of n rows does not fit in shared memory or the batch exceeds a launch's grid (the
 // caller's one-CTA form takes those)
 bool lu_f64(double *A, int n, long strideA, int *perm, int *info, int nd, cudaStream_t st) {
-    const size_t most = 226 * 1024;
+    const size_t most = kPanelSmem;
     if (lu64_panel_smem<8>(n) > most || nd > 65535) return false;
     int dev = 0, sms = 0;
     PDD_CUDA(cudaGetDevice(&dev));

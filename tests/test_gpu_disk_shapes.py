@@ -35,3 +35,28 @@ def test_mixed_rows_match_fp64_rows(n_r, n_theta, n_knots, drift):
         scale = np.linalg.norm(ref["val"][s])
         assert np.linalg.norm(got["val"][s] - ref["val"][s]) <= 1e-10 * scale, i
         assert abs(got["b"][i] - ref["b"][i]) <= 1e-10 * max(1.0, abs(ref["b"][i])), i
+
+
+@pytest.mark.parametrize("n_knots", [6, 10, 16, 32])
+def test_many_disks(n_knots):
+    """More disks than SMs: the solves in groups of 8, 12 and 17 columns, two CTAs an SM."""
+    import paper_2311_08946_gb300 as pdd
+
+    m, s = 15, 0.25
+    cfg = workloads.tiny(paths=32)
+    cfg["domain"] = {"kind": "square", "p": [0.0, 0.0, m * s, m * s]}
+    cfg["cover"] = {"kind": "square_lattice", "nx": m, "ny": m, "x_origin": s / 2, "y_origin": s / 2, "spacing": s,
+                    "radius": 0.8 * s}
+    cfg["n_r"], cfg["n_theta"], cfg["n_knots"] = 11, 20, n_knots
+    cfg["op"] = {"b": "zero", "c": "quadratic", "f": "one", "g": "sin_cos"}
+    cov = pdd.Cover(cfg)
+    a = {k: v.cpu().numpy() for k, v in cov.arrays().items()}
+    ref, got = (pdd.System(cov, cfg, p, path_precision="fp64") for p in ("fp64", "mixed"))
+    assert got.stats()["floating_disks"] == (m - 2) ** 2 and got.stats()["unconverged_disks"] == 0
+    g, r = ({k: v.cpu().numpy() for k, v in x.csr().items()} for x in (got, ref))
+    for i in range(cov.N):
+        if a["row_sub"][i] < 0 or not a["floating"][a["row_sub"][i]]:
+            continue
+        e = slice(a["rowptr"][i], a["rowptr"][i + 1])
+        assert np.linalg.norm(g["val"][e] - r["val"][e]) <= 1e-10 * np.linalg.norm(r["val"][e]), i
+        assert abs(g["b"][i] - r["b"][i]) <= 1e-10 * max(1.0, abs(r["b"][i])), i
