@@ -4,11 +4,12 @@
 //   a10 k_imq_inverse: K_lk = ((u_l - u_k)^2 + c^2)^-1/2 per perimeter stencil
 //       (u the knots' local angles in radians), Cholesky factor and K^-1 in FP64
 //       (one CTA per circle), and kappa_1(K).
-//   a11 k_paths: Euler-Maruyama paths of dX = b dt + dW, dY = c Y dt,
+//   a11 k_paths (short paths), k_paths_long, k_paths64 (FP64 form), with exit
+//       points by k_exit32, k_exit64: Euler-Maruyama paths of dX = b dt + dW, dY = c Y dt,
 //       dZ = f Y dt from the knot, stopped at the first step whose end point
 //       leaves the open disk or the open domain (optionally both shrunk by the
-//       Gobet-Menozzi shift).  One CTA per (row, subdomain) slot; a lane takes
-//       the row's next path id as soon as its path exits.  Exit point: the
+//       Gobet-Menozzi shift).  A lane takes the next path id (of its row or of
+//       the launch) as soon as its path exits.  Exit point: the
 //       first crossing of the segment with the circle or dOmega (ties to
 //       dOmega).  Normals: Philox4x32-10, key (seed, knot), counter (step,
 //       path, 0, k) with k the subdomain's position in the row's list.  FP64
@@ -949,11 +950,14 @@ __global__ void __launch_bounds__(256) k_exit32(Problem P, PathArgs A, Pool32 Q)
 //     of unequal path lengths or fewer rows than SMs leave nothing idle);
 //   * when the queue is empty, a warp with few paths left hands their states over and ends; the next
 //     launch packs them into full warps (four launches, the last runs to completion);
+//   * without drift, killing and source the second launch is k_walk64, which finishes what the first
+//     hands over: the longest path's steps, one after the other, are the end of the launch, and their
+//     normals are known beforehand, so eight lanes take a path and form the normals of eight steps at once;
 //   * the exit point of a path (roots, divisions, an arctangent) is left to k_exit64, one thread per
 //     record, instead of being computed by one lane while 31 wait;
 //   * the uniforms are put together from their bits, the comparisons with the domain's box are integer
 //     comparisons, the circle is tested in FP32 first.
-// 4 x 4 lattice (116 rows x 1,000 paths): 9.4 -> 6.1 ms; 140 circles with variable coefficients, 10^4
+// 4 x 4 lattice (116 rows x 1,000 paths): 9.4 -> 3.2 ms (6.1 without k_walk64); 140 circles with variable coefficients, 10^4
 // paths a row: 325 -> 189 ms.
 // ---------------------------------------------------------------------------
 struct alignas(16) Slot64 {          // what a path reads when it starts
@@ -1189,6 +1193,113 @@ __global__ void __launch_bounds__(kP64Threads) k_paths64(Problem P, PathArgs A, 
         my_capped += __shfl_xor_sync(kAll, my_capped, o);
     }
     if ((threadIdx.x & 31) == 0) {
+        if (my_steps) atomicAdd(A.steps, my_steps);
+        if (my_capped) atomicAdd(A.capped, my_capped);
+    }
+}
+
+// The paths of Q.in to their ends, b = c = f = 0 (Y = 1 and Z = 0 stay): eight lanes per path, whose
+// normals of the next eight steps they form one each; the steps then run in all of them alike.
+static constexpr int kWalkLanes = 8;
+__global__ void __launch_bounds__(kP64Threads) k_walk64(Problem P, PathArgs A, PathPool Q) {
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31, gl = lane & (kWalkLanes - 1), lead = lane - gl;
+    const bool sq_dom = P.dom_kind == 0;
+    const double sft = A.shift;
+    const double d0 = sq_dom ? P.dom[0] + sft : P.dom[0], d1 = sq_dom ? P.dom[1] + sft : P.dom[1];
+    const double d2 = P.dom[2] - sft, d3 = P.dom[3] - sft;
+    const double dr2 = (P.dom[2] - sft) * (P.dom[2] - sft);
+    const long long q0 = order_key(d0 + 0.0), q1 = order_key(d1 + 0.0), q2 = order_key(d2), q3 = order_key(d3);
+    const double sh = sqrt(A.h);
+    const unsigned total = *Q.n_in;
+    unsigned long long my_steps = 0;
+    int my_capped = 0;
+    bool have = false, drained = false;
+    double x = 0.0, y = 0.0, cx = 0.0, cy = 0.0, r2 = 0.0, Yv = 1.0, Zv = 0.0;
+    float r2f = 0.f;
+    long rec = 0;
+    int p = 0, k = 0, knot = 0, max_steps = 0;
+    uint32_t kw = 0;
+    for (;;) {
+        unsigned g = 0;
+        if (!have && !drained && gl == 0) g = (unsigned)min(atomicAdd(Q.next, 1ULL), (unsigned long long)total);
+        g = __shfl_sync(kAll, g, lead);
+        if (!have && !drained) {
+            drained = g >= total;
+            if (!drained) {
+                const PathState s = Q.in[g];
+                const Slot64 *S = Q.slots + s.slot;
+                have = true;
+                p = s.p;
+                k = s.k;
+                x = s.x;
+                y = s.y;
+                Yv = s.Y;
+                Zv = s.Z;
+                cx = S->cx;
+                cy = S->cy;
+                r2 = S->r2;
+                r2f = trunc32(r2) * 0.9999f;
+                rec = S->rbase + p;
+                knot = S->i;
+                max_steps = S->max_steps;
+                kw = S->kw;
+            }
+        }
+        if (!__ballot_sync(kAll, have)) break;
+        double z0 = 0.0, z1 = 0.0;
+        if (have) normals64(A.seed, (uint32_t)knot, kw, (uint32_t)(k + gl), (uint32_t)p, z0, z1);
+#pragma unroll
+        for (int j = 0; j < kWalkLanes; ++j) {
+            const double xi0 = __shfl_sync(kAll, z0, lead + j), xi1 = __shfl_sync(kAll, z1, lead + j);
+            if (!have) continue;
+            if (k >= max_steps) {
+                if (gl == 0) {
+                    A.side[rec] = 2;
+                    A.su[rec] = 0.0;
+                    A.Y[rec] = 0.0;
+                    A.Z[rec] = 0.0;
+                    ++my_capped;
+                    my_steps += (unsigned long long)k;
+                }
+                have = false;
+                continue;
+            }
+            const double nx = x + sh * xi0, ny = y + sh * xi1;
+            ++k;
+            const double ddx = nx - cx, ddy = ny - cy;
+            const float fx = trunc32(ddx), fy = trunc32(ddy);
+            const unsigned top =
+                max((unsigned)__double2hiint(ddx) & 0x7fffffffu, (unsigned)__double2hiint(ddy) & 0x7fffffffu);
+            bool out = !(fx * fx + fy * fy < r2f && top < 0x43000000u);
+            if (out) out = !(ddx * ddx + ddy * ddy < r2);
+            if (sq_dom) {
+                const long long kx = order_key(nx), ky = order_key(ny);
+                out = out || !(kx > q0 && kx < q2 && ky > q1 && ky < q3);
+            } else {
+                const double ex0 = nx - d0, ey0 = ny - d1;
+                out = out || !(ex0 * ex0 + ey0 * ey0 < dr2);
+            }
+            if (!out) {
+                x = nx;
+                y = ny;
+                continue;
+            }
+            if (gl == 0) {
+                A.side[rec] = 3;
+                Q.seg[rec] = Seg64{x, y, nx, ny};
+                A.Y[rec] = Yv;
+                A.Z[rec] = Zv;
+                my_steps += (unsigned long long)k;
+            }
+            have = false;
+        }
+    }
+    for (int o = 16; o; o >>= 1) {
+        my_steps += __shfl_xor_sync(kAll, my_steps, o);
+        my_capped += __shfl_xor_sync(kAll, my_capped, o);
+    }
+    if (lane == 0) {
         if (my_steps) atomicAdd(A.steps, my_steps);
         if (my_capped) atomicAdd(A.capped, my_capped);
     }
@@ -2004,6 +2115,7 @@ static void run_paths64(const Problem &P, const PathArgs &A, int nrows, long tot
     PathPool Q{B.slots.p, nrows, (unsigned long long)total, nullptr, nullptr, nullptr, nullptr, nullptr, 0, nullptr,
                nullptr, B.seg.p};
     int grid = ctas;
+    const bool walk = P.b_kind == PDD_B_ZERO && P.c_kind == PDD_C_ZERO && P.f_kind == PDD_F_ZERO && A.cvd == 0;
     for (int pass = 0; pass < kP64Passes; ++pass) {
         const bool last = pass == kP64Passes - 1;
         Q.next = B.next.p + pass;
@@ -2014,6 +2126,11 @@ static void run_paths64(const Problem &P, const PathArgs &A, int nrows, long tot
         Q.cq_out = B.cq[pass & 1].p;
         Q.n_out = B.count.p + pass;
         Q.keep = last ? 0 : 16;
+        if (walk && pass == 1) {
+            const int most = cdiv(15L * ctas * (kP64Threads / 32), kP64Threads / kWalkLanes);     // its paths, at most
+            PDD_LAUNCH(k_walk64, std::min(most, 8 * sms), kP64Threads, 0, st, P, A, Q);
+            break;
+        }
         if (A.cvd > 0) launch_pass64<true>(P, A, Q, grid, sm, st);
         else launch_pass64<false>(P, A, Q, grid, sm, st);
         grid = std::max(1, (grid + 1) / 2);               // every warp hands over at most half its lanes
