@@ -11,7 +11,9 @@
 //   k_lu64_rows    moves those rows in the columns outside the panel and solves U12 = L11^-1 A12, by
 //                  column tiles;
 //   k_lu64_update  A22 -= L21 U12 by tiles, 4 x 4 entries a thread.
-// 4 disks of n = 256: 2.63 -> 0.90 ms; 104 of n = 1,024: 113 -> 65 ms (57 at the FP64 peak).
+// NB = 32, 16, 8 or 4, the widest whose panel fits in shared memory (n <= 863, 1,653, 3,045 and 5,259).
+// 4 disks of n = 256: 2.63 -> 0.90 ms; 104 of n = 1,024: 113 -> 65 ms (57 at the FP64 peak); one of
+// n = 3,072: 3,510 -> 38 ms.
 #include <algorithm>
 
 #include "handles.cuh"
@@ -273,14 +275,15 @@ static void lu64_run(double *A, int n, long sA, int *perm, int *info, int nd, in
 // caller's one-CTA form takes those)
 bool lu_f64(double *A, int n, long strideA, int *perm, int *info, int nd, cudaStream_t st) {
     const size_t most = kPanelSmem;
-    if (lu64_panel_smem<8>(n) > most || nd > 65535) return false;
+    if (lu64_panel_smem<4>(n) > most || nd > 65535) return false;
     int dev = 0, sms = 0;
     PDD_CUDA(cudaGetDevice(&dev));
     PDD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     PDD_LAUNCH(k_lu64_init, cdiv(std::max<long>((long)n * nd, nd), 256), 256, 0, st, n, nd, perm, info);
     if (lu64_panel_smem<32>(n) <= most) lu64_run<32>(A, n, strideA, perm, info, nd, sms, st);
     else if (lu64_panel_smem<16>(n) <= most) lu64_run<16>(A, n, strideA, perm, info, nd, sms, st);
-    else lu64_run<8>(A, n, strideA, perm, info, nd, sms, st);
+    else if (lu64_panel_smem<8>(n) <= most) lu64_run<8>(A, n, strideA, perm, info, nd, sms, st);
+    else lu64_run<4>(A, n, strideA, perm, info, nd, sms, st);
     return true;
 }
 

@@ -1,7 +1,7 @@
 """Disk grids at which the tiled disk kernels can go wrong, the mixed form against the FP64 form.
 
 The two share neither the factorisation (pivot-free FP32 on the tensor cores / blocked FP64 with partial
-pivoting, panels of 32, 16 and 8 columns by n), nor the solves, nor the evaluation, nor the residuals
+pivoting, panels of 32, 16, 8 and 4 columns by n), nor the solves, nor the evaluation, nor the residuals
 (angle pairs in tiles of 32 angles and 8 rings without drift; node by node with it).  Grids: fewer rings
 than a tile and more, rings and angle halves that are no multiples, halves above 32, column counts that
 leave ragged groups.  Bar: 1e-10 of each floating row, the one both forms meet against the oracle."""
@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("n_r,n_theta,n_knots,drift", [
     (3, 4, 6, False), (13, 22, 10, False), (13, 22, 10, True), (20, 70, 16, False), (33, 50, 18, False),
-    (32, 64, 20, True), (45, 64, 44, False)])
+    (32, 64, 20, True), (45, 64, 44, False), (48, 64, 16, True)])
 def test_mixed_rows_match_fp64_rows(n_r, n_theta, n_knots, drift):
     import paper_2311_08946_gb300 as pdd
 
