@@ -950,14 +950,16 @@ __global__ void __launch_bounds__(256) k_exit32(Problem P, PathArgs A, Pool32 Q)
 //     of unequal path lengths or fewer rows than SMs leave nothing idle);
 //   * when the queue is empty, a warp with few paths left hands their states over and ends; the next
 //     launch packs them into full warps (four launches, the last runs to completion);
-//   * without drift, killing and source the second launch is k_walk64, which finishes what the first
-//     hands over: the longest path's steps, one after the other, are the end of the launch, and their
-//     normals are known beforehand, so eight lanes take a path and form the normals of eight steps at once;
+//   * without drift, and with killing and source zero or by Gaussians, the second launch is k_walk64,
+//     which finishes what the first hands over: the longest path's steps, one after the other, are the end
+//     of the launch, so eight lanes take a path, form the normals of eight steps at once (they depend on
+//     the step's number alone) and share a step's Gaussians;
 //   * the exit point of a path (roots, divisions, an arctangent) is left to k_exit64, one thread per
 //     record, instead of being computed by one lane while 31 wait;
 //   * the uniforms are put together from their bits, the comparisons with the domain's box are integer
 //     comparisons, the circle is tested in FP32 first.
-// 4 x 4 lattice (116 rows x 1,000 paths): 9.4 -> 3.2 ms (6.1 without k_walk64); 140 circles with variable coefficients, 10^4
+// 4 x 4 lattice (116 rows x 1,000 paths): 9.4 -> 3.2 ms (6.1 without k_walk64), with 64 Gaussians of c
+// and 16 of f 159 -> 61 ms (110); 140 circles with variable coefficients, 10^4
 // paths a row: 325 -> 189 ms.
 // ---------------------------------------------------------------------------
 struct alignas(16) Slot64 {          // what a path reads when it starts
@@ -1198,10 +1200,57 @@ __global__ void __launch_bounds__(kP64Threads) k_paths64(Problem P, PathArgs A, 
     }
 }
 
-// The paths of Q.in to their ends, b = c = f = 0 (Y = 1 and Z = 0 stay): eight lanes per path, whose
-// normals of the next eight steps they form one each; the steps then run in all of them alike.
+// The paths of Q.in to their ends, b = 0, c and f zero or by Gaussians: eight lanes per path.  They form
+// the normals of the next eight steps one each; a step then runs in all of them alike, but for the
+// exponentials of its Gaussians, of which each lane takes every eighth (added up in their order).
 static constexpr int kWalkLanes = 8;
+__device__ __forceinline__ double from_lane(double v, int lane) { return __shfl_sync(0xffffffffu, v, lane); }
+
+// sum_q w_q e(q), e evaluated by lane q mod 8 of the group that starts at lane `lead`
+template <typename Eval>
+__device__ __forceinline__ double walk_sum(int n, const double *w, int lead, int gl, Eval eval) {
+    constexpr int B = 4;
+    double s = 0.0;
+    for (int q0 = 0; q0 < n; q0 += B * kWalkLanes) {
+        double e[B];
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            const int q = q0 + b * kWalkLanes + gl;
+            e[b] = q < n ? eval(q) : 0.0;
+        }
+#pragma unroll
+        for (int b = 0; b < B; ++b)
+#pragma unroll
+            for (int i = 0; i < kWalkLanes; ++i) {
+                const int q = q0 + b * kWalkLanes + i;
+                const double v = from_lane(e[b], lead + i);
+                if (q < n) s += w[q] * v;
+            }
+    }
+    return s;
+}
+
+template <bool KILL, bool SRC>
 __global__ void __launch_bounds__(kP64Threads) k_walk64(Problem P, PathArgs A, PathPool Q) {
+    extern __shared__ __align__(16) double psm64[];       // killing: exp_neg's table, then x, y, w as in k_paths64
+    const double2 *etab = reinterpret_cast<const double2 *>(psm64);
+    const int nr = KILL ? P.n_rbf : 0, nf = SRC ? P.n_frbf : 0;
+    const bool staged = nr <= kP64Staged;
+    const double *rx = staged ? psm64 + 2 * kExpTab : P.rbf_x, *ry = staged ? rx + nr : P.rbf_y;
+    const double *rw = staged ? ry + nr : P.rbf_w;
+    const double inv2s = KILL ? 1.0 / (2.0 * P.rbf_sigma * P.rbf_sigma) : 0.0;
+    const double finv = SRC ? 1.0 / (2.0 * P.frbf_sigma * P.frbf_sigma) : 0.0;
+    if (KILL) {
+        double2 *et = reinterpret_cast<double2 *>(psm64);
+        double *rt = psm64 + 2 * kExpTab;
+        for (int q = threadIdx.x; q < kExpTab; q += kP64Threads) et[q] = kExp2Tab[q];
+        for (int q = threadIdx.x; staged && q < nr; q += kP64Threads) {
+            rt[q] = P.rbf_x[q];
+            rt[nr + q] = P.rbf_y[q];
+            rt[2 * nr + q] = P.rbf_w[q];
+        }
+        __syncthreads();
+    }
     constexpr unsigned kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31, gl = lane & (kWalkLanes - 1), lead = lane - gl;
     const bool sq_dom = P.dom_kind == 0;
@@ -1249,9 +1298,24 @@ __global__ void __launch_bounds__(kP64Threads) k_walk64(Problem P, PathArgs A, P
         if (!__ballot_sync(kAll, have)) break;
         double z0 = 0.0, z1 = 0.0;
         if (have) normals64(A.seed, (uint32_t)knot, kw, (uint32_t)(k + gl), (uint32_t)p, z0, z1);
-#pragma unroll
         for (int j = 0; j < kWalkLanes; ++j) {
-            const double xi0 = __shfl_sync(kAll, z0, lead + j), xi1 = __shfl_sync(kAll, z1, lead + j);
+            const double xi0 = from_lane(z0, lead + j), xi1 = from_lane(z1, lead + j);
+            double cv = 0.0, fv = 0.0;
+            if (KILL || SRC) {
+                if (!__ballot_sync(kAll, have)) break;
+                if (KILL) {
+                    const double sum = walk_sum(nr, rw, lead, gl, [&](int q) {
+                        const double dx = x - rx[q], dy = y - ry[q];
+                        return exp_neg(-(dx * dx + dy * dy) * inv2s, etab);
+                    });
+                    cv = sum < 0.0 ? sum : 0.0;
+                }
+                if (SRC)
+                    fv = walk_sum(nf, P.frbf_w, lead, gl, [&](int q) {
+                        const double dx = x - P.frbf_x[q], dy = y - P.frbf_y[q];
+                        return exp(-(dx * dx + dy * dy) * finv);
+                    });
+            }
             if (!have) continue;
             if (k >= max_steps) {
                 if (gl == 0) {
@@ -1265,6 +1329,8 @@ __global__ void __launch_bounds__(kP64Threads) k_walk64(Problem P, PathArgs A, P
                 have = false;
                 continue;
             }
+            if (SRC) Zv = Zv + fv * Yv * A.h;
+            if (KILL) Yv = Yv * (1.0 + cv * A.h);
             const double nx = x + sh * xi0, ny = y + sh * xi1;
             ++k;
             const double ddx = nx - cx, ddy = ny - cy;
@@ -2115,7 +2181,9 @@ static void run_paths64(const Problem &P, const PathArgs &A, int nrows, long tot
     PathPool Q{B.slots.p, nrows, (unsigned long long)total, nullptr, nullptr, nullptr, nullptr, nullptr, 0, nullptr,
                nullptr, B.seg.p};
     int grid = ctas;
-    const bool walk = P.b_kind == PDD_B_ZERO && P.c_kind == PDD_C_ZERO && P.f_kind == PDD_F_ZERO && A.cvd == 0;
+    const bool kill = P.c_kind == PDD_C_RBF, src = P.f_kind == PDD_F_RBF;
+    const bool walk = P.b_kind == PDD_B_ZERO && (P.c_kind == PDD_C_ZERO || kill) && (P.f_kind == PDD_F_ZERO || src) &&
+                      A.cvd == 0;
     for (int pass = 0; pass < kP64Passes; ++pass) {
         const bool last = pass == kP64Passes - 1;
         Q.next = B.next.p + pass;
@@ -2128,7 +2196,9 @@ static void run_paths64(const Problem &P, const PathArgs &A, int nrows, long tot
         Q.keep = last ? 0 : 16;
         if (walk && pass == 1) {
             const int most = cdiv(15L * ctas * (kP64Threads / 32), kP64Threads / kWalkLanes);     // its paths, at most
-            PDD_LAUNCH(k_walk64, std::min(most, 8 * sms), kP64Threads, 0, st, P, A, Q);
+            auto kern = kill ? (src ? k_walk64<true, true> : k_walk64<true, false>)
+                             : (src ? k_walk64<false, true> : k_walk64<false, false>);
+            PDD_LAUNCH(kern, std::min(most, 8 * sms), kP64Threads, sm, st, P, A, Q);
             break;
         }
         if (A.cvd > 0) launch_pass64<true>(P, A, Q, grid, sm, st);
