@@ -274,7 +274,8 @@ typedef struct {
                               /*   launches alone (CUDA events around each, a8)      */
     double ms_tc_gemm;        /* mixed form: device time of the tensor-core Schur    */
                               /*   update launches alone (a7)                        */
-    int64_t disk_solves;      /* (disk, sweep) triangular solves run (a8)            */
+    int64_t disk_solves;      /* (disk, sweep) triangular solves run (a8); without   */
+                              /*   drift and killing (group of columns, sweep)       */
     double tc_gemm_flop;      /* useful flops (2MNK per matrix) of those launches    */
     int lu_pivoted_fallback;  /* 1: a wave of the pivot-free LU was redone with partial
                                  pivoting (a tiny pivot or a refinement that missed its
