@@ -1070,6 +1070,7 @@ struct RlArgs {
 template <int CG, int NT = kRlThreads>
 static void launch_rl_cg(const RlArgs &a, cudaStream_t st) {
     const size_t sm = rl_smem_bytes(a.n, CG);
+    if (!a.LU || !a.Dinv) fail(PDD_ECUDA, "right-looking solve without its factors");
     auto kern = k_lu_solve_rl<CG, NT>;
     PDD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     PDD_LAUNCH(kern, NT == kRlThreads ? dim3(a.nd, a.groups) : dim3(a.nd * a.groups), NT, sm, st, a.LU, a.n, a.sA, a.perm, a.Dinv, a.R, a.nrhs, a.sR, a.X, a.conv,
@@ -2020,7 +2021,10 @@ static float shared_disks(const pdd_cover &cov, const Problem &P, const pdd_asse
     if (src) {
         RHS.alloc((size_t)nvmax * S.n * kShareCols);
         scl.alloc(chunk);
-        B.choose(Ss, nvmax);
+        // The right-looking solve needs the factors transposed and their blocks inverted, which the first
+        // disk's have only when its own columns took it: three columns of n > 7,036 rows do not (no group of
+        // eight fits), while a group of four of the 17 source columns would.
+        if (F.AT) B.choose(Ss, nvmax);
         B.alloc(Ss, nvmax);
     }
     if (Bx.rlW) Bx.Dhl.alloc((size_t)chunk * S.n * S.nrhs);
