@@ -34,6 +34,10 @@ struct Fail {
         }                                                                       \
     } while (0)
 
+// A kernel's limit of dynamic shared memory belongs to the kernel, not to a call or a thread: it is only
+// ever raised, so that no thread's call lowers it between another's setting and launch (api.cu).
+void allow_smem(const void *kernel, size_t bytes);
+
 // launch accounting: every kernel launch goes through this macro
 #define PDD_LAUNCH(kernel, grid, block, smem, stream, ...)                      \
     do {                                                                        \

@@ -306,7 +306,7 @@ static void build_operator(const Problem &P, const Shape &S, const DiskDesc *dd,
     const int rpb = (int)std::max<size_t>(1, std::min<size_t>(8, (size_t)(96 * 1024) / row_bytes));
     if (row_bytes > (size_t)200 * 1024) fail(PDD_EINVAL, "disk grid too large for the operator kernel");
     const size_t sm = rpb * row_bytes;
-    PDD_CUDA(cudaFuncSetAttribute(k_fill_operator<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    allow_smem((const void *)k_fill_operator<T>, sm);
     dim3 g(cdiv(S.n, rpb), nd);
     PDD_LAUNCH(k_fill_operator<T>, g, 32 * rpb, sm, st, S, A, sA, coef, sC, rpb);
 }
@@ -608,7 +608,7 @@ static void launch_solve(const T *LU, int n, long sA, const int *perm, const dou
     if (!conv) groups = std::max(1, std::min(cdiv(2L * sms, nd), nrhs / 4));
     const int ncg = cdiv(nrhs, groups);
     const size_t sm = solve_smem<T>(ncg);
-    PDD_CUDA(cudaFuncSetAttribute(k_lu_solve<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    allow_smem((const void *)k_lu_solve<T>, sm);
     PDD_LAUNCH(k_lu_solve<T>, dim3(nd, cdiv(nrhs, ncg)), 256, sm, st, LU, n, sA, perm, R, nrhs, ncg, sR, W, X, accumulate, conv, sweeps, tol);
 }
 
@@ -1072,7 +1072,7 @@ static void launch_rl_cg(const RlArgs &a, cudaStream_t st) {
     const size_t sm = rl_smem_bytes(a.n, CG);
     if (!a.LU || !a.Dinv) fail(PDD_ECUDA, "right-looking solve without its factors");
     auto kern = k_lu_solve_rl<CG, NT>;
-    PDD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    allow_smem((const void *)kern, sm);
     PDD_LAUNCH(kern, NT == kRlThreads ? dim3(a.nd, a.groups) : dim3(a.nd * a.groups), NT, sm, st, a.LU, a.n, a.sA, a.perm, a.Dinv, a.R, a.nrhs, a.sR, a.X, a.conv,
                a.dmb, a.xmb, a.D, a.dmode, a.groups);
 }
@@ -1708,8 +1708,7 @@ static void launch_lu(T *A, int n, long strideA, int *perm, int *info, int nd, c
     switch (nb) {
 #define PDD_LU_CASE(NBV)                                                                      \
     case NBV:                                                                                  \
-        PDD_CUDA(cudaFuncSetAttribute(k_lu<T, NBV>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                      (int)smem));                                            \
+        allow_smem((const void *)k_lu<T, NBV>, smem);                                          \
         PDD_LAUNCH((k_lu<T, NBV>), nd, 256, smem, st, A, n, strideA, perm, info);              \
         break;
         PDD_LU_CASE(32)
@@ -1840,8 +1839,8 @@ static void solve_wave(const Problem &P, const pdd_assembly_opts &o, const Shape
         const int nw = (S.nc - 1) + S.nt;
         const size_t rsm = (size_t)kResNP * nw * sizeof(double);
         const size_t rsm_df = ((size_t)kResNPdf * nw + 6 * kResNPdf) * sizeof(float2);
-        PDD_CUDA(cudaFuncSetAttribute(k_residual, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm));
-        PDD_CUDA(cudaFuncSetAttribute(k_residual_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm_df));
+        allow_smem((const void *)k_residual, rsm);
+        allow_smem((const void *)k_residual_df, rsm_df);
         dim3 g_res(cdiv(S.n, kResNP), nd), g_res_df(cdiv(S.n, kResNPdf), nd);
         // without drift, the forms over angle pairs (nd <= 65535 is the grid's limit for both)
         const int cg1 = P.b_kind == PDD_B_ZERO ? sym_columns<double>(S) : 0;
@@ -1927,7 +1926,7 @@ static void eval_wave(const pdd_cover &cov, pdd_system &sys, const Shape &S, con
         const long cnt = (long)nd * sR;
         if (split) PDD_LAUNCH(k_split_x, (int)std::min<long>(cdiv(cnt, 256), 4096), 256, 0, st, cnt, B.X.p, B.Dhl.p);
         const size_t esm = sizeof(float2) * kEvalKnots * std::max<size_t>(2 * kEvalChunk, kEvalThreads);
-        PDD_CUDA(cudaFuncSetAttribute(k_disk_eval_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)esm));
+        allow_smem((const void *)k_disk_eval_df, esm);
         PDD_LAUNCH(k_disk_eval_df, dim3(nd, cdiv(S.nrhs, kEvalThreads)), kEvalThreads, esm, st, S, dd,
                    cov.sub_rows.p, cov.sub_off.p, cov.kx.p, cov.ky.p, cov.rowptr.p, B.Dhl.p, sR, sys.val.p, sys.bs.p);
     } else {
@@ -1936,7 +1935,7 @@ static void eval_wave(const pdd_cover &cov, pdd_system &sys, const Shape &S, con
         const int per = (int)std::min<size_t>(256 / group, (180 * 1024) / rowb);
         if (per < 1) fail(PDD_EINVAL, "disk grid too large for the evaluation kernel");
         const size_t esm = per * rowb;
-        PDD_CUDA(cudaFuncSetAttribute(k_disk_eval, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)esm));
+        allow_smem((const void *)k_disk_eval, esm);
         PDD_LAUNCH(k_disk_eval, nd, 256, esm, st, S, dd, cov.sub_rows.p, cov.sub_off.p, cov.kx.p, cov.ky.p,
                    cov.rowptr.p, B.X.p, sR, group, per, sys.val.p, sys.bs.p);
     }
@@ -2503,7 +2502,7 @@ void grad_disks(const pdd_cover &cov, const Problem &P, const double *u, const d
                        lambda, Vb.p, Eb.p);
             PDD_LAUNCH(k_lu_solve_T, nd, 256, 0, st, A.p, S.n, sA, perm.p, coef.p, sC, Eb.p, Wt.p, Zb.p);
             const size_t csm = (size_t)4 * S.n * sizeof(double);
-            PDD_CUDA(cudaFuncSetAttribute(k_adjoint_contract, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm));
+            allow_smem((const void *)k_adjoint_contract, csm);
             PDD_LAUNCH(k_adjoint_contract, nd, 256, csm, st, P, S, dd.p, Vb.p, Zb.p,
                        partial.p + (size_t)(done + w0) * (nw + nf));
         }

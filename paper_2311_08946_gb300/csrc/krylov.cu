@@ -811,7 +811,7 @@ static SolveResult gmres_run(int n, const int *rowptr, const int *col, const dou
     }
     double *rr = &B.gs->rr;                                // device address: the residual's squared norm
     const size_t upper_smem = (size_t)kUpperCols * m * sizeof(double);
-    PDD_CUDA(cudaFuncSetAttribute(k_upper_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)upper_smem));
+    allow_smem((const void *)k_upper_solve, upper_smem);
     SolveResult res;
     for (int cycle = 0;; ++cycle) {
         // the residual: b on the first cycle (u = 0), what the previous cycle ended with after that

@@ -399,8 +399,7 @@ struct RecLU {
         switch (W) {
 #define PDD_LEAF(WV)                                                                                      \
     case WV:                                                                                              \
-        PDD_CUDA(cudaFuncSetAttribute(k_panel_leaf<WV>, cudaFuncAttributeMaxDynamicSharedMemorySize,      \
-                                      (int)std::max<size_t>(smem, 1)));                                   \
+        allow_smem((const void *)k_panel_leaf<WV>, smem);                                                 \
         PDD_LAUNCH(k_panel_leaf<WV>, nd, 256, smem, st, A, n, sA, k0, w, perm, info);                     \
         break;
             PDD_LEAF(32)

@@ -1836,7 +1836,7 @@ void build_imq_inverses(const pdd_cover &cov, double c2, DevBuf<double> &kinv, D
         PDD_CUDA(cudaMemcpyAsync(circ.p, per.data(), per.size() * sizeof(int), cudaMemcpyHostToDevice, st));
         PDD_CUDA(cudaMemcpyAsync(koff_c.p, offc.data(), per.size() * sizeof(long), cudaMemcpyHostToDevice, st));
         const size_t smem = (size_t)2 * cov.max_stencil * cov.max_stencil * sizeof(double);
-        PDD_CUDA(cudaFuncSetAttribute(k_imq_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        allow_smem((const void *)k_imq_inverse, smem);
         PDD_LAUNCH(k_imq_inverse, (int)per.size(), 128, smem, st, circ.p, cov.knot_ptr.p, cov.ku.p, koff_c.p, c2,
                    kinv.p, kcond.p, bad.p);
     }
@@ -2261,7 +2261,7 @@ McStats assemble_mc(const pdd_cover &cov, const Problem &P, const pdd_assembly_o
     if (ncv) cvq.alloc((size_t)wave * P_ * ncv);
     const size_t cv_smem = ((size_t)kCvThreads * ncv + 2 * kCvThreads + 2 * ncv * ncv + (size_t)cv_stride * ncv +
                             cv_stride + ncv + (size_t)kBatches * ncv + 32 * cv_stride) * sizeof(double);
-    if (ncv) PDD_CUDA(cudaFuncSetAttribute(k_cv_regress, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cv_smem));
+    if (ncv) allow_smem((const void *)k_cv_regress, cv_smem);
     DevBuf<unsigned long long> steps;
     DevBuf<int> capped;
     steps.alloc(1);
@@ -2275,9 +2275,9 @@ McStats assemble_mc(const pdd_cover &cov, const Problem &P, const pdd_assembly_o
     float tp = 0, tf = 0;
     const size_t fsm = (size_t)2 * kBatches * cov.max_stencil * sizeof(double);
     const int nq_launch = std::max(1, (cov.max_stencil + 31) / 32);
-    PDD_CUDA(cudaFuncSetAttribute(k_mc_finalize<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm));
-    PDD_CUDA(cudaFuncSetAttribute(k_mc_finalize<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm));
-    PDD_CUDA(cudaFuncSetAttribute(k_mc_finalize<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm));
+    allow_smem((const void *)k_mc_finalize<1>, fsm);
+    allow_smem((const void *)k_mc_finalize<2>, fsm);
+    allow_smem((const void *)k_mc_finalize<3>, fsm);
     // per-slot arrays (subs, spos, kword, momp, bmean) are indexed like the global slot gs: offset to
     // the wave's first slot when gsl is null, or the whole arrays with gsl
     Paths64Bufs p64;
@@ -2713,8 +2713,7 @@ void grad_mc(const pdd_cover &cov, const Problem &P, const pdd_assembly_opts &o,
     const bool src = P.f_kind != PDD_F_ZERO;
 #define PDD_GRAD_LAUNCH(R, SRCV)                                                                          \
     do {                                                                                                  \
-        PDD_CUDA(cudaFuncSetAttribute(k_paths_grad<R, SRCV>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                      (int)smem));                                                       \
+        allow_smem((const void *)k_paths_grad<R, SRCV>, smem);                                            \
         PDD_LAUNCH((k_paths_grad<R, SRCV>), nmc * splits, kGradThreads, smem, st, P, A, G);                                   \
     } while (0)
     if (path_mixed(o)) {

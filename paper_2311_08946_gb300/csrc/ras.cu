@@ -193,7 +193,7 @@ void RasPrecond::build(const pdd_cover &cov, const int *rowptr, const int *col, 
         PDD_LAUNCH(k_ras_locate_rows, cdiv(nrows, 256), 256, 0, st, nrows, cov.sub_rows.p, cov.sub_ptr.p,
                    cov.row_sub.p, l2.p);
     const size_t sm = (size_t)NP * (2 * NP + 1) * sizeof(float);
-    PDD_CUDA(cudaFuncSetAttribute(k_ras_invert, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    allow_smem((const void *)k_ras_invert, sm);
     PDD_LAUNCH(k_ras_invert, P, kRasThreads, sm, st, P, NP, wptr.p, widx.p, rowptr, col, val, cov.kowner.p,
                cov.row_sub.p, l1.p, l2.p, cinvT.p, sing.p);
     int hs = 0;
