@@ -366,7 +366,8 @@ typedef struct {
 
 typedef struct {
     int iters;
-    double rel_residual;      /* true residual after the last restart              */
+    double rel_residual;      /* true residual after the last restart; NaN where C   */
+                              /*   or b is not finite or a norm overflows            */
     int converged;
 } pdd_solve_info;
 

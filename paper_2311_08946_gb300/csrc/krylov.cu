@@ -833,10 +833,21 @@ static SolveResult gmres_run(int n, const int *rowptr, const int *col, const dou
         PDD_CUDA(cudaMemcpyAsync(&hg, B.gs, sizeof(GState), cudaMemcpyDeviceToHost, st));
         PDD_CUDA(cudaStreamSynchronize(st));
         if (hg.err) fail(PDD_ECUDA, "GMRES grid barrier timed out");
-        const double rel = hg.bnorm > 0.0 ? std::sqrt(hg.rr) / hg.bnorm : 0.0;
         res.iters = hg.iters;
-        res.rel = rel;
-        if (hg.bnorm == 0.0 || rel <= o.rtol) {
+        if (hg.bnorm == 0.0) {                           // u = 0
+            res.rel = 0.0;
+            res.converged = 1;
+            break;
+        }
+        // a NaN or an infinity in C or b, or a norm that overflows: no later cycle ends it
+        if (!std::isfinite(hg.bnorm) || !std::isfinite(hg.rr)) {
+            res.rel = std::nan("");
+            break;
+        }
+        // (the test of the next cycle's start, rounding for rounding: a cycle that it skips would come again)
+        const double beta = std::sqrt(hg.rr);
+        res.rel = beta / hg.bnorm;
+        if (beta <= o.rtol * hg.bnorm) {
             res.converged = 1;
             break;
         }
