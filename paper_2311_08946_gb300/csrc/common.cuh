@@ -308,6 +308,25 @@ __device__ __forceinline__ float2 df_split(double v) {
     return make_float2(h, (float)(v - (double)h));
 }
 
+// df_split, value by value, by integer operations (the FP64 pipe of this part is 1/64 of the FP32 rate):
+// v's bits above the 29 lowest rounded to nearest, ties to even, and the 29 lowest as a signed rest.
+// Below 2^-74, where lo's scale is no normal FP32 number, and beyond 2^127 it is df_split itself, but for
+// zeros (and FP64 denormals), which are common: a source column of zeros among others.
+// (out of line, or its FP64 instructions are issued for every value: 43.0 ms against 41.9 on the scaled workload)
+__device__ __noinline__ static float2 df_split_far(double v) { return df_split(v); }
+
+__device__ __forceinline__ float2 df_split_int(double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL;
+    const unsigned sign = (unsigned)__double2hiint(v) & 0x80000000u;
+    const int e = (int)(b >> 52);
+    if (e == 0) return make_float2(__uint_as_float(sign), 0.f);
+    if ((unsigned)(e - 949) > 200u) return df_split_far(v);
+    const unsigned hb = (unsigned)((b + 0x0fffffffULL + ((b >> 29) & 1)) >> 29), up = hb - (unsigned)(b >> 29);
+    const int rest = (int)((unsigned)b & 0x1fffffffu) - (int)(up << 29);
+    const float lo = __fmul_rn(__int2float_rn(rest), __uint_as_float((unsigned)(e - 948) << 23));
+    return make_float2(__uint_as_float((hb - (896u << 23)) | sign), __uint_as_float(__float_as_uint(lo) ^ sign));
+}
+
 // v = hi + lo with hi = v truncated to 24 significant bits and lo the rest rounded to FP32, built
 // from the bit fields by integer operations (the FP64 pipe of this part is 1/64 of the FP32 rate).
 // |v| < 2^-126 gives (0, 0) and |v| < 2^-74 drops lo (relative error up to 2^-23 there); above

@@ -1411,8 +1411,8 @@ __global__ void __launch_bounds__(kSymThreads, 1) k_residual_sym(Shape S, const 
                 const long o = (long)p * S.nrhs + c0 + c;
                 const T t = h ? Pol::sub(E, O) : Pol::add(E, O);
                 if constexpr (DF) {
-                    const float2 au = df_add(df_mul(al, t), df_mul(split_df_bits(cf.c), U[o]));
-                    const float2 v = df_mul(split_df_bits(cf.s), au);
+                    const float2 au = df_add(df_mul(al, t), df_mul(df_split_int(cf.c), U[o]));
+                    const float2 v = df_mul(df_split_int(cf.s), au);
                     Rall[disk * strideR + o] = (double)df_add(R1all[disk * strideR + o], make_float2(-v.x, -v.y)).x;
                 } else {
                     const double r = RHSall[disk * strideR + o] - cf.s * (al * t + cf.c * U[o]);
@@ -1571,14 +1571,17 @@ __global__ void __launch_bounds__(kEvalThreads, 3) k_disk_eval_df(Shape S, const
                 den += __shfl_xor_sync(0xffffffffu, den, o);
                 hit = max(hit, __shfl_xor_sync(0xffffffffu, hit, o));
             }
+            // v / den: the product with the reciprocal, corrected by its residual
             const double inv = 1.0 / den;
-            for (int l = lane; l <= S.nc; l += 32)
-                lr[warp][l] = (hit >= 0) ? (l == hit ? 1.0 : 0.0) : lr[warp][l] * inv;
+            for (int l = lane; l <= S.nc; l += 32) {
+                const double v = lr[warp][l], q = v * inv;
+                lr[warp][l] = (hit >= 0) ? (l == hit ? 1.0 : 0.0) : fma(fma(-q, den, v), inv, q);
+            }
             for (int a = lane; a < S.nt; a += 32) sa[warp][a] = fourier_cardinal_cf(phi - PDD_TWO_PI * a / S.nt, S.nt);
             __syncwarp();
             const double l0 = lr[warp][0], ln = lr[warp][S.nc];
             for (int a = lane; a < S.nt; a += 32)
-                eb[warp][a] = split_df_bits(l0 * sa[warp][a] + ln * sa[warp][a < half ? a + half : a - half]);
+                eb[warp][a] = df_split_int(l0 * sa[warp][a] + ln * sa[warp][a < half ? a + half : a - half]);
         }
         float2 acc[K];
 #pragma unroll
@@ -1592,7 +1595,7 @@ __global__ void __launch_bounds__(kEvalThreads, 3) k_disk_eval_df(Shape S, const
                 float2 w = make_float2(0.f, 0.f);
                 if (g < nkn) {
                     const double l1 = lr[g][kk + 1], l2 = lr[g][S.nc - 1 - kk], s1 = sa[g][a], s2 = sa[g][a + half];
-                    w = split_df_bits(od ? 0.5 * (l1 - l2) * (s1 - s2) : 0.5 * (l1 + l2) * (s1 + s2));
+                    w = df_split_int(od ? 0.5 * (l1 - l2) * (s1 - s2) : 0.5 * (l1 + l2) * (s1 + s2));
                 }
                 edf[e] = w;
             }
@@ -1991,7 +1994,7 @@ __global__ void __launch_bounds__(256) k_gather_x(Shape S, int nd, const double 
         double v = 0.0;
         if (c < S.nk) v = X0[q];
         else if (Xs) v = Xs[((long)(d / kShareCols) * S.n + p) * kShareCols + d % kShareCols] * scl[d];
-        if constexpr (std::is_same<V, float2>::value) out[e] = split_df_bits(v);
+        if constexpr (std::is_same<V, float2>::value) out[e] = df_split_int(v);
         else out[e] = v;
     }
 }
