@@ -817,7 +817,8 @@ void build_cover_impl(const pdd_domain &dom, const pdd_cover_spec &spec, pdd_cov
     cov.h_nr = to_host(cov.nr, M, st);
     cov.h_nt = to_host(cov.nt, M, st);
     cov.h_floating = to_host(cov.floating, M, st);
-    std::vector<double> hr = to_host(cov.r, M, st);
+    cov.h_r = to_host(cov.r, M, st);
+    const std::vector<double> &hr = cov.h_r;
     std::vector<double> hcx = to_host(cov.cx, M, st), hcy = to_host(cov.cy, M, st);
     cov.max_nk = 0;
     cov.M_floating = 0;

@@ -45,6 +45,7 @@ struct pdd_cover {
     pdd::DevBuf<int> cell_ptr, cell_items;
     // host copies of small per-circle data
     std::vector<int> h_knot_ptr, h_sub_ptr, h_nk, h_nr, h_nt;
+    std::vector<double> h_r;
     std::vector<uint8_t> h_floating;
 };
 

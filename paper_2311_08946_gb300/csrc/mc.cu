@@ -2103,12 +2103,12 @@ static void launch_paths(const Problem &P, const PathArgs &A, int nrows, int nc,
 }
 
 // nrows slots with `total` paths in all, their records contiguous in slot order
-static void run_paths32(const Problem &P, const PathArgs &A, int nrows, long total, double max_r, Paths32Bufs &B,
+static void run_paths32(const Problem &P, const PathArgs &A, int nrows, long total, bool long_paths, Paths32Bufs &B,
                         cudaStream_t st) {
     const int nc = P.c_kind == PDD_C_RBF && P.n_rbf <= kP32Staged ? P.n_rbf : 0;
     const int nf = P.f_kind == PDD_F_RBF && P.n_frbf <= kP32Staged ? P.n_frbf : 0;
     const size_t sm = (nc ? gauss_smem(nc) : 0) + (nf ? gauss_smem(nf) : 0);
-    if (max_r * max_r / (4.0 * A.h) < kLongSteps) {        // mean steps of a path of the largest circle
+    if (!long_paths) {
         if (A.cvd > 0) launch_paths<true>(P, A, nrows, nc, nf, sm, st);
         else launch_paths<false>(P, A, nrows, nc, nf, sm, st);
         return;
@@ -2282,6 +2282,12 @@ McStats assemble_mc(const pdd_cover &cov, const Problem &P, const pdd_assembly_o
     // the wave's first slot when gsl is null, or the whole arrays with gsl
     Paths64Bufs p64;
     Paths32Bufs p32;
+    // the steps of a path from a circle's centre (r^2 / 4h), on average over the slots
+    double mean_steps = 0.0;
+    for (int m = 0; m < cov.M; ++m)
+        if (!cov.h_floating[m] || mcf)
+            mean_steps += (cov.h_sub_ptr[m + 1] - cov.h_sub_ptr[m]) * (cov.h_r[m] * cov.h_r[m] / (4.0 * o.h)) / nmc;
+    const bool long_paths = mean_steps >= kLongSteps;
     auto run_wave = [&](const int *rows, int nr, long nrec, const int *np, const long *roff, const int *gsl,
                         const int *momp, double *bmean, size_t w0) {
         const int *subs = sys.mc_subs.p + w0, *spos = sys.mc_spos.p + w0, *kword = sys.mc_kword.p + w0;
@@ -2289,7 +2295,7 @@ McStats assemble_mc(const pdd_cover &cov, const Problem &P, const pdd_assembly_o
                    cov.theta_s.p, o.paths, o.h, o.seed, side.p, su.p, Y.p, Z.p, steps.p, capped.p, np, roff, ez.p,
                    o.boundary_shift ? kGmC0 * sqrt(o.h) : 0.0, gsl, o.max_steps, cvd, ncv, cvq.p};
         PDD_CUDA(cudaEventRecord(e0, st));
-        if (mixed) run_paths32(P, A, nr, nrec, cov.max_r, p32, st);
+        if (mixed) run_paths32(P, A, nr, nrec, long_paths, p32, st);
         else run_paths64(P, A, nr, nrec, p64, st);
         PDD_CUDA(cudaEventRecord(e1, st));
         FinalArgs F{rows, subs, spos, cov.sub_off.p, cov.knot_ptr.p, cov.rowptr.p, cov.floating.p,
