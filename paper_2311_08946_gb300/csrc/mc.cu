@@ -1020,7 +1020,9 @@ __device__ __forceinline__ long long order_key(double v) {
     return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
 }
 
-// the leading 24 bits of a double as FP32 (values below 2^-126 give an arbitrary value at most 4)
+// the leading 24 bits of a double as FP32, for |v| in [2^-126, 2^128); beside that range an arbitrary value,
+// infinity and NaN among them.  In the circle's pre-test a displacement below it can only send the step to the
+// FP64 comparison (its square may come out too large, never too small), one above it is tested for.
 __device__ __forceinline__ float trunc32(double v) {
     const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
     return __uint_as_float(((__funnelshift_l(lo, hi, 3) ^ 0x40000000u) & 0x7fffffffu) | (hi & 0x80000000u));
@@ -1094,7 +1096,7 @@ __global__ void __launch_bounds__(kP64Threads) k_paths64(Problem P, PathArgs A, 
                 cy = S->cy;
                 if (CV) crad = S->r;
                 r2 = S->r2;
-                r2f = trunc32(r2) * 0.9999f;
+                r2f = (float)r2 * 0.9999f;
                 rec = S->rbase + p;
                 knot = S->i;
                 max_steps = S->max_steps;
@@ -1288,7 +1290,7 @@ __global__ void __launch_bounds__(kP64Threads) k_walk64(Problem P, PathArgs A, P
                 cx = S->cx;
                 cy = S->cy;
                 r2 = S->r2;
-                r2f = trunc32(r2) * 0.9999f;
+                r2f = (float)r2 * 0.9999f;
                 rec = S->rbase + p;
                 knot = S->i;
                 max_steps = S->max_steps;
