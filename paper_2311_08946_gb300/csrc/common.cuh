@@ -346,6 +346,15 @@ __device__ __forceinline__ float2 split_df_bits(double v) {
     return make_float2(hi, __uint_as_float(__float_as_uint(lo) | sign));
 }
 
+// a / b rounded to nearest, rb = 1 / b: quotient and residual corrected twice by FMAs (P. Markstein, IBM
+// J. Res. Dev. 34, 1990), where the compiler's division takes a dozen instructions and a branch; for numerators above 2^-100, whose
+// residuals do not underflow
+__device__ __forceinline__ float quotient(float a, float b, float rb) {
+    float q = __fmul_rn(a, rb);
+    q = fmaf(fmaf(-q, b, a), rb, q);
+    return fmaf(fmaf(-q, b, a), rb, q);
+}
+
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     s = a + b;
     const float bb = s - a;

@@ -276,14 +276,6 @@ __device__ __forceinline__ void cv_accumulate(R (&cq)[kMaxCv], int D, R xr, R yr
     }
 }
 
-// a / b rounded to nearest, rb = 1 / b: quotient and residual corrected twice by FMAs (P. Markstein, IBM
-// J. Res. Dev. 34, 1990), where the compiler's division takes a dozen instructions and a branch
-__device__ __forceinline__ float quotient(float a, float b, float rb) {
-    float q = __fmul_rn(a, rb);
-    q = fmaf(fmaf(-q, b, a), rb, q);
-    return fmaf(fmaf(-q, b, a), rb, q);
-}
-
 // packed FP32 pairs, each lane of the pair rounded like the scalar operation
 __device__ __forceinline__ unsigned long long pack2(float a, float b) {
     unsigned long long r;
