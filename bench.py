@@ -240,7 +240,7 @@ def run_ours(args, rank, world):
             times.append(e0.elapsed_time(e1))
             stats.append(S.stats())
             solve.append(S.last_solve)
-            N = cov.N
+            N, nnz = cov.N, cov.nnz
             del cov, S, u
     launches = pdd.launch_count() - launches0            # this library's kernels in the K timed steps
     timed_solve_ms = statistics.mean(SOLVE_MS[-args.steps:])
@@ -291,7 +291,7 @@ def run_ours(args, rank, world):
            "clocks": clk.summary()}
 
     # rooflines: the dominant kernel (device time from CUDA events inside the library) and the disk path
-    out["roofline"] = roofline(stats, cfg, N, timed_solve_ms)
+    out["roofline"] = roofline(stats, cfg, N, nnz, timed_solve_ms, solve[-1]["iters"])
 
     if not args.no_fp64 and rank == 0:
         out["fp64_form"] = fp64_form(pdd, stream, flush)
@@ -321,6 +321,8 @@ def run_ours(args, rank, world):
 PATHS_THREAD_INST_PER_STEP = 149.3
 # FP32 FMA peak from the unit counts: 152 SMs x 128 FP32 lanes x 2 flop x the maximum SM clock
 FP32_LANES_PER_SM = 128
+# FP64 FMAs per clock and SM
+FP64_FMA_PER_CLOCK = 2
 # DRAM bytes (read + write) per useful flop of k_tc_gemm_pipe<1> from one ncu capture: the top-level
 # Schur update (M = N = K = 1536) of 16 disks of the scaled workload, 795.7 MB read + 138.1 MB written
 # for 1.1596e11 flop (profiles/k_tc_gemm_pipe_scaled_mixed.md).  Its operands and C grow with the
@@ -333,10 +335,13 @@ def tf32_peak(pk):
     return pk["bf16_tflops"] * (1.1 / 2.25)
 
 
-def roofline(stats, cfg, N, ms_solve):
+def roofline(stats, cfg, N, nnz, ms_solve, iters, restart=64):
     """Rooflines of the heaviest kernels, each from its own device time (CUDA events around its launches
-    inside the library, on the stream they run on); the dominant one is the line's roofline, the others
-    go under "others"; "disk_path" is the whole floating-disk stage (a6-a9) against the TF32 peak."""
+    inside the library, on the stream they run on; the solve's around the whole call); the dominant one is
+    the line's roofline, the others go under "others"; "disk_path" is the whole floating-disk stage (a6-a9)
+    against the TF32 peak.  For workloads without a source, all of whose triangular solves take n_knots + 1
+    columns (with one, shared factors are solved for 17 source columns at a time)."""
+    assert cfg["op"]["f"] == "zero"
     pk, src = peaks()
     sm_mhz = pk.get("sm_max_mhz", 2070.0)
     st = stats[-1]
@@ -386,7 +391,17 @@ def roofline(stats, cfg, N, ms_solve):
            "peak_source": (f"152 SMs x 4 schedulers x 32 lanes x {sm_mhz:.0f} MHz / "
                            f"{PATHS_THREAD_INST_PER_STEP:.0f} thread-instructions per step (ncu, this "
                            "kernel variant on a 6 x 6 lattice of the workload's circles)")}
-    ks = [gem, fz, tri, pth]
+    # a13: GMRES, FP64 pipe: an iteration's product with C and two passes of Gram-Schmidt (dots and updates)
+    # against its j vectors
+    cycles, rest = divmod(iters, restart)
+    vectors = cycles * restart * (restart + 1) // 2 + rest * (rest + 1) // 2
+    fp64_peak = 152 * FP64_FMA_PER_CLOCK * 2 * sm_mhz * 1e6 / 1e12
+    gmr = {"kernel": "k_arnoldi_fused (a13, with the solve's other launches)", "bound": "alu", "ms": ms_solve,
+           "unit": "TFLOP/s", "achieved": (2.0 * nnz * iters + 8.0 * N * vectors) / (ms_solve / 1e3) / 1e12,
+           "traffic": None, "peak": fp64_peak,
+           "peak_source": f"152 SMs x {FP64_FMA_PER_CLOCK} FP64 FMAs x 2 flop x {sm_mhz:.0f} MHz",
+           "note": "FP64 flop of the products and the orthogonalisation; the FP32 RAS step is not counted"}
+    ks = [gem, fz, tri, pth, gmr]
     for k in ks:
         k["frac"] = (k["achieved"] / k["peak"]) if (k.get("achieved") and k.get("peak")) else None
     ks.sort(key=lambda k: -(k["ms"] or 0.0))

@@ -16,6 +16,14 @@
  *     pointers are host memory.
  *   - `stream` is a cudaStream_t (NULL = legacy default stream).  Work is
  *     queued on it; calls that return counts or statuses synchronise it.
+ *   - Device memory of handles and workspaces comes from one stream-ordered
+ *     pool per device, made at its first allocation there.  What the calls
+ *     have given back stays in the pool for later ones: up to 16 GB while a
+ *     cover or system lives on the device, up to 1 GB from the destruction of
+ *     the last one to the end of the process.  A cudaMalloc of the same
+ *     process that runs short gets that memory (driver 580); other processes
+ *     do not.  Buffers above 8 GB come from cudaMalloc and go back when their
+ *     call or handle ends.  Do not reset the device between calls.
  *   - Every call returns a pdd_status; PDD_OK is 0.  pdd_last_error()
  *     returns a thread-local message for the last failure.
  *   - Sizes are counts of elements unless stated.
@@ -406,9 +414,9 @@ pdd_status pdd_solve_csr(int n, const int *rowptr_dev, const int *col_dev, const
  * The paper has no counterpart: this entry point exists for callers that
  * cannot allocate device memory while they run -- a process whose device
  * heap belongs to another allocator (a caching allocator that must not be
- * bypassed or fragmented), a latency-critical loop that cannot absorb the
- * device-wide synchronisation of cudaFree, or a service that must not fail
- * with out-of-memory in the middle of a request.
+ * bypassed or fragmented), a latency-critical loop that must not wait for an
+ * allocator, or a service that must not fail with out-of-memory in the
+ * middle of a request.
  *   Workspace: a fixed 64 MiB array in device memory, reserved by every GPU
  *   that loads the library and held until the process exits.  The Krylov
  *   basis, partial sums and Hessenberg state of one solve must fit in it:

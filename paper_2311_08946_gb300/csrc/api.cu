@@ -42,6 +42,8 @@ void count_launch(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 // ---------------------------------------------------------------------------
 // What a pool keeps of the memory that is not in use: the working set of a repeated assembly while the
 // device has covers or systems (the 864 disks of the variable-coefficient workload take 9 GB), little when it has none.
+// The driver gives it to a cudaMalloc of the process that runs short: with 5 GB free and 7 GB unused in the
+// pool, 9 GB by cudaMalloc succeed, the library's own and other callers' (driver 580.159).
 static constexpr unsigned long long kPoolKeep = 16ULL << 30, kPoolKeepIdle = 1ULL << 30;
 // Buffers that the pool could not keep anyway come from cudaMalloc: mapping and unmapping them in the
 // pool added 47 ms a call on the scaled workload (two buffers of 23 GB)

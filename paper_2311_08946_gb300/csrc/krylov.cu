@@ -939,9 +939,9 @@ void csr_transpose(int n, int64_t nnz, const int *rowptr, const int *col, const 
 //
 // Some callers cannot allocate device memory while they run: a host process
 // whose device heap is owned by another allocator (a caching allocator that
-// must not be bypassed or fragmented), a latency-critical loop that cannot
-// absorb the device-wide synchronisation cudaFree implies, or a service that
-// must not meet an out-of-memory failure half-way through a request.  For them
+// must not be bypassed or fragmented), a latency-critical loop that must not
+// wait for an allocator, or a service that must not meet an out-of-memory
+// failure half-way through a request.  For them
 // pdd_solve_csr_noalloc runs the same GMRES kernels on a fixed workspace that
 // lives in this file-scope device array, reserved when the library is loaded
 // and held by every GPU that loads it until the process exits.
